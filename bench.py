@@ -78,8 +78,8 @@ def parse():
     ap.add_argument("--chunk", type=int, default=0, help="elements per chunk (0 = library default)")
     ap.add_argument("--pipeline", type=int, default=0, help="persistent double-buffered operator kernel")
     ap.add_argument("--operator-kernel", type=int, default=0,
-                    help="FP32 CG operator kernel of 3D meshes: 0 auto, 1 one patch per thread, 2 paired patches")
-    ap.add_argument("--operator-threads", type=int, default=0, help="threads per block of the paired-patch kernel")
+                    help="FP32 CG operator kernel of 3D meshes: 0 auto, 1 gathered shared nodes, 2 staged records with a halo")
+    ap.add_argument("--operator-threads", type=int, default=0, help="threads per block of operator kernel 2")
     ap.add_argument("--engine", default="auto", choices=["auto", "graph", "persistent", "fused"])
     ap.add_argument("--workload", default="headline",
                     choices=["headline", "c1", "c2", "c3", "c4", "c5", "projection", "periodic", "eos"],
@@ -320,7 +320,7 @@ def kernel_roofline(P, m, stats, mode, fused, stream, workload, lumped=False):
     if fused:
         which, kname = P.PS_KERNEL_CG1_F32, "k_cg1_chunks<%d>" % stats.dim
     elif mode == P.PS_MODE_MIXED and stats.operator_kernel == 2:
-        which, kname = P.PS_KERNEL_CG_F32, "k_cg2_units<%s,128,5>" % ("true" if lumped else "false")
+        which, kname = P.PS_KERNEL_CG_F32, "k_cg2_stars<384,3>"
     elif mode == P.PS_MODE_MIXED:
         which, kname = P.PS_KERNEL_CG_F32, "k_cg2_chunks<%d,float>" % stats.dim
     else:

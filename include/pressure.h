@@ -84,20 +84,20 @@ typedef int64_t ps_ticket;
 typedef struct {
     int32_t chunk_elems;     /* target elements per chunk (0 = auto by size)       */
     int32_t chunk_nodes_max; /* cap on distinct nodes per chunk (0 = auto)          */
-    int32_t pipeline;        /* FP32 CG operator kernel: 0 = one block per chunk,  */
-                             /* 1 = persistent blocks with double-buffered staging */
+    int32_t pipeline;        /* accepted for compatibility; one block per chunk     */
+                             /* whatever its value                                  */
     int32_t update_blocks_per_sm; /* grid of the CG update kernel in blocks per SM */
                              /* (0 = auto)                                          */
-    int32_t operator_kernel; /* FP32 CG operator kernel of 3D meshes: 0 = auto     */
-                             /* (paired patches), 1 = one patch per thread,        */
-                             /* 2 = paired patches (packed FP32x2 arithmetic,      */
-                             /* fixed-point node sums)                              */
-    int32_t operator_threads; /* threads per block of the paired-patch kernel:     */
-                             /* 0 = auto (128), 128 or 256                          */
+    int32_t operator_kernel; /* FP32 CG operator kernel of 3D meshes: 0 = auto (2),*/
+                             /* 1 = shared nodes gathered one by one, last-block   */
+                             /* completion, 2 = star records staged by bulk        */
+                             /* copies, shared nodes from a chunk-major halo        */
+    int32_t operator_threads; /* threads per block of operator_kernel 2:           */
+                             /* 0 = auto (384), 128 or 256                          */
     int32_t split_lead;      /* chunks at the head of the (Morton) chunk order split */
                              /* in halves when the mesh has at least four times as */
                              /* many, so the first wave of blocks ends out of step:*/
-                             /* 0 = auto (3D meshes with the paired-patch kernel:  */
+                             /* 0 = auto (3D meshes with operator_kernel 2:        */
                              /* one per SM; ps_debug_prepare: none), -1 = none,    */
                              /* n > 0 = n                                           */
     int32_t reserved[1];
@@ -170,8 +170,7 @@ typedef struct {
     int32_t max_chunk_elems, max_chunk_nodes;
     int64_t solve_bytes;     /* device bytes of this mesh's solver state while a solve
                                 is in flight (the serving loop's admission unit)    */
-    int64_t operator_kernel; /* FP32 CG operator kernel in use: 1 one patch per
-                                thread, 2 paired patches (ps_mesh_opts)             */
+    int64_t operator_kernel; /* FP32 CG operator kernel in use (ps_mesh_opts)       */
     int64_t reserved[2];
 } ps_mesh_stats;
 
@@ -212,10 +211,10 @@ int64_t ps_ctx_bytes_in_use(const ps_ctx *ctx);
  *   opts        preprocessing options or NULL
  * Host work: element partition into chunks along a Morton curve, node
  * renumbering (chunk-interior nodes contiguous per chunk, nodes shared between
- * chunks after them), per-chunk local connectivity and incidence lists, and
- * the FP64 stiffness weights of every element for the FP64 passes (about
- * 75 B per tetrahedron, 40 B per triangle of device memory, padding
- * included; ps_mesh_stats.device_bytes gives the total).
+ * chunks after them), per-chunk star patches and incidence lists, and the FP64
+ * stiffness weights of every element, from which the passes' star weights are
+ * formed whenever coefficients change (about 120 B per tetrahedron, 75 B per
+ * triangle of device memory; ps_mesh_stats.device_bytes gives the total).
  * Errors: PS_EINVAL for dim not 2/3, n_elems < 1, a vertex id out of range, a
  * non-finite coordinate or an element of zero volume; PS_ENOMEM. */
 int ps_mesh_upload(ps_ctx *ctx, int dim, int64_t n_nodes, const double *coords,
@@ -546,15 +545,15 @@ int ps_debug_cg_apply(ps_mesh *mesh, const void *x_dev, void *y_dev, double *pap
  *   PS_KERNEL_CG_F32     FP32 CG operator kernel: chunk staging, p = D^-1 r + beta p,
  *                        q = A p, chunk shares of p.Ap (the solver's dominant kernel)
  *   PS_KERNEL_UPDATE_F32 FP32 CG update kernel: shared-node rows, x and r update, rz, rr
- *                        (with the paired-patch kernel its blocks only store their
- *                        rz, rr shares: the halo gather sums them)
+ *                        (with operator_kernel 2 its blocks only store their rz, rr
+ *                        shares: the halo gather sums them)
  *   PS_KERNEL_APPLY_F32  FP32 operator apply alone (chunk kernel + shared-node sums)
  *   PS_KERNEL_RESID_F64  FP64 true-residual chunk kernel
  *   PS_KERNEL_CG_F64     FP64 CG operator kernel
  *   PS_KERNEL_CG1_F32    FP32 fused one-reduction CG pass (node updates of x, r, s, p,
  *                        u = D^-1 r, w = A u, gamma, delta, rho): the whole inner
  *                        iteration of the default mixed-precision solve
- *   PS_KERNEL_HALO_F32   the paired-patch kernel's halo gather ((D^-1 r, p) of every
+ *   PS_KERNEL_HALO_F32   the halo gather of operator_kernel 2 ((D^-1 r, p) of every
  *                        shared node into its chunks' slots) with, in its first block,
  *                        the sum of the update kernel's rz, rr shares and the end of
  *                        the iteration: the third kernel of that iteration (nothing

@@ -1,14 +1,13 @@
 """Autotuner for the solver's free parameters: for single solves the chunk
-size, the FP32 CG operator kernel (one patch per thread, its pipelined
-persistent form, or paired patches with 128 or 256 threads per block), the
-engine and the inner tolerance of the mixed solver; for meshes solved in
+size, the FP32 CG operator kernel (shared nodes gathered one by one, or
+staged records with a halo and 128 or 256 threads per block), the engine and the inner tolerance of the mixed solver; for meshes solved in
 batches the chunk size, the persistent kernel's threads per block and its
 task order (batch packing).
 
 It measures through the C ABI only: each candidate mesh layout is uploaded,
 the FP32 CG kernels are timed with ps_profile_kernel (CUDA events on the
 caller's stream): the operator and update kernels of the two-kernel
-iteration (plus the halo gather of the paired-patch kernel) and the fused
+iteration (plus the halo gather) and the fused
 one-reduction pass; the cheaper iteration picks the engine.  On the best
 layout whole solves are timed with ps_pressure_solve to pick the inner
 tolerance.  Batches are timed as whole ps_batch_solve calls on a sample.
@@ -24,8 +23,8 @@ import numpy as np
 CHUNKS = (768, 1536, 3072)
 PIPELINES = (0, 1)
 INNER_TOLS = (1e-3, 1e-4, 1e-5)
-# FP32 CG operator kernels: (operator_kernel, operator_threads); the paired
-# kernel exists for 3D meshes only
+# FP32 CG operator kernels: (operator_kernel, operator_threads); kernel 2
+# exists for 3D meshes only
 KERNELS = ((1, 0), (2, 128), (2, 256))
 
 

@@ -103,7 +103,7 @@ __device__ void batch_mesh_scalars(const BMesh &M, double *red, int *active_cnt)
 // inner phase, one grid barrier per pass.  At the start of a pass every block
 // reads each mesh's (run, parity, alpha, beta) into its shared-memory cache,
 // so a task costs no scalar round trip.
-__global__ void __launch_bounds__(256) k_batch_pcg(PcgArgs A) {
+__global__ void __launch_bounds__(256, 3) k_batch_pcg(PcgArgs A) {
     extern __shared__ __align__(128) unsigned char smem[];
     const ChunkSmem<float> S = chunk_smem<float>(smem, A.L);
     float2 *c_ab = reinterpret_cast<float2 *>(smem + A.L.total);          // [n_meshes]
@@ -200,9 +200,9 @@ __global__ void __launch_bounds__(256) k_batch_pcg(PcgArgs A) {
             }
             DotF acc[3];
             if (s_md.dim == 3)
-                chunk_cg1f<3>(s_md, cg1_pass(s_v, par), s_v.dinv, tk.y, ab.x, ab.y, S, phase, acc, failed);
+                chunk_cg1f<3, false>(s_md, cg1_pass(s_v, par), s_v.dinv, tk.y, ab.x, ab.y, S, phase, acc, failed);
             else
-                chunk_cg1f<2>(s_md, cg1_pass(s_v, par), s_v.dinv, tk.y, ab.x, ab.y, S, phase, acc, failed);
+                chunk_cg1f<2, false>(s_md, cg1_pass(s_v, par), s_v.dinv, tk.y, ab.x, ab.y, S, phase, acc, failed);
             if (failed) return;
             double out[3];
             block_sum_n<3>(acc, S.red, out);
@@ -239,17 +239,13 @@ __global__ void __launch_bounds__(256) k_b_resid1(const BMesh *meshes, const int
     a.x = M.x64;
     a.y = M.r64;
     a.b = M.b64;
-    a.p = nullptr;
-    a.r = nullptr;
-    a.dinv = nullptr;
     a.partial = M.part64;
     a.dotbuf = nullptr;
     a.st = nullptr;
-    a.host_done = nullptr;
     uint32_t phase = 0;
     bool failed = false;
-    DotD acc = (M.d.dim == 3) ? process_chunk<3, double, kResid>(M.d, a, tk.y, smem, L, phase, 0.0, failed)
-                              : process_chunk<2, double, kResid>(M.d, a, tk.y, smem, L, phase, 0.0, failed);
+    DotD acc = (M.d.dim == 3) ? process_chunk<3, double, kResid>(M.d, a, tk.y, smem, L, phase, failed)
+                              : process_chunk<2, double, kResid>(M.d, a, tk.y, smem, L, phase, failed);
     const double v = block_sum(acc, S.red);
     if (threadIdx.x == 0) M.dots64[tk.y] = v;
 }
@@ -513,15 +509,13 @@ void batch_plan_free(BatchPlan &plan) {
 
 // Combined shared-memory layout: every mesh's segments fit.
 static SmemLayout max_layout(const std::vector<ps_mesh *> &meshes, bool fp64) {
-    int max_loc = 0, max_patch = 0, max_inc = 0, max_sh = 0;
+    int max_loc = 0, max_patch = 0, max_inc = 0;
     for (ps_mesh *m : meshes) {
         max_loc = std::max(max_loc, m->prep.max_loc);
         max_patch = std::max(max_patch, m->prep.max_patch);
         max_inc = std::max(max_inc, m->prep.max_inc);
-        max_sh = std::max(max_sh, m->prep.max_sh);
     }
-    return fp64 ? make_layout(8, sizeof(NodeD), max_loc, max_patch, max_inc, max_sh)
-                : make_layout(4, sizeof(NodeF), max_loc, max_patch, max_inc, max_sh);
+    return make_layout(fp64 ? 8 : 4, max_loc, max_patch, max_inc);
 }
 
 int batch_plan_build(ps_ctx *ctx, ps_mesh *const *meshes, int n, int epoch_iters, const ps_solve_opts &o,

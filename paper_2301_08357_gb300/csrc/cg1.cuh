@@ -85,13 +85,18 @@ __device__ __forceinline__ float2 df_pack(double v) {
 
 // The fused pass over chunk c (block-uniform).  B: the buffers of this pass.
 // acc: this thread's shares of gamma, delta, rho.
-template <int D>
+// PRE: the thread's first star is loaded before the node updates (costs
+// registers, which the persistent batch kernel needs for resident blocks).
+template <int D, bool PRE>
 __device__ __forceinline__ void chunk_cg1f(const MeshDev &m, const CG1Pass &B, const float *__restrict__ dinv, int c,
                                            float alpha, float beta, const ChunkSmem<float> &S, uint32_t &phase,
                                            DotF acc[3], bool &failed) {
     const ChunkDesc cd = m.chunks[c];
     const int n_loc = cd.n_loc, n_int = cd.n_int;
     stage_issue<float>(m, cd, S);
+    const float *mrow = chunk_mrow<float>(m, cd);
+    StarF<D> pre;
+    if (PRE) star_prefetch<D>(m, cd, pre);
     // The node updates need none of the staged data, so they run while the
     // bulk copies are in flight (S.val and S.aux are not staged regions).
     // No Dirichlet mask is needed: D^-1 = 0 there and r starts at 0, so u,
@@ -128,11 +133,12 @@ __device__ __forceinline__ void chunk_cg1f(const MeshDev &m, const CG1Pass &B, c
         failed = true;
         return;
     }
-    patches_eval<D, float, false>(m, cd, S);
+    stars_eval<D, PRE>(m, cd, S, pre);
     for (int l = threadIdx.x; l < n_loc; l += blockDim.x) {
-        float wv = node_sum(S, l);
         const float u = S.val[l], r = S.aux[l];
-        if (is_dirichlet(S.node[l].w)) wv = 0.f;
+        const float mr = mrow[l];
+        float wv = fmaf(fabsf(mr), u, node_sum(S, l));
+        if (is_dirichlet(mr)) wv = 0.f;
         acc[1].add_prod(u, wv);                   // element-wise u^T A_e u
         if (l < n_int) {
             B.w_o[cd.int_begin + l] = wv;
@@ -239,7 +245,7 @@ __global__ void __launch_bounds__(256) k_cg1_chunks(MeshDev m, CG1Vec V, CgState
     uint32_t phase = 0;
     bool failed = false;
     DotF acc[3];
-    chunk_cg1f<D>(m, cg1_pass(V, s_par), V.dinv, blockIdx.x, s_ab[0], s_ab[1], S, phase, acc, failed);
+    chunk_cg1f<D, true>(m, cg1_pass(V, s_par), V.dinv, blockIdx.x, s_ab[0], s_ab[1], S, phase, acc, failed);
     if (failed) return;
     double out[3];
     block_sum_n<3>(acc, S.red, out);

@@ -79,18 +79,16 @@ struct Cg2Args {
     PT *z2;            // [2][g3]: block shares of rz and rr
     int g3;            // grid of K2 (and of the start kernel)
     CgState *st;
-    // paired-patch operator kernel only (else null): per chunk-major shared
+    // k_cg2_stars only (else null): per chunk-major shared
     // slot, (D^-1 r, p) of the slot's node, gathered after K2 for the next K1
     float2 *halo;
 };
 
-// K1: one block per chunk.  PRE: fetch the element phase's beta*dt^2 and the
-// first shared nodes' partial-sum destinations into registers before the
-// staging wait (FP32; costs registers, so it is used where shared memory, not
-// registers, limits the blocks per SM).
-template <int D, typename T, bool PRE = false>
+// K1: one block per chunk.
+template <int D, typename T>
 __global__ void __launch_bounds__(256) k_cg2_chunks(MeshDev m, Cg2Args<T> a) {
     extern __shared__ __align__(128) unsigned char smem[];
+    constexpr bool kPre = sizeof(T) == 4;
     const SmemLayout &L = (sizeof(T) == 4) ? m.sm32 : m.sm64;
     const ChunkSmem<T> S = chunk_smem<T>(smem, L);
     __shared__ double s_beta;
@@ -108,28 +106,18 @@ __global__ void __launch_bounds__(256) k_cg2_chunks(MeshDev m, Cg2Args<T> a) {
     stage_issue<T>(m, cd, S);
     const T beta = (T)s_beta;
     const int n_loc = cd.n_loc, n_int = cd.n_int;
-    // Every gather runs while the bulk copies are in flight: shared-node ids
-    // come from sh_info in global memory (not from the staged copy) and S.val
-    // is not a staged region.  No Dirichlet mask is needed: D^-1 = 0 and
-    // r = 0 on Dirichlet nodes and p starts at 0, so p stays 0 there.  Loads
-    // of four nodes are issued before any store (the stores to p could alias
-    // them).
-    // The element phase's beta*dt^2 values and the partial-sum destinations
-    // of the thread's first shared nodes are fetched here as well.
-    BdPrefetch<T> bdp;
-    if constexpr (PRE) prefetch_bd<T>(m, cd, bdp);
-    int dst[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int l = threadIdx.x + k * blockDim.x;
-        dst[k] = (PRE && l >= n_int && l < n_loc) ? m.sh_dest[cd.sh_off + (l - n_int)] : -1;
-    }
+    const T *mrow = chunk_mrow<T>(m, cd);
+    StarF<D> pre;
+    if (kPre) star_prefetch<D>(m, cd, pre);
+    // No Dirichlet mask is needed: D^-1 = 0 and r = 0 on Dirichlet nodes and
+    // p starts at 0, so p stays 0 there.  Loads of four nodes are issued
+    // before any store (the stores to p could alias them).
     for (int l0 = threadIdx.x; l0 < n_loc; l0 += 4 * blockDim.x) {
         int gg[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int l = l0 + k * blockDim.x;
-            gg[k] = l < n_int ? cd.int_begin + l : (l < n_loc ? m.sh_info[cd.sh_off + (l - n_int)].x : -1);
+            gg[k] = l < n_int ? cd.int_begin + l : (l < n_loc ? m.sh_ids[cd.sh_off + (l - n_int)] : -1);
         }
         T dv[4], rv[4], pv[4];
 #pragma unroll
@@ -153,31 +141,17 @@ __global__ void __launch_bounds__(256) k_cg2_chunks(MeshDev m, Cg2Args<T> a) {
     }
     uint32_t ph = 0;
     if (!stage_wait<T>(m, S, ph)) return;   // also the barrier for S.val
-    if constexpr (PRE)
-        patches_eval_pre<D, T>(m, cd, S, bdp);
-    else
-        patches_eval<D, T, false>(m, cd, S);
+    stars_eval<D, kPre>(m, cd, S, pre);
     typename DotOf<T>::type acc;
-    auto emit = [&](int l, int d) {
-        T s = node_sum(S, l);
-        acc.add_prod(S.val[l], s);                 // element-wise p^T A_e p over the chunk
-        if (is_dirichlet(S.node[l].w)) s = T(0);
+    for (int l = threadIdx.x; l < n_loc; l += blockDim.x) {
+        const T mr = mrow[l], v = S.val[l];
+        T s = fma(fabs(mr), v, node_sum(S, l));
+        acc.add_prod(v, s);                 // element-wise p^T A_e p over the chunk
+        if (is_dirichlet(mr)) s = T(0);
         if (l < n_int)
             a.q[cd.int_begin + l] = s;
         else
-            a.partial[d] = s;
-    };
-    if constexpr (PRE) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int l = threadIdx.x + k * blockDim.x;
-            if (l < n_loc) emit(l, dst[k]);
-        }
-        for (int l = threadIdx.x + 4 * blockDim.x; l < n_loc; l += blockDim.x)
-            emit(l, l < n_int ? -1 : m.sh_dest[cd.sh_off + (l - n_int)]);
-    } else {
-        for (int l = threadIdx.x; l < n_loc; l += blockDim.x)
-            emit(l, l < n_int ? -1 : m.sh_dest[cd.sh_off + (l - n_int)]);
+            a.partial[m.sh_dest[cd.sh_off + (l - n_int)]] = s;
     }
     const double v = block_sum(acc, S.red);
     if (threadIdx.x == 0) {
@@ -210,122 +184,6 @@ __device__ __forceinline__ DotF warp_merge(DotF a) {
         a.merge(h2, l2);
     }
     return a;
-}
-
-// K1, pipelined: a persistent CTA walks chunks blockIdx.x, +gridDim.x, ...
-// with two shared-memory stages for the static chunk data: while chunk i is
-// computed from one stage, the bulk copies of chunk i+1 fill the other.  The
-// per-chunk p.Ap shares are reduced per warp and combined by thread 0 after
-// the next block barrier (no extra barriers); they are indexed by chunk, so
-// the result does not depend on the grid.  FP32 only.
-template <int D>
-__global__ void __launch_bounds__(256) k_cg2_chunks_pipe(MeshDev m, Cg2Args<float> a, SmemLayout L0, SmemLayout L1) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    const ChunkSmem<float> S0 = chunk_smem<float>(smem, L0);
-    const ChunkSmem<float> S1 = chunk_smem<float>(smem, L1);
-    __shared__ float2 s_wred[8];
-    __shared__ float s_beta;
-    __shared__ int s_done;
-    __shared__ bool s_last;
-    if (threadIdx.x == 0) {
-        s_done = a.st->done;
-        s_beta = (float)a.st->beta;
-        mbar_init(S0.bar, 1);
-        mbar_init(S1.bar, 1);
-        fence_mbar_init();
-    }
-    __syncthreads();
-    if (s_done) return;
-    const float beta = s_beta;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    uint32_t ph0 = 0, ph1 = 0;
-    int c = blockIdx.x;
-    if (c < m.n_chunks) stage_issue<float>(m, m.chunks[c], S0);
-    int prev_c = -1;
-    for (int it = 0; c < m.n_chunks; ++it, c += gridDim.x) {
-        const ChunkSmem<float> &S = (it & 1) ? S1 : S0;
-        const ChunkDesc cd = m.chunks[c];
-        const int cn = c + gridDim.x;
-        if (cn < m.n_chunks) stage_issue<float>(m, m.chunks[cn], (it & 1) ? S0 : S1);
-        const int n_loc = cd.n_loc, n_int = cd.n_int;
-        float vin[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int l = threadIdx.x + k * blockDim.x;
-            vin[k] = 0.f;
-            if (l < n_int) {
-                const int g = cd.int_begin + l;
-                vin[k] = cg_dir(a.dinv[g], a.r[g], beta, a.p[g]);
-            }
-        }
-        // finish the previous chunk's share (its warp sums are in s_wred)
-        if (threadIdx.x == 0 && prev_c >= 0) {
-            DotF t;
-            for (int w = 0; w < nw; ++w) t.merge(s_wred[w].x, s_wred[w].y);
-            a.pq[prev_c] = part_pack((double)t.hi + (double)t.lo);
-        }
-        const bool ok = stage_wait<float>(m, S, (it & 1) ? ph1 : ph0);
-        if (!ok) {
-            // let the prefetch into the other stage land before leaving
-            if (cn < m.n_chunks) stage_wait<float>(m, (it & 1) ? S0 : S1, (it & 1) ? ph0 : ph1);
-            return;
-        }
-        auto finish = [&](int l, float v) {
-            if (is_dirichlet(S.node[l].w)) v = 0.f;
-            if (l < n_int) a.p[cd.int_begin + l] = v;
-            S.val[l] = v;
-        };
-        auto fetch = [&](int l) -> float {
-            const int g = l < n_int ? cd.int_begin + l : S.shid[l - n_int];
-            return cg_dir(a.dinv[g], a.r[g], beta, a.p[g]);
-        };
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int l = threadIdx.x + k * blockDim.x;
-            if (l < n_loc) finish(l, l < n_int ? vin[k] : fetch(l));
-        }
-        for (int l = threadIdx.x + 4 * blockDim.x; l < n_loc; l += blockDim.x) finish(l, fetch(l));
-        __syncthreads();
-        patches_eval<D, float, false>(m, cd, S);
-        DotF acc;
-        for (int l = threadIdx.x; l < n_loc; l += blockDim.x) {
-            float sv = node_sum(S, l);
-            acc.add_prod(S.val[l], sv);
-            if (is_dirichlet(S.node[l].w)) sv = 0.f;
-            if (l < n_int)
-                a.q[cd.int_begin + l] = sv;
-            else
-                a.partial[m.sh_dest[cd.sh_off + (l - n_int)]] = sv;
-        }
-        acc = warp_merge(acc);
-        if (lane == 0) s_wred[wid] = make_float2(acc.hi, acc.lo);
-        prev_c = c;
-        __syncthreads();   // stage, val, contrib and s_wred released / published
-    }
-    if (threadIdx.x == 0 && prev_c >= 0) {
-        DotF t;
-        for (int w = 0; w < nw; ++w) t.merge(s_wred[w].x, s_wred[w].y);
-        a.pq[prev_c] = part_pack((double)t.hi + (double)t.lo);
-        const unsigned int t2 = atomic_add_acq_rel(&a.st->cnt_a, 1u);
-        s_last = (t2 == gridDim.x - 1);
-    } else if (threadIdx.x == 0) {
-        const unsigned int t2 = atomic_add_acq_rel(&a.st->cnt_a, 1u);
-        s_last = (t2 == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    const double pq = part_sum(a.pq, m.n_chunks, S0.red);
-    if (threadIdx.x == 0) {
-        CgState *st = a.st;
-        st->cnt_a = 0;
-        st->pq = pq;
-        if (!(pq > 0.0) || !isfinite(pq)) {
-            st->status = kCgBreakdown;
-            st->done = 1;
-        } else {
-            st->alpha = st->rz / pq;
-        }
-    }
 }
 
 // K2: fixed grid over the padded node range [0, n_pad).  Interior nodes in
@@ -487,7 +345,7 @@ __device__ __forceinline__ void cg2_update_tail(CgState *st, double rz, double r
     if (done) st->done = 1;
 }
 
-// K2.  With the paired-patch operator kernel (a.halo set) the blocks only
+// K2.  With k_cg2_stars (a.halo set) the blocks only
 // store their shares of rz and rr: the halo gather that follows in the same
 // iteration sums them in its first block (k_halo_gather), concurrently with
 // its gather, so no block of K2 waits for the others.

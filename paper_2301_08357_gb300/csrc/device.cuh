@@ -16,15 +16,8 @@ constexpr uint32_t kGridSpinLimit = 1u << 26;
 
 enum DevErr : int { kErrNone = 0, kErrMbarTimeout = 1, kErrGridTimeout = 2, kErrBadSize = 4 };
 
-// Node record staged per chunk: coordinates relative to the chunk origin in
-// x, y, z (z = 0 in 2D) and alpha in w, with the sign bit of w set on
-// Dirichlet nodes (alpha itself is >= 0).
-struct alignas(16) NodeF { float x, y, z, w; };
-struct alignas(32) NodeD { double x, y, z, w; };
-template <typename T> struct NodeOf;
-template <> struct NodeOf<float> { using type = NodeF; };
-template <> struct NodeOf<double> { using type = NodeD; };
-
+// Per local node, the star passes read the row sum m_l of the chunk's patches
+// (layout.h), its sign bit set on Dirichlet nodes (m_l itself is >= 0).
 __device__ __forceinline__ bool is_dirichlet(float w) { return __float_as_int(w) < 0; }
 __device__ __forceinline__ bool is_dirichlet(double w) { return __double_as_longlong(w) < 0; }
 
@@ -52,6 +45,18 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
             smem_u32(dst)),
         "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+}
+// The same for data read once per pass of a working set larger than L2: the
+// lines are the first to be replaced, so that they do not push out what the
+// next kernels read again.
+__device__ __forceinline__ void bulk_g2s_stream(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+            smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
         : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
@@ -235,349 +240,258 @@ __device__ __forceinline__ void block_sum2(const DotF &a, const DotF &b, double 
     rb = o[1];
 }
 
-// ---------------------------------------------------------------- P1 element kernels
-// Notation: vertices p0..pd with coordinates (x,y[,z]) and nodal alpha in w;
-// nodal values v0..vd; bdt2 = beta_e * dt^2.  Jacobian columns e_k = p_k - p0,
-// cofactor vectors c_k with grad(lambda_k) = c_k / det (k = 1..d) and
-// c_0 = -(c_1 + ... + c_d); |T| = |det| / d!.
-//   stiffness:  (K v)_i = beta |T| grad(lambda_i) . grad(v_h)
-//                       = bdt2 / (d! |det|) * c_i . g,   g = sum_k (v_k - v_0) c_k
-//   mass:       (M_alpha v)_i = sum_jk alpha_k v_j int lambda_i lambda_j lambda_k
-//                 = cm (S X + Q + S v_i + alpha_i (X + 2 v_i)),
-//               S = sum alpha_k, X = sum v_k, Q = sum alpha_k v_k,
-//               cm = |T| d! / (d+3)!  (= |det|/720 in 3D, |det|/120 in 2D),
-//   from int lambda^a = d! |T| prod(a_i!) / (d + sum a_i)!.
-
-// One thread evaluates a whole patch (layout.h): element j is (a, b, r_j,
-// r_{j+1}) in 3D and (a, r_j, r_{j+1}) in 2D.  With e1 = b - a and
-// d_j = r_j - a, the cofactor vectors of element j are
-//   c1 = d_j x d_{j+1},  c2 = -(e1 x d_{j+1}),  c3 = e1 x d_j   (3D)
-//   c1 = perp(d_{j+1}),  c2 = -perp(d_j), perp(v) = (v.y, -v.x)  (2D)
-// so e1 x d_j and the node data of r_j carry over from element j-1 to j.
-// Per element: the stiffness and mass formulas above; the diagonal (DIAG)
-// takes v = e_i: kc |c_i|^2 and cm (2 S + 4 alpha_i).
-// out[slot]: 0 -> a, 1 -> b, 2 + j -> r_j (j = 0..m); other slots untouched.
-__device__ __forceinline__ float fdiv_fast(float a, float b) { return __fdividef(a, b); }
-__device__ __forceinline__ double fdiv_fast(double a, double b) { return a / b; }
-
-// beta*dt^2 of a patch's elements: vector loads, all up front.
+// ---------------------------------------------------------------- P1 star patches
+// One thread evaluates a whole star patch (layout.h) from its weights:
+//   out_i = sum over the patch's edges (i, j) of A^s_ij (v_j - v_i).
+// The row-sum term m_i v_i is added once per local node (mrow).  Per edge
+// one difference and two multiply-adds: 57 operations for the 19 edges of a
+// closed star of six tetrahedra, against ~55 for each of its tetrahedra when
+// the element matrices are applied one by one.
+// out[slot]: 0 -> a, 1 -> b (3D), 2 + j -> r_j, j < nr; other slots untouched.
+struct StarIds {
+    uint32_t w[kStarIds];
+    __device__ __forceinline__ int nr() const { return (int)((w[4] >> 16) & 7u); }
+    __device__ __forceinline__ bool closed() const { return (w[4] >> 20) & 1u; }
+    // byte offsets of an FP32 value per node
+    __device__ __forceinline__ uint32_t a() const { return w[0] & 0xffffu; }
+    __device__ __forceinline__ uint32_t b() const { return w[0] >> 16; }
+    __device__ __forceinline__ uint32_t ring(int j) const {
+        return j & 1 ? w[1 + j / 2] >> 16 : w[1 + j / 2] & 0xffffu;
+    }
+};
+// A node's value from its byte offset of an FP32 value.
 template <typename T>
-__device__ __forceinline__ void load_bd(const T *__restrict__ bdt2, T (&bd)[kPatchMax]) {
-    if (sizeof(T) == 4) {
-        const float2 *b2 = reinterpret_cast<const float2 *>(bdt2);
+__device__ __forceinline__ T node_value(const T *__restrict__ s_val, uint32_t off) {
+    return *reinterpret_cast<const T *>(reinterpret_cast<const char *>(s_val) + off * (sizeof(T) / 4));
+}
+
+// FP32: the whole record in registers.  rec: the patch's entry of row 0.  The
+// rows of a star of up to six ring nodes are loaded before its size is known.
+template <int D>
+struct StarF {
+    uint4 v[kStarVec<D>];
+    __device__ __forceinline__ uint32_t word(int k) const {
+        const uint4 &q = v[k / 4];
+        return k % 4 == 0 ? q.x : k % 4 == 1 ? q.y : k % 4 == 2 ? q.z : q.w;
+    }
+    __device__ __forceinline__ float weight(int k) const { return __uint_as_float(word(kStarIds + k)); }
+    __device__ __forceinline__ StarIds ids() const {
+        return StarIds{{word(0), word(1), word(2), word(3), word(4)}};
+    }
+    __device__ __forceinline__ void load(const uint4 *__restrict__ rec) {
+        constexpr int n = D == 3 ? 6 : kStarVec<D>;
 #pragma unroll
-        for (int k = 0; k < kPatchMax / 2; ++k) {
-            const float2 v = __ldg(b2 + k);
-            bd[2 * k] = (T)v.x;
-            bd[2 * k + 1] = (T)v.y;
-        }
-    } else {
-        const double2 *b2 = reinterpret_cast<const double2 *>(bdt2);
+        for (int k = 0; k < n; ++k) v[k] = __ldg(rec + k * kStarLanes);
+        if (D == 3 && ids().nr() == 7) v[6] = __ldg(rec + 6 * kStarLanes);
+    }
+    __device__ __forceinline__ void load_shared(const uint4 *rec) {
+        constexpr int n = D == 3 ? 6 : kStarVec<D>;
 #pragma unroll
-        for (int k = 0; k < kPatchMax / 2; ++k) {
-            const double2 v = __ldg(b2 + k);
-            bd[2 * k] = (T)v.x;
-            bd[2 * k + 1] = (T)v.y;
+        for (int k = 0; k < n; ++k) v[k] = rec[k * kStarLanes];
+        if (D == 3 && ids().nr() == 7) v[6] = rec[6 * kStarLanes];
+    }
+};
+// FP64 weights of a star of NR ring nodes.
+template <int D, int NR>
+struct StarD {
+    static constexpr int n = D == 3 ? (4 + 3 * (NR - 1) + 1) / 2 : (2 + 2 * (NR - 1)) / 2;
+    double2 v[n];
+    __device__ __forceinline__ double weight(int k) const { return k & 1 ? v[k / 2].y : v[k / 2].x; }
+    __device__ __forceinline__ void load(const double2 *__restrict__ wt) {
+#pragma unroll
+        for (int k = 0; k < n; ++k) v[k] = __ldg(wt + k * kStarLanes);
+    }
+};
+
+template <int D, int NR, typename T, typename W>
+__device__ __forceinline__ void star_eval_nr(const W &S, const StarIds &id, const T *__restrict__ s_val,
+                                             T *__restrict__ out) {
+    constexpr int w0 = D == 3 ? 2 : 1;   // first weight of ring node 0
+    const T va = node_value(s_val, id.a());
+    T vb = T(0), oa = T(0), ob = T(0);
+    if (D == 3) {
+        vb = node_value(s_val, id.b());
+        oa = S.weight(0) * (vb - va);
+        ob = -oa;
+    }
+    T v0 = T(0), first = T(0), pv = T(0), po = T(0);
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+        const int w = j == 0 ? w0 : w0 + (D - 1) + D * (j - 1);
+        const T v = node_value(s_val, id.ring(j));
+        T d = v - va;
+        oa = fma(S.weight(w), d, oa);
+        T o = -(S.weight(w) * d);
+        if (D == 3) {
+            d = v - vb;
+            ob = fma(S.weight(w + 1), d, ob);
+            o = fma(-S.weight(w + 1), d, o);
         }
+        if (j == 0) {
+            v0 = v;
+        } else {
+            d = v - pv;
+            po = fma(S.weight(w + D - 1), d, po);
+            o = fma(-S.weight(w + D - 1), d, o);
+            if (j == 1) first = po; else out[2 + j - 1] = po;
+        }
+        pv = v;
+        po = o;
+    }
+    const T wrap = S.weight(D == 3 ? 1 : 0);
+    const T d = v0 - pv;
+    out[2 + NR - 1] = fma(wrap, d, po);
+    out[2] = fma(-wrap, d, first);
+    out[0] = oa;
+    if (D == 3) out[1] = ob;
+}
+template <int D>
+__device__ __forceinline__ void star_eval(const StarF<D> &S, const float *__restrict__ s_val, float *__restrict__ out) {
+    const StarIds id = S.ids();
+    switch (id.nr()) {
+        case 6: star_eval_nr<D, 6>(S, id, s_val, out); break;
+        case 7: star_eval_nr<D, 7>(S, id, s_val, out); break;
+        case 5: star_eval_nr<D, 5>(S, id, s_val, out); break;
+        case 4: star_eval_nr<D, 4>(S, id, s_val, out); break;
+        case 3: star_eval_nr<D, 3>(S, id, s_val, out); break;
+        default: star_eval_nr<D, 2>(S, id, s_val, out); break;
+    }
+}
+__device__ __forceinline__ StarIds star_ids(const uint4 *__restrict__ rec) {
+    const uint4 q = __ldg(rec);
+    return StarIds{{q.x, q.y, q.z, q.w, __ldg(reinterpret_cast<const uint32_t *>(rec + kStarLanes))}};
+}
+template <int D, int NR>
+__device__ __forceinline__ void star_eval64_nr(const double2 *__restrict__ wt, const StarIds &id,
+                                               const double *__restrict__ s_val, double *__restrict__ out) {
+    StarD<D, NR> S;
+    S.load(wt);
+    star_eval_nr<D, NR>(S, id, s_val, out);
+}
+template <int D>
+__device__ __forceinline__ void star_eval64(const StarIds &id, const double2 *__restrict__ wt,
+                                            const double *__restrict__ s_val, double *__restrict__ out) {
+    switch (id.nr()) {
+        case 6: star_eval64_nr<D, 6>(wt, id, s_val, out); break;
+        case 7: star_eval64_nr<D, 7>(wt, id, s_val, out); break;
+        case 5: star_eval64_nr<D, 5>(wt, id, s_val, out); break;
+        case 4: star_eval64_nr<D, 4>(wt, id, s_val, out); break;
+        case 3: star_eval64_nr<D, 3>(wt, id, s_val, out); break;
+        default: star_eval64_nr<D, 2>(wt, id, s_val, out); break;
     }
 }
 
-// lumped: the mass term by vertex quadrature (int alpha_h phi_i phi_j ~
-// delta_ij alpha_i |T| / (d+1) per element: the mass-lumped variant), else
-// the consistent form above.
-template <int D, typename T, typename N4, bool DIAG, bool LUMP = false>
-__device__ __forceinline__ void patch_eval(const N4 *__restrict__ s_node, const T *__restrict__ s_val,
-                                           const uint16_t *__restrict__ rec, const T (&bd)[kPatchMax],
-                                           T *__restrict__ out) {
-    constexpr bool lumped = LUMP;
-    // the 24-byte record as three 8-byte loads: [m, a, b, r0], [r1..r4], [r5, r6, -, -]
-    const ushort4 q0 = reinterpret_cast<const ushort4 *>(rec)[0];
-    const ushort4 q1 = reinterpret_cast<const ushort4 *>(rec)[1];
-    const ushort4 q2 = reinterpret_cast<const ushort4 *>(rec)[2];
-    const int pm = q0.x;
-    const int ring[7] = {q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y};
-    const int ia = q0.y;
-    const N4 A = s_node[ia];
-    const T va = DIAG ? T(0) : s_val[ia];
-    const T aa = fabs(A.w);
-    T acc_a = T(0), acc_b = T(0);
-    if (D == 3) {
-        const int ib = q0.z;
-        const N4 B = s_node[ib];
-        const T vb = DIAG ? T(0) : s_val[ib];
-        const T ab = fabs(B.w);
-        const T e1x = B.x - A.x, e1y = B.y - A.y, e1z = B.z - A.z;
-        N4 R0 = s_node[ring[0]];
-        T v0 = DIAG ? T(0) : s_val[ring[0]];
-        T d0x = R0.x - A.x, d0y = R0.y - A.y, d0z = R0.z - A.z;
-        T w0x = e1y * d0z - e1z * d0y, w0y = e1z * d0x - e1x * d0z, w0z = e1x * d0y - e1y * d0x;
-        T acc_c = T(0);
+// Weights and row sums of one patch from its elements: with cm = |T| d! /
+// (d+3)! (= |det|/720 in 3D, |det|/120 in 2D) and S the sum of an element's
+// alpha (int lambda^a = d! |T| prod(a_i!) / (d + sum a_i)!),
+//   consistent: A_ij = b G_ij + cm (S + alpha_i + alpha_j),  m_i = (d+3) cm (S + alpha_i)
+//   lumped:     A_ij = b G_ij,                               m_i = |det|/(d+1)! alpha_i
+// with b = beta dt^2 and G_ij = c_i . c_j / (d! |det|) the element's stiffness
+// weights, computed once per mesh (kGeoWords).  geo: the patch's entry of row
+// 0 of element 0; bd: its elements' beta dt^2; al: alpha of the local nodes;
+// w32, w64: the patch's record and weights; mass[slot]: the row sums.
+template <int D>
+__device__ __forceinline__ void star_build(const StarIds &id, const double *__restrict__ geo,
+                                           const double (&bd)[kPatchMax], const double *__restrict__ al, bool lumped,
+                                           float *__restrict__ w32, double *__restrict__ w64,
+                                           double *__restrict__ mass) {
+    constexpr int GW = kGeoWords<D>;
+    const int nr = id.nr();
+    const bool closed = id.closed();
+    const int m = closed ? nr : nr - 1;
+    auto alpha_of = [&](uint32_t off) { return fabs(node_value(al, off)); };
+    const double aa = alpha_of(id.a()), ab = D == 3 ? alpha_of(id.b()) : 0.0;
+    const double cmf = lumped ? 0.0 : (D == 3 ? 1.0 / 720.0 : 1.0 / 120.0);
+    const double clf = D == 3 ? 1.0 / 24.0 : 1.0 / 6.0;
+    double wab = 0.0, ma = 0.0, mb = 0.0;
+    double wa0 = 0.0, wb0 = 0.0, m0 = 0.0;           // ring node 0 (a closed star's last element adds to it)
+    double pa = 0.0, pb = 0.0, pm = 0.0, wrap = 0.0; // the current ring node, its edge to the next element's
+    auto put = [&](int k, double v) {                // weight k
+        w64[(k / 2) * 2 * kStarLanes + k % 2] = v;
+        w32[((kStarIds + k) / 4) * 4 * kStarLanes + (kStarIds + k) % 4] = (float)v;
+    };
+    auto first_w = [](int j) { return (D == 3 ? 4 : 2) + D * (j - 1); };   // first weight of ring node j >= 1
+    double a0 = alpha_of(id.ring(0));
+    // the next element's words are loaded while this one is computed
+    double gc[GW], gn[GW];
 #pragma unroll
-        for (int j = 0; j < kPatchMax; ++j) {
-            if (j >= pm) break;
-            const N4 R1 = s_node[ring[j + 1]];
-            const T v1 = DIAG ? T(0) : s_val[ring[j + 1]];
-            const T d1x = R1.x - A.x, d1y = R1.y - A.y, d1z = R1.z - A.z;
-            const T w1x = e1y * d1z - e1z * d1y, w1y = e1z * d1x - e1x * d1z, w1z = e1x * d1y - e1y * d1x;
-            const T c1x = d0y * d1z - d0z * d1y, c1y = d0z * d1x - d0x * d1z, c1z = d0x * d1y - d0y * d1x;
-            const T ad = fabs(e1x * c1x + e1y * c1y + e1z * c1z);
-            const T kc = fdiv_fast(bd[j], T(6) * ad);
-            const T a2 = fabs(R0.w), a3 = fabs(R1.w);
-            const T S = (aa + ab) + (a2 + a3);
-            const T cm = ad * T(1.0 / 720.0);
-            T o0, o1, o2, o3;
-            if (DIAG) {
-                const T c0x = -(c1x - w1x + w0x), c0y = -(c1y - w1y + w0y), c0z = -(c1z - w1z + w0z);
-                const T cl = ad * T(1.0 / 24.0);
-                o0 = (lumped ? cl * aa : cm * (T(2) * S + T(4) * aa)) + kc * (c0x * c0x + c0y * c0y + c0z * c0z);
-                o1 = (lumped ? cl * ab : cm * (T(2) * S + T(4) * ab)) + kc * (c1x * c1x + c1y * c1y + c1z * c1z);
-                o2 = (lumped ? cl * a2 : cm * (T(2) * S + T(4) * a2)) + kc * (w1x * w1x + w1y * w1y + w1z * w1z);
-                o3 = (lumped ? cl * a3 : cm * (T(2) * S + T(4) * a3)) + kc * (w0x * w0x + w0y * w0y + w0z * w0z);
-            } else {
-                // g = (vb - va) c1 + (v0 - va) c2 + (v1 - va) c3, c2 = -w1, c3 = w0
-                const T t1 = vb - va, t2 = v0 - va, t3 = v1 - va;
-                const T gx = t1 * c1x - t2 * w1x + t3 * w0x;
-                const T gy = t1 * c1y - t2 * w1y + t3 * w0y;
-                const T gz = t1 * c1z - t2 * w1z + t3 * w0z;
-                const T k1 = kc * (c1x * gx + c1y * gy + c1z * gz);
-                const T k2 = -kc * (w1x * gx + w1y * gy + w1z * gz);
-                const T k3 = kc * (w0x * gx + w0y * gy + w0z * gz);
-                const T k0 = -(k1 + k2 + k3);
-                if constexpr (lumped) {
-                    const T cl = ad * T(1.0 / 24.0);
-                    o0 = cl * aa * va + k0;
-                    o1 = cl * ab * vb + k1;
-                    o2 = cl * a2 * v0 + k2;
-                    o3 = cl * a3 * v1 + k3;
-                } else {
-                    const T X = (va + vb) + (v0 + v1);
-                    const T Q = (aa * va + ab * vb) + (a2 * v0 + a3 * v1);
-                    const T base = S * X + Q;
-                    o0 = cm * (base + S * va + aa * (X + T(2) * va)) + k0;
-                    o1 = cm * (base + S * vb + ab * (X + T(2) * vb)) + k1;
-                    o2 = cm * (base + S * v0 + a2 * (X + T(2) * v0)) + k2;
-                    o3 = cm * (base + S * v1 + a3 * (X + T(2) * v1)) + k3;
-                }
-            }
-            acc_a += o0;
-            acc_b += o1;
-            out[2 + j] = acc_c + o2;
-            acc_c = o3;
-            d0x = d1x; d0y = d1y; d0z = d1z;
-            w0x = w1x; w0y = w1y; w0z = w1z;
-            R0 = R1;
-            v0 = v1;
-        }
-        out[2 + pm] = acc_c;
-        out[0] = acc_a;
-        out[1] = acc_b;
-    } else {
-        N4 R0 = s_node[ring[0]];
-        T v0 = DIAG ? T(0) : s_val[ring[0]];
-        T d0x = R0.x - A.x, d0y = R0.y - A.y;
-        T acc_c = T(0);
+    for (int k = 0; k < GW; ++k) gn[k] = __ldg(geo + k * kStarLanes);
 #pragma unroll
-        for (int j = 0; j < kPatchMax; ++j) {
-            if (j >= pm) break;
-            const N4 R1 = s_node[ring[j + 1]];
-            const T v1 = DIAG ? T(0) : s_val[ring[j + 1]];
-            const T d1x = R1.x - A.x, d1y = R1.y - A.y;
-            // c1 = perp(d1) = (d1y, -d1x), c2 = -perp(d0) = (-d0y, d0x)
-            const T c1x = d1y, c1y = -d1x, c2x = -d0y, c2y = d0x;
-            const T ad = fabs(d0x * d1y - d0y * d1x);
-            const T kc = fdiv_fast(bd[j], T(2) * ad);
-            const T a1 = fabs(R0.w), a2 = fabs(R1.w);
-            const T S = aa + a1 + a2;
-            const T cm = ad * T(1.0 / 120.0);
-            T o0, o1, o2;
-            if (DIAG) {
-                const T c0x = -(c1x + c2x), c0y = -(c1y + c2y);
-                const T cl = ad * T(1.0 / 6.0);
-                o0 = (lumped ? cl * aa : cm * (T(2) * S + T(4) * aa)) + kc * (c0x * c0x + c0y * c0y);
-                o1 = (lumped ? cl * a1 : cm * (T(2) * S + T(4) * a1)) + kc * (c1x * c1x + c1y * c1y);
-                o2 = (lumped ? cl * a2 : cm * (T(2) * S + T(4) * a2)) + kc * (c2x * c2x + c2y * c2y);
-            } else {
-                const T t1 = v0 - va, t2 = v1 - va;
-                const T gx = t1 * c1x + t2 * c2x, gy = t1 * c1y + t2 * c2y;
-                const T k1 = kc * (c1x * gx + c1y * gy);
-                const T k2 = kc * (c2x * gx + c2y * gy);
-                const T k0 = -(k1 + k2);
-                if constexpr (lumped) {
-                    const T cl = ad * T(1.0 / 6.0);
-                    o0 = cl * aa * va + k0;
-                    o1 = cl * a1 * v0 + k1;
-                    o2 = cl * a2 * v1 + k2;
-                } else {
-                    const T X = va + v0 + v1, Q = aa * va + a1 * v0 + a2 * v1;
-                    const T base = S * X + Q;
-                    o0 = cm * (base + S * va + aa * (X + T(2) * va)) + k0;
-                    o1 = cm * (base + S * v0 + a1 * (X + T(2) * v0)) + k1;
-                    o2 = cm * (base + S * v1 + a2 * (X + T(2) * v1)) + k2;
-                }
-            }
-            acc_a += o0;
-            out[2 + j] = acc_c + o1;
-            acc_c = o2;
-            d0x = d1x; d0y = d1y;
-            R0 = R1;
-            v0 = v1;
+    for (int j = 0; j < kPatchMax; ++j) {
+        if (j >= m) break;
+#pragma unroll
+        for (int k = 0; k < GW; ++k) gc[k] = gn[k];
+        if (j + 1 < kPatchMax && j + 1 < m) {
+#pragma unroll
+            for (int k = 0; k < GW; ++k) gn[k] = __ldg(geo + ((j + 1) * GW + k) * kStarLanes);
         }
-        out[2 + pm] = acc_c;
-        out[0] = acc_a;
+        const bool last = closed && j == m - 1;
+        const double a1 = alpha_of(last ? id.ring(0) : id.ring(j + 1));
+        const double b = bd[j];
+        const double gAB = D == 3 ? gc[0] : 0.0, gA0 = gc[D == 3 ? 1 : 0], gA1 = gc[D == 3 ? 2 : 1];
+        const double gB0 = D == 3 ? gc[3] : 0.0, gB1 = D == 3 ? gc[4] : 0.0, g01 = gc[D == 3 ? 5 : 2];
+        const double ad = gc[GW - 1];
+        const double cm = ad * cmf;
+        const double S = (aa + ab) + (a0 + a1);
+        const double sa = S + aa, sb = S + ab, s0 = S + a0, s1 = S + a1;
+        if (lumped) {
+            const double cl = ad * clf;
+            ma = fma(cl, aa, ma);
+            mb = fma(cl, ab, mb);
+            pm = fma(cl, a0, pm);
+        } else {
+            const double cr = (D + 3) * cm;
+            ma = fma(cr, sa, ma);
+            mb = fma(cr, sb, mb);
+            pm = fma(cr, s0, pm);
+        }
+        if (D == 3) {
+            wab = fma(b, gAB, fma(cm, sa + ab, wab));
+            pb = fma(b, gB0, fma(cm, sb + a0, pb));
+        }
+        pa = fma(b, gA0, fma(cm, sa + a0, pa));
+        const double w01 = fma(b, g01, cm * (s0 + a1));
+        // ring node j is complete, except node 0 (the wrapping element may add to it)
+        if (j == 0) {
+            wa0 = pa;
+            wb0 = pb;
+            m0 = pm;
+        } else {
+            put(first_w(j), pa);
+            if (D == 3) put(first_w(j) + 1, pb);
+            mass[2 + j] = pm;
+        }
+        pa = fma(b, gA1, cm * (sa + a1));
+        pb = D == 3 ? fma(b, gB1, cm * (sb + a1)) : 0.0;
+        pm = lumped ? ad * clf * a1 : (D + 3) * cm * s1;
+        if (last) {
+            wa0 += pa;
+            wb0 += pb;
+            m0 += pm;
+            wrap = w01;
+        } else {
+            // edge (r_j, r_{j+1}) belongs to ring node j + 1
+            put(first_w(j + 1) + D - 1, w01);
+        }
+        a0 = a1;
     }
-}
-
-// FP64 evaluation of one star patch from geometry computed once per mesh on
-// the host (mesh upload): for every element slot the symmetric stiffness
-// weights G_ab = c_a.c_b / (d! |det|) of its vertex pairs (K^e_ab = beta G_ab)
-// and |det|.  The element arithmetic per tet drops to differences, products
-// and sums (no cross products, no division), which is what matters on a GPU
-// whose FP64 rate is a small fraction of its FP32 rate.  The result equals
-// patch_eval<D, double, ...> up to rounding.
-// Slot layout, 3D (8 doubles): G_AB, G_A0, G_A1, G_B0, G_B1, G_01, |det|, 0
-// with A, B the patch's edge and 0, 1 ring nodes j, j+1; 2D (4 doubles):
-// G_A0, G_A1, G_01, |det|.  Rows of G sum to zero (sum_a c_a = 0), so
-// (K^e v)_a = beta sum_b G_ab (v_b - v_a) and G_aa = -sum_{b != a} G_ab.
-template <int D, bool DIAG, bool LUMP>
-__device__ __forceinline__ void patch_eval_geo(const NodeD *__restrict__ s_node, const double *__restrict__ s_val,
-                                               const uint16_t *__restrict__ rec, const double (&bd)[kPatchMax],
-                                               const double *__restrict__ geo, double *__restrict__ out) {
-    const ushort4 q0 = reinterpret_cast<const ushort4 *>(rec)[0];
-    const ushort4 q1 = reinterpret_cast<const ushort4 *>(rec)[1];
-    const ushort4 q2 = reinterpret_cast<const ushort4 *>(rec)[2];
-    const int pm = q0.x;
-    const int ring[7] = {q0.w, q1.x, q1.y, q1.z, q1.w, q2.x, q2.y};
-    const int ia = q0.y;
-    const double aa = fabs(s_node[ia].w);
-    const double va = DIAG ? 0.0 : s_val[ia];
-    double acc_a = 0.0, acc_b = 0.0, acc_c = 0.0;
-    if (D == 3) {
-        const int ib = q0.z;
-        const double ab = fabs(s_node[ib].w);
-        const double vb = DIAG ? 0.0 : s_val[ib];
-        double a2 = fabs(s_node[ring[0]].w);
-        double v0 = DIAG ? 0.0 : s_val[ring[0]];
-        const double2 *g2 = reinterpret_cast<const double2 *>(geo);
-#pragma unroll
-        for (int j = 0; j < kPatchMax; ++j) {
-            if (j >= pm) break;
-            const double2 g0 = __ldg(g2 + 4 * j), g1 = __ldg(g2 + 4 * j + 1), gg = __ldg(g2 + 4 * j + 2),
-                          g3 = __ldg(g2 + 4 * j + 3);
-            const double gAB = g0.x, gA0 = g0.y, gA1 = g1.x, gB0 = g1.y, gB1 = gg.x, g01 = gg.y, ad = g3.x;
-            const int r1 = ring[j + 1];
-            const double a3 = fabs(s_node[r1].w);
-            const double v1 = DIAG ? 0.0 : s_val[r1];
-            const double b = bd[j];
-            double o0, o1, o2, o3;
-            if (DIAG) {
-                const double kA = -(gAB + gA0 + gA1), kB = -(gAB + gB0 + gB1), k0 = -(gA0 + gB0 + g01),
-                             k1 = -(gA1 + gB1 + g01);
-                if (LUMP) {
-                    const double cl = ad * (1.0 / 24.0);
-                    o0 = cl * aa + b * kA;
-                    o1 = cl * ab + b * kB;
-                    o2 = cl * a2 + b * k0;
-                    o3 = cl * a3 + b * k1;
-                } else {
-                    const double cm = ad * (1.0 / 720.0);
-                    const double S = (aa + ab) + (a2 + a3);
-                    o0 = cm * (2.0 * S + 4.0 * aa) + b * kA;
-                    o1 = cm * (2.0 * S + 4.0 * ab) + b * kB;
-                    o2 = cm * (2.0 * S + 4.0 * a2) + b * k0;
-                    o3 = cm * (2.0 * S + 4.0 * a3) + b * k1;
-                }
-            } else {
-                const double wAB = gAB * (vb - va), wA0 = gA0 * (v0 - va), wA1 = gA1 * (v1 - va);
-                const double wB0 = gB0 * (v0 - vb), wB1 = gB1 * (v1 - vb), w01 = g01 * (v1 - v0);
-                const double kA = b * ((wAB + wA0) + wA1);
-                const double kB = b * ((wB0 + wB1) - wAB);
-                const double k0 = b * (w01 - (wA0 + wB0));
-                const double k1 = -b * ((wA1 + wB1) + w01);
-                if (LUMP) {
-                    const double cl = ad * (1.0 / 24.0);
-                    o0 = cl * aa * va + kA;
-                    o1 = cl * ab * vb + kB;
-                    o2 = cl * a2 * v0 + k0;
-                    o3 = cl * a3 * v1 + k1;
-                } else {
-                    const double cm = ad * (1.0 / 720.0);
-                    const double S = (aa + ab) + (a2 + a3);
-                    const double X = (va + vb) + (v0 + v1);
-                    const double Q = (aa * va + ab * vb) + (a2 * v0 + a3 * v1);
-                    const double base = S * X + Q;
-                    o0 = cm * (base + S * va + aa * (X + 2.0 * va)) + kA;
-                    o1 = cm * (base + S * vb + ab * (X + 2.0 * vb)) + kB;
-                    o2 = cm * (base + S * v0 + a2 * (X + 2.0 * v0)) + k0;
-                    o3 = cm * (base + S * v1 + a3 * (X + 2.0 * v1)) + k1;
-                }
-            }
-            acc_a += o0;
-            acc_b += o1;
-            out[2 + j] = acc_c + o2;
-            acc_c = o3;
-            a2 = a3;
-            v0 = v1;
-        }
-        out[2 + pm] = acc_c;
-        out[0] = acc_a;
-        out[1] = acc_b;
-    } else {
-        double a1 = fabs(s_node[ring[0]].w);
-        double v0 = DIAG ? 0.0 : s_val[ring[0]];
-        const double2 *g2 = reinterpret_cast<const double2 *>(geo);
-#pragma unroll
-        for (int j = 0; j < kPatchMax; ++j) {
-            if (j >= pm) break;
-            const double2 g0 = __ldg(g2 + 2 * j), g1 = __ldg(g2 + 2 * j + 1);
-            const double gA0 = g0.x, gA1 = g0.y, g01 = g1.x, ad = g1.y;
-            const int r1 = ring[j + 1];
-            const double a2 = fabs(s_node[r1].w);
-            const double v1 = DIAG ? 0.0 : s_val[r1];
-            const double b = bd[j];
-            double o0, o1, o2;
-            if (DIAG) {
-                const double kA = -(gA0 + gA1), k0 = -(gA0 + g01), k1 = -(gA1 + g01);
-                if (LUMP) {
-                    const double cl = ad * (1.0 / 6.0);
-                    o0 = cl * aa + b * kA;
-                    o1 = cl * a1 + b * k0;
-                    o2 = cl * a2 + b * k1;
-                } else {
-                    const double cm = ad * (1.0 / 120.0);
-                    const double S = aa + a1 + a2;
-                    o0 = cm * (2.0 * S + 4.0 * aa) + b * kA;
-                    o1 = cm * (2.0 * S + 4.0 * a1) + b * k0;
-                    o2 = cm * (2.0 * S + 4.0 * a2) + b * k1;
-                }
-            } else {
-                const double wA0 = gA0 * (v0 - va), wA1 = gA1 * (v1 - va), w01 = g01 * (v1 - v0);
-                const double kA = b * (wA0 + wA1);
-                const double k0 = b * (w01 - wA0);
-                const double k1 = -b * (wA1 + w01);
-                if (LUMP) {
-                    const double cl = ad * (1.0 / 6.0);
-                    o0 = cl * aa * va + kA;
-                    o1 = cl * a1 * v0 + k0;
-                    o2 = cl * a2 * v1 + k1;
-                } else {
-                    const double cm = ad * (1.0 / 120.0);
-                    const double S = aa + a1 + a2;
-                    const double X = va + v0 + v1, Q = aa * va + a1 * v0 + a2 * v1;
-                    const double base = S * X + Q;
-                    o0 = cm * (base + S * va + aa * (X + 2.0 * va)) + kA;
-                    o1 = cm * (base + S * v0 + a1 * (X + 2.0 * v0)) + k0;
-                    o2 = cm * (base + S * v1 + a2 * (X + 2.0 * v1)) + k1;
-                }
-            }
-            acc_a += o0;
-            out[2 + j] = acc_c + o1;
-            acc_c = o2;
-            a1 = a2;
-            v0 = v1;
-        }
-        out[2 + pm] = acc_c;
-        out[0] = acc_a;
+    if (!closed) {
+        put(first_w(m), pa);
+        if (D == 3) put(first_w(m) + 1, pb);
+        mass[2 + m] = pm;
     }
+    if (D == 3) {
+        put(0, wab);
+        put(1, wrap);
+        put(2, wa0);
+        put(3, wb0);
+        mass[1] = mb;
+    } else {
+        put(0, wrap);
+        put(1, wa0);
+    }
+    mass[2] = m0;
+    mass[0] = ma;
 }
 
 }  // namespace ps

@@ -36,7 +36,7 @@ struct Workspace {
     double *part64 = nullptr;
     double *dot1 = nullptr, *dot2 = nullptr;
     double *pq2 = nullptr, *z3 = nullptr;   // two-kernel CG partials
-    // paired-patch operator kernel: chunk shares of p.Ap, all bits set
+    // operator kernel with the halo: chunk shares of p.Ap, all bits set
     // (0xffffffff, a NaN no arithmetic produces) while not yet written
     float2 *pqu = nullptr;
     // fused CG (FP32): second buffers of x, r, p, w (first: x32, r32, p32,
@@ -44,7 +44,7 @@ struct Workspace {
     float *x32b = nullptr, *r32b = nullptr, *p32b = nullptr, *q32b = nullptr;
     float *s32a = nullptr, *s32b = nullptr, *part32b = nullptr;
     double *dots1 = nullptr;
-    float2 *halo32 = nullptr;   // paired-patch CG: (D^-1 r, p) per chunk-major shared slot
+    float2 *halo32 = nullptr;   // (D^-1 r, p) per chunk-major shared slot
     CgState *st = nullptr;
     CgState *h_st = nullptr;
     float *one32 = nullptr;
@@ -59,7 +59,7 @@ int dalloc(ps_ctx *ctx, void **p, size_t bytes, std::vector<DevAlloc> &owner);
 void dfree_all(ps_ctx *ctx, std::vector<DevAlloc> &owner);
 int grid_for(int64_t n, int dev_sms);
 int cuda_status(cudaError_t e);
-SmemLayout make_layout(int esz, int nsz, int max_loc, int max_patch, int max_inc, int max_sh);
+SmemLayout make_layout(int esz, int max_loc, int max_patch, int max_inc);
 int ensure_workspace(ps_mesh *m);
 template <typename T, int MODE>
 int launch_pass(ps_mesh *m, const VecArgs<T> &a, cudaStream_t s);
@@ -107,15 +107,11 @@ struct ps_mesh {
     int32_t *d_old_of_new = nullptr, *d_new_of_old = nullptr;
     int32_t *d_slave_ptr = nullptr, *d_slave = nullptr;   // merged periodic vertices (null: none)
     int grid2 = 1, grid3 = 1, g3c = 1;
-    ps::SmemLayout pipe_L0, pipe_L1;   // two-stage layout of the pipelined CG kernel
-    int pipe_grid = 0;                 // its persistent grid (0 = not used)
-    int pipeline = 0;                  // ps_mesh_opts::pipeline
+    double *d_lump = nullptr;          // [loc_total] lumped weight of each local node over its chunk's elements
     int update_bps = 0;                // ps_mesh_opts::update_blocks_per_sm
     int k1_variant = 0;                // ps_mesh_opts::operator_kernel
-    bool k1_pre = false;               // FP32 operator kernel variant (beta prefetch)
-    bool use_units = false;            // FP32 CG operator kernel on paired patches (3D)
-    int unit_threads = 128;            // its threads per block (ps_mesh_opts::operator_threads)
-    int32_t *d_uelem = nullptr;        // element of each (unit, element, half) slot, -1 none
+    bool use_halo = false;             // FP32 CG operator kernel with the chunk-major halo (3D)
+    int op_threads = 0;                // its threads per block (ps_mesh_opts::operator_threads)
     bool coeff_ok = false, alpha_set = false;
     bool alpha_newton = false;         // alpha last set by the general-EOS Newton iteration
     double dt2 = 0.0;

@@ -22,11 +22,13 @@ namespace ps {
 constexpr int kPatchMax = 6;     // elements per patch (star) at most
 constexpr int kPatchIds = 12;    // u16 per patch record: m, a, b, ring[0..m], padding
 constexpr int kPatchSlots = 9;   // contribution slots per patch: a, b, ring[0..6]
-// FP64 element geometry per patch slot: 3D G_AB, G_A0, G_A1, G_B0, G_B1, G_01, |det|, pad;
-// 2D G_A0, G_A1, G_01, |det| (G_ab = c_a.c_b / (d! |det|), c_a the cofactor vectors)
+// FP64 element geometry per patch slot: 3D G_AB, G_A0, G_A1, G_B0, G_B1, G_01, |det|;
+// 2D G_A0, G_A1, G_01, |det| (G_ab = c_a.c_b / (d! |det|), c_a the cofactor vectors).
+// Read when the star weights are formed; word k of element j of a patch lies
+// at row j * W + k of its group of 32 patches (kStarLanes).
 template <int D>
-constexpr int kGeoWords = D == 3 ? 8 : 4;
-constexpr int kPatchPad = 4;     // patch segments padded to 4 patches (96 B)
+constexpr int kGeoWords = D == 3 ? 7 : 4;
+constexpr int kPatchPad = 32;    // patch segments padded to whole groups (kStarLanes)
 constexpr int kIncPad = 8;       // incidence segments padded to 8 u16
 constexpr int kIncpPad = 8;      // incidence-pointer segments padded to 8 u16
 constexpr int kShPad = 4;        // shared-id segments padded to 4 int32
@@ -41,29 +43,38 @@ constexpr int kChunkThreads = 256;  // threads of a block that processes a chunk
 // [1] = a, [2] = b (3D), [3 + j] = ring[j], j = 0..m; all local node ids.
 // Contribution slots: 0 -> a, 1 -> b, 2 + j -> ring[j].
 
-// Paired-patch layout of the FP32 3D CG operator kernel (k_cg2_units): the
-// star patches of a chunk are taken two at a time ("units"), two patches of
-// the same size m, so that one thread evaluates both with packed FP32x2
-// arithmetic (one half per patch).  Units are ordered by m, largest first; a
-// size class with an odd count pairs its last patch with itself, and that
-// unit's second half is flagged so its contributions are dropped.  Each
-// chunk holds an even number of units (a pad unit with m = 0 and no element
-// makes it even), so that a chunk's unit records (40 bytes each) and
-// beta*dt^2/6 values (48 bytes each) start and end on 16-byte boundaries.
-//   unit record (u32): [0] = m | kUnitDup (second half duplicate),
-//                      [1] = (a | a' << 16), [2] = (b | b' << 16),
-//                      [3 + j] = (r_j | r'_j << 16), j = 0..m; local node ids
-// Node sums are fixed-point shared-memory integer atomics (exact additions:
-// the result does not depend on their order), so no incidence list is needed.
-constexpr int kURecWords = 10;
-constexpr uint32_t kUnitDup = 0x100u;
-struct ChunkUnits {
-    int32_t unit_off;   // first unit of the chunk
-    int32_t n_unit;
-    int32_t max_star;   // most elements of the chunk around one of its nodes
-    int32_t pad;
-};
-static_assert(sizeof(ChunkUnits) == 16, "ChunkUnits layout");
+// Star weights.  Every operator pass evaluates a patch as one macro element:
+// the sum of its elements' matrices, stored by its edges.  With A^s that sum
+// and m_i = sum_j A^s_ij its row sums (the stiffness part has none, so m_i is
+// the mass of the row: int alpha_h phi_i over the patch),
+//     (A^s v)_i = sum_{j != i} A^s_ij (v_j - v_i) + m_i v_i,
+// so an edge costs one difference and two multiply-adds whatever the number
+// of elements around it, and a constant v meets no cancellation.  The m_i are
+// summed over the chunk once and kept per local node (mrow).  A closed star
+// (ring[m] = ring[0]) has nr = m ring nodes, an open one nr = m + 1.
+// Patches are stored in groups of 32 (every chunk padded to whole groups), 16
+// bytes per lane and row, so that a warp reads a row with one 512-byte load
+// and every row lies at a constant offset from the patch's first:
+//   FP32 record, rows of four words: words 0..4 the ids, 5.. the weights; six
+//           rows hold a star of up to six ring nodes, a 3D mesh with an open
+//           star of six has seven (kStarVec; MeshDev::srows)
+//   FP64 weights, kStarVec64 rows of two
+//   ids: a | b << 16, r0 | r1 << 16, r2 | r3 << 16, r4 | r5 << 16,
+//           r6 | nr << 16 | closed << 20; node ids times 4, the byte offset of an
+//           FP32 value (an uploaded chunk has fewer than 16,384 nodes)
+//   weights, 3D: ab, (r_{nr-1}, r_0) (0 on an open star), (a, r_0), (b, r_0),
+//           then for j = 1..nr-1: (a, r_j), (b, r_j), (r_{j-1}, r_j)
+//   weights, 2D: (r_{nr-1}, r_0), (a, r_0), then for j = 1..nr-1: (a, r_j),
+//           (r_{j-1}, r_j)
+constexpr int kStarIds = 5;
+constexpr int kStarRing = kPatchMax + 1;
+constexpr int kStarLanes = 32;
+template <int D>
+constexpr int kStarW = D == 3 ? 22 : 14;                              // weights of an open star of six
+template <int D>
+constexpr int kStarVec = (kStarIds + kStarW<D> + 3) / 4;              // 7, 5
+template <int D>
+constexpr int kStarVec64 = kStarW<D> / 2;                             // 11, 7
 
 struct ChunkDesc {
     int32_t patch_off;  // first (padded) patch of the chunk

@@ -532,11 +532,14 @@ std::string prepare_mesh(int dim, int64_t n_nodes, const double *coords, int64_t
         const int64_t np_pad = round_up(np, kPatchPad);
         m.pids.resize((patch_off + np_pad) * kPatchIds, 0);
         m.elem_src.resize((patch_off + np_pad) * kPatchMax, -1);
+        m.sids.resize((patch_off + np_pad) * kStarIds, 0);
         std::vector<int32_t> cnt(cd.n_loc + 1, 0);
         auto each_slot = [&](const PatchRec &P, auto &&fn) {
             fn(P.a, 0);
             if (dim == 3) fn(P.b, 1);
-            for (int j = 0; j <= P.m; ++j) fn(P.ring[j], 2 + j);
+            // a closed star's last ring node is its first
+            const int nr = P.m >= 2 && P.ring[P.m] == P.ring[0] ? P.m : P.m + 1;
+            for (int j = 0; j < nr; ++j) fn(P.ring[j], 2 + j);
         };
         for (int q = 0; q < np; ++q) {
             const PatchRec &P = patches[q];
@@ -547,6 +550,14 @@ std::string prepare_mesh(int dim, int64_t n_nodes, const double *coords, int64_t
             for (int j = 0; j <= P.m; ++j) rec[3 + j] = (uint16_t)P.ring[j];
             for (int j = 0; j < P.m; ++j)
                 m.elem_src[(patch_off + q) * kPatchMax + j] = order[chunk_begin[c] + P.elem[j]];
+            const bool closed = P.m >= 2 && P.ring[P.m] == P.ring[0];
+            const int nr = closed ? P.m : P.m + 1;
+            auto off = [](uint32_t l) { return (4u * l) & 0xffffu; };   // (a mesh with more nodes per chunk is not uploaded)
+            uint32_t ids[2 * kStarIds] = {off(rec[1]), off(rec[2])};
+            for (int j = 0; j < nr; ++j) ids[2 + j] = off(rec[3 + j]);
+            ids[2 * kStarIds - 1] = (uint32_t)nr | (closed ? 16u : 0u);
+            for (int k = 0; k < kStarIds; ++k)
+                m.sids[(patch_off + q) * kStarIds + k] = ids[2 * k] | ids[2 * k + 1] << 16;
             each_slot(P, [&](int node, int) { cnt[node + 1]++; });
         }
         for (int32_t l = 0; l < cd.n_loc; ++l) cnt[l + 1] += cnt[l];
@@ -621,78 +632,6 @@ std::string prepare_mesh(int dim, int64_t n_nodes, const double *coords, int64_t
         m.sh_info[4 * k + 2] = m.shr_ptr[s + 1];
         m.sh_info[4 * k + 3] = m.shr_slot[m.shr_ptr[s]] == k ? 1 : 0;
     }
-    if (dim == 3) return build_units(m);
-    return "";
-}
-
-std::string build_units(PrepMesh &m) {
-    if (m.dim != 3) return "paired-patch layout: 3D only";
-    m.chunks_u.assign(m.n_chunks, ChunkUnits{});
-    m.urec.clear();
-    m.uelem.clear();
-    m.unit_total = 0;
-    m.max_unit = 0;
-    struct Ref { int p, m; };
-    std::vector<Ref> ps;
-    std::vector<int> star;
-    for (int c = 0; c < m.n_chunks; ++c) {
-        const ChunkDesc &cd = m.chunks[c];
-        ChunkUnits &cu = m.chunks_u[c];
-        // patches by size, largest first (stable), paired two by two
-        ps.clear();
-        for (int q = 0; q < cd.n_patch; ++q) ps.push_back({q, (int)m.pids[(size_t)(cd.patch_off + q) * kPatchIds]});
-        std::stable_sort(ps.begin(), ps.end(), [](const Ref &x, const Ref &y) { return x.m > y.m; });
-        std::vector<std::array<int, 2>> units;
-        for (size_t i = 0; i < ps.size();) {
-            if (i + 1 < ps.size() && ps[i + 1].m == ps[i].m) {
-                units.push_back({ps[i].p, ps[i + 1].p});
-                i += 2;
-            } else {
-                units.push_back({ps[i].p, -1});   // paired with itself
-                i += 1;
-            }
-        }
-        // an even count per chunk: every chunk's records start and end on a
-        // 16-byte boundary (bulk copies); the pad unit has no element (m = 0)
-        if (units.size() & 1) units.push_back({-1, -1});
-        const int nu = (int)units.size();
-        cu.unit_off = (int32_t)m.unit_total;
-        cu.n_unit = nu;
-        star.assign(cd.n_loc, 0);
-        for (int u = 0; u < nu; ++u) {
-            uint32_t w[kURecWords] = {0};
-            int32_t el[kPatchMax * 2];
-            for (int k = 0; k < kPatchMax * 2; ++k) el[k] = -1;
-            int pm = 0;
-            for (int h = 0; h < 2 && units[u][0] >= 0; ++h) {
-                const bool dup = units[u][h] < 0;
-                const int q = dup ? units[u][0] : units[u][h];
-                const uint16_t *rec = &m.pids[(size_t)(cd.patch_off + q) * kPatchIds];
-                pm = rec[0];
-                const int shift = 16 * h;
-                w[0] = (uint32_t)pm | (dup ? kUnitDup : 0u);
-                w[1] |= (uint32_t)rec[1] << shift;
-                w[2] |= (uint32_t)rec[2] << shift;
-                for (int j = 0; j <= pm; ++j) w[3 + j] |= (uint32_t)rec[3 + j] << shift;
-                if (dup) continue;   // no element behind the duplicate half
-                for (int j = 0; j < pm; ++j) {
-                    el[2 * j + h] = m.elem_src[(size_t)(cd.patch_off + q) * kPatchMax + j];
-                    // elements around each of the element's vertices (a, b, r_j, r_{j+1})
-                    star[rec[1]]++;
-                    star[rec[2]]++;
-                    star[rec[3 + j]]++;
-                    star[rec[4 + j]]++;
-                }
-            }
-            for (int k = 0; k < kURecWords; ++k) m.urec.push_back(w[k]);
-            for (int k = 0; k < kPatchMax * 2; ++k) m.uelem.push_back(el[k]);
-        }
-        int ms = 1;
-        for (int l = 0; l < cd.n_loc; ++l) ms = std::max(ms, star[l]);
-        cu.max_star = ms;
-        m.unit_total += nu;
-        m.max_unit = std::max(m.max_unit, nu);
-    }
     return "";
 }
 
@@ -718,7 +657,16 @@ std::string validate_prep(const PrepMesh &m, const int32_t *conn) {
             if (pm < 1 || pm > kPatchMax) return "bad patch size";
             slot_node[q * kPatchSlots + 0] = rec[1];
             if (m.dim == 3) slot_node[q * kPatchSlots + 1] = rec[2];
-            for (int j = 0; j <= pm; ++j) slot_node[q * kPatchSlots + 2 + j] = rec[3 + j];
+            const bool closed = pm >= 2 && rec[3 + pm] == rec[3];
+            const int nr = closed ? pm : pm + 1;
+            for (int j = 0; j < nr; ++j) slot_node[q * kPatchSlots + 2 + j] = rec[3 + j];
+            {
+                const uint32_t *w = &m.sids[(int64_t)(cd.patch_off + q) * kStarIds];
+                auto off = [](uint32_t l) { return (4u * l) & 0xffffu; };
+                bool ok = w[0] == (off(rec[1]) | off(rec[2]) << 16) && (w[4] >> 16) == ((uint32_t)nr | (closed ? 16u : 0u));
+                for (int j = 0; j < nr; ++j) ok = ok && ((w[1 + j / 2] >> (16 * (j & 1))) & 0xffffu) == off(rec[3 + j]);
+                if (!ok) return "star record does not match the patch";
+            }
             for (int j = 0; j < pm; ++j) {
                 int32_t src = m.elem_src[(int64_t)(cd.patch_off + q) * kPatchMax + j];
                 if (src < 0 || src >= m.n_elems) return "bad element source";

@@ -45,6 +45,7 @@ struct PrepMesh {
     std::vector<int32_t> slave_ptr, slave;         // [n_dofs + 1], merged vertices per unknown (empty: no merging)
     std::vector<ChunkDesc> chunks;                 // [n_chunks]
     std::vector<uint16_t> pids;                    // [patch_total * kPatchIds]
+    std::vector<uint32_t> sids;                    // [patch_total * kStarIds] ids of the star records (layout.h)
     std::vector<int32_t> elem_src;                 // [patch_total * kPatchMax] original element, -1 unused
     std::vector<uint16_t> incp;                    // [incp_total]
     std::vector<uint16_t> inc;                     // [inc_total] patch * kPatchSlots + slot
@@ -58,18 +59,7 @@ struct PrepMesh {
     // [sh_total * 4] per chunk slot: node id, begin and end of the node's
     // partial-sum range, 1 on the owner slot (the node's first chunk); pads -1, 0, 0, 0
     std::vector<int32_t> sh_info;
-
-    // paired-patch layout (layout.h; 3D only, empty in 2D)
-    std::vector<ChunkUnits> chunks_u;              // [n_chunks]
-    std::vector<uint32_t> urec;                    // [unit_total * kURecWords]
-    std::vector<int32_t> uelem;                    // [unit_total * kPatchMax * 2] element of (tet j, half h), -1 none
-    int64_t unit_total = 0;
-    int max_unit = 0;
 };
-
-// Build the paired-patch layout from a prepared 3D mesh (its patch records
-// and element map).  Returns "" on success.
-std::string build_units(PrepMesh &m);
 
 // Returns "" on success, else an error message (bad input).
 std::string prepare_mesh(int dim, int64_t n_nodes, const double *coords, int64_t n_elems,

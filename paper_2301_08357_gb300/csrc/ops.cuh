@@ -1,17 +1,18 @@
 // Chunked matrix-free P1 operator and the fused CG kernels.
 //
 // One thread block processes one chunk (layout.h):
-//   1. one elected thread moves the chunk's static data (node records,
-//      local connectivity, beta*dt^2, incidence lists, shared-node ids) into
+//   1. one elected thread moves the chunk's incidence pointers and lists into
 //      shared memory with bulk copies signalled on an mbarrier;
 //   2. the block gathers the input vector for its local nodes (contiguous for
 //      interior nodes, through the shared-node ids otherwise), masking
 //      Dirichlet nodes; in CG mode it forms the new search direction
 //      p = D^-1 r + beta p on the fly and stores it for its interior nodes;
-//   3. one thread per element computes the element's (d+1) contributions into
-//      shared memory;
+//   3. one thread per star patch forms the patch's contributions to its nodes
+//      in shared memory, from the patch's record and weights (read coalesced
+//      from global memory: nothing of them is staged);
 //   4. one thread per local node sums its contributions in incidence-list
-//      order and writes its row (interior node) or a partial sum (shared node).
+//      order, adds the row-sum term and writes its row (interior node) or a
+//      partial sum (shared node).
 // A second kernel adds the partial sums of shared nodes in a fixed order.
 // Dot products are accumulated in FP64 per block and reduced by the last
 // block to finish, in a fixed order, so every result is bitwise reproducible.
@@ -20,44 +21,43 @@
 
 namespace ps {
 
-enum Mode : int { kApply = 0, kCG = 1, kResid = 2, kDiag = 3 };
+enum Mode : int { kApply = 0, kResid = 2, kDiag = 3 };
 
 struct SmemLayout {
-    uint32_t node, val, aux, pids, incp, inc, shid, contrib, red, bar, total;
+    uint32_t val, aux, incp, inc, contrib, red, bar, total;
 };
 
-// Shared memory of the paired-patch CG operator kernel (cg2u.cuh): node
-// records | values | fixed-point node sums | partial-sum destinations of the
-// shared nodes | per-thread dot partials | mbarrier.
-struct UnitSmem {
-    uint32_t node, val, acc, shd, urec, ubd, bar, total;
+// Shared memory of k_cg2_stars (cg2s.cuh): the chunk's records, its incidence
+// pointers and lists, node values.
+struct StarSmem {
+    uint32_t rec, incp, inc, val, bar, total;
 };
 
 struct MeshDev {
     int dim, n_chunks;
     int64_t n_nodes, n_int, n_shared, n_pad;
     const ChunkDesc *chunks;
-    const uint16_t *pids;    // [patch_total * kPatchIds]
+    const uint4 *srec;       // star records: ids and FP32 weights (layout.h)
+    int srows;               // rows per record
+    int stream;              // 1: the records exceed what L2 keeps from one pass to the next
+    const uint16_t *inc_rec; // incidence lists of k_cg2_stars (null: not used): contributions in the records' place
+    const double2 *sw64;     // FP64 star weights
+    const float *mrow32;     // [loc_total] row sums of the chunk's patches, sign bit set on Dirichlet nodes
+    const double *mrow64;
     const uint16_t *incp, *inc;
     const int32_t *sh_ids, *shr_ptr, *sh_dest;
     const int4 *sh_info;     // [sh_total] node id, partial range [begin, end), owner flag
-    const NodeF *node32;
-    const NodeD *node64;
-    const float *bdt2_32;
-    const double *bdt2_64;
-    const double *geo64;     // [patch_total * kPatchMax * kGeoWords<dim>] FP64 element geometry
     const float *dinv32;
     const double *dinv64;
+    // what the weights are formed from (k_star_build)
+    const double *geo64;     // [patch_total * kPatchMax * kGeoWords<dim>] element geometry
+    const double *bdt2_64;   // [patch_total * kPatchMax] beta*dt^2 per element slot
+    const double *alpha64;   // [loc_total] alpha of the local nodes, sign bit set on Dirichlet nodes
     const uint8_t *dirichlet;
     int *err;
     int lumped;              // 1: mass term by vertex quadrature (mass-lumped variant)
     SmemLayout sm32, sm64;
-    // paired-patch layout (3D; null in 2D)
-    const ChunkUnits *chunks_u;
-    const uint32_t *urec;    // [unit_total * kURecWords]
-    const float *ubd;        // [unit_total * kPatchMax * 2] beta*dt^2/6 per (unit, element, half)
-    const float *dmax;       // [n_chunks] largest diagonal entry over each chunk's free nodes
-    UnitSmem smu;
+    StarSmem sms;
 };
 
 // Scalars of one CG run, kept on the device.
@@ -76,15 +76,11 @@ enum CgStatus : int { kCgRunning = 0, kCgConverged = 1, kCgMaxIter = 2, kCgBreak
 template <typename T>
 struct VecArgs {
     const T *x;      // apply / resid: input vector
-    T *y;            // apply: output; cg: q; resid: r
+    T *y;            // apply: output; resid: r
     const T *b;      // resid: right-hand side (0 on Dirichlet nodes)
-    T *p;            // cg: search direction (read old, write new)
-    const T *r;      // cg: residual
-    const T *dinv;   // cg: Jacobi inverse diagonal (0 on Dirichlet nodes)
     T *partial;      // [sh_total] partial sums of shared local nodes
-    double *dotbuf;  // per-block dot partials
-    CgState *st;
-    int *host_done;  // optional host-mapped copy of st->done
+    double *dotbuf;  // resid: per-block dot partials
+    CgState *st;     // resid: receives r.r
 };
 
 __device__ __forceinline__ float cg_dir(float dinv, float r, float beta, float p) {
@@ -96,13 +92,11 @@ __device__ __forceinline__ double cg_dir(double dinv, double r, double beta, dou
 
 __device__ __forceinline__ int ld_flag(const int *p) { return *(volatile const int *)p; }
 
-// Shared-memory view of one staged chunk.
+// Shared-memory view of one chunk.
 template <typename T>
 struct ChunkSmem {
-    typename NodeOf<T>::type *node;
     T *val, *aux, *contrib;
-    uint16_t *pids, *incp, *inc;
-    int32_t *shid;
+    uint16_t *incp, *inc;
     uint64_t *bar;
     double *red;
 };
@@ -110,45 +104,44 @@ struct ChunkSmem {
 template <typename T>
 __device__ __forceinline__ ChunkSmem<T> chunk_smem(unsigned char *smem, const SmemLayout &L) {
     ChunkSmem<T> S;
-    S.node = reinterpret_cast<typename NodeOf<T>::type *>(smem + L.node);
     S.val = reinterpret_cast<T *>(smem + L.val);
     S.aux = reinterpret_cast<T *>(smem + L.aux);
     S.contrib = reinterpret_cast<T *>(smem + L.contrib);
-    S.pids = reinterpret_cast<uint16_t *>(smem + L.pids);
     S.incp = reinterpret_cast<uint16_t *>(smem + L.incp);
     S.inc = reinterpret_cast<uint16_t *>(smem + L.inc);
-    S.shid = reinterpret_cast<int32_t *>(smem + L.shid);
     S.bar = reinterpret_cast<uint64_t *>(smem + L.bar);
     S.red = reinterpret_cast<double *>(smem + L.red);
     return S;
 }
 
-// Thread 0 issues the bulk copies of chunk cd's static data (node records,
-// patch records, incidence pointers and lists, shared-node ids).  When the
-// shared memory was used by an earlier chunk, the caller has synchronised the
-// block; the proxy fence orders those generic-proxy reads before the
-// async-proxy writes.
+// Row 0 of patch q of a chunk (kStarLanes patches per group).
+template <int D>
+__device__ __forceinline__ const uint4 *star_rec(const MeshDev &m, const ChunkDesc &cd, int q) {
+    return m.srec + (size_t)((cd.patch_off + q) / kStarLanes) * (m.srows * kStarLanes) + q % kStarLanes;
+}
+template <int D>
+__device__ __forceinline__ const double2 *star_wt64(const MeshDev &m, const ChunkDesc &cd, int q) {
+    return m.sw64 + (size_t)((cd.patch_off + q) / kStarLanes) * (kStarVec64<D> * kStarLanes) + q % kStarLanes;
+}
+template <typename T>
+__device__ __forceinline__ const T *chunk_mrow(const MeshDev &m, const ChunkDesc &cd) {
+    return (sizeof(T) == 4 ? reinterpret_cast<const T *>(m.mrow32) : reinterpret_cast<const T *>(m.mrow64)) +
+           cd.node_off;
+}
+
+// Thread 0 issues the bulk copies of chunk cd's incidence pointers and lists.
+// When the shared memory was used by an earlier chunk, the caller has
+// synchronised the block; the proxy fence orders those generic-proxy reads
+// before the async-proxy writes.
 template <typename T>
 __device__ __forceinline__ void stage_issue(const MeshDev &m, const ChunkDesc &cd, const ChunkSmem<T> &S) {
-    using N4 = typename NodeOf<T>::type;
     if (threadIdx.x != 0) return;
-    const int p_pad = (cd.n_patch + kPatchPad - 1) / kPatchPad * kPatchPad;
-    const int incp_n = (cd.n_loc + 1 + kIncpPad - 1) / kIncpPad * kIncpPad;
-    const int inc_n = (cd.n_inc + kIncPad - 1) / kIncPad * kIncPad;
-    const int sh_n = (cd.n_sh + kShPad - 1) / kShPad * kShPad;
-    const N4 *gnode = (sizeof(T) == 4) ? reinterpret_cast<const N4 *>(m.node32) : reinterpret_cast<const N4 *>(m.node64);
-    const uint32_t b_node = (uint32_t)cd.n_loc * sizeof(N4);
-    const uint32_t b_pids = (uint32_t)p_pad * (kPatchIds * 2u);
-    const uint32_t b_incp = (uint32_t)incp_n * 2u;
-    const uint32_t b_inc = (uint32_t)inc_n * 2u;
-    const uint32_t b_sh = (uint32_t)sh_n * 4u;
+    const uint32_t b_incp = (uint32_t)((cd.n_loc + 1 + kIncpPad - 1) / kIncpPad * kIncpPad) * 2u;
+    const uint32_t b_inc = (uint32_t)((cd.n_inc + kIncPad - 1) / kIncPad * kIncPad) * 2u;
     fence_proxy_async_smem();
-    mbar_arrive_expect_tx(S.bar, b_node + b_pids + b_incp + b_inc + b_sh);
-    bulk_g2s(S.node, gnode + cd.node_off, b_node, S.bar);
-    bulk_g2s(S.pids, m.pids + (size_t)cd.patch_off * kPatchIds, b_pids, S.bar);
+    mbar_arrive_expect_tx(S.bar, b_incp + b_inc);
     bulk_g2s(S.incp, m.incp + cd.incp_off, b_incp, S.bar);
     bulk_g2s(S.inc, m.inc + cd.inc_off, b_inc, S.bar);
-    if (b_sh) bulk_g2s(S.shid, m.sh_ids + cd.sh_off, b_sh, S.bar);
 }
 
 // Wait for the staged data (bounded); block-uniform result.  On timeout the
@@ -165,190 +158,120 @@ __device__ __forceinline__ bool stage_wait(const MeshDev &m, const ChunkSmem<T> 
     return ok;
 }
 
-// Element contributions of every star patch of the chunk into S.contrib
-// (the mesh's mass form chosen once per chunk, so each variant of the loop
-// is compiled on its own).
-template <int D, typename T, bool DIAG>
-__device__ __forceinline__ void patches_eval(const MeshDev &m, const ChunkDesc &cd, const ChunkSmem<T> &S) {
-    using N4 = typename NodeOf<T>::type;
-    const T *gbdt2 = (sizeof(T) == 4) ? reinterpret_cast<const T *>(m.bdt2_32) : reinterpret_cast<const T *>(m.bdt2_64);
-    const T *g_bdt2 = gbdt2 + (size_t)cd.patch_off * kPatchMax;
-    if constexpr (sizeof(T) == 8) {
-        // FP64: element geometry precomputed per slot (patch_eval_geo)
-        constexpr int GW = kGeoWords<D>;
-        const double *g_geo = m.geo64 + (size_t)cd.patch_off * kPatchMax * GW;
-        if (m.lumped) {
-            for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x) {
-                double bd[kPatchMax];
-                load_bd(g_bdt2 + q * kPatchMax, bd);
-                patch_eval_geo<D, DIAG, true>(S.node, S.val, S.pids + q * kPatchIds, bd, g_geo + q * kPatchMax * GW,
-                                              S.contrib + q * kPatchSlots);
-            }
-        } else {
-            for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x) {
-                double bd[kPatchMax];
-                load_bd(g_bdt2 + q * kPatchMax, bd);
-                patch_eval_geo<D, DIAG, false>(S.node, S.val, S.pids + q * kPatchIds, bd, g_geo + q * kPatchMax * GW,
-                                               S.contrib + q * kPatchSlots);
-            }
-        }
-    } else if (m.lumped) {
-        for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x) {
-            T bd[kPatchMax];
-            load_bd(g_bdt2 + q * kPatchMax, bd);
-            patch_eval<D, T, N4, DIAG, true>(S.node, S.val, S.pids + q * kPatchIds, bd, S.contrib + q * kPatchSlots);
-        }
-    } else {
-        for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x) {
-            T bd[kPatchMax];
-            load_bd(g_bdt2 + q * kPatchMax, bd);
-            patch_eval<D, T, N4, DIAG>(S.node, S.val, S.pids + q * kPatchIds, bd, S.contrib + q * kPatchSlots);
-        }
+// Contributions of every star patch of the chunk into S.contrib; ends with a
+// block barrier.  FP32: a thread's first patch may have been loaded earlier
+// (PRE: before the gather, so that its record arrives while the gather waits).
+template <int D, bool PRE>
+__device__ __forceinline__ void stars_eval(const MeshDev &m, const ChunkDesc &cd, const ChunkSmem<float> &S,
+                                           const StarF<D> &pre) {
+    int q = threadIdx.x;
+    if (PRE && q < cd.n_patch) {
+        star_eval<D>(pre, S.val, S.contrib + q * kPatchSlots);
+        q += blockDim.x;
+    }
+    for (; q < cd.n_patch; q += blockDim.x) {
+        StarF<D> st;
+        st.load(star_rec<D>(m, cd, q));
+        star_eval<D>(st, S.val, S.contrib + q * kPatchSlots);
     }
     __syncthreads();
 }
-
-// The same with beta*dt^2 of the thread's first R patches loaded earlier
-// (prefetch_bd, before the staging wait): the element phase then starts
-// without a global-memory round trip.
-constexpr int kBdRounds = 3;
-template <typename T>
-struct BdPrefetch {
-    T v[kBdRounds][kPatchMax];
-};
-template <typename T>
-__device__ __forceinline__ void prefetch_bd(const MeshDev &m, const ChunkDesc &cd, BdPrefetch<T> &P) {
-    const T *gbdt2 = (sizeof(T) == 4) ? reinterpret_cast<const T *>(m.bdt2_32) : reinterpret_cast<const T *>(m.bdt2_64);
-    const T *g_bdt2 = gbdt2 + (size_t)cd.patch_off * kPatchMax;
-#pragma unroll
-    for (int k = 0; k < kBdRounds; ++k) {
-        const int q = threadIdx.x + k * blockDim.x;
-        if (q < cd.n_patch) load_bd(g_bdt2 + q * kPatchMax, P.v[k]);
-    }
-}
-template <int D, typename T, bool LUMP>
-__device__ __forceinline__ void patches_eval_pre_v(const MeshDev &m, const ChunkDesc &cd, const ChunkSmem<T> &S,
-                                                   const BdPrefetch<T> &P) {
-    using N4 = typename NodeOf<T>::type;
-#pragma unroll
-    for (int k = 0; k < kBdRounds; ++k) {
-        const int q = threadIdx.x + k * blockDim.x;
-        if (q < cd.n_patch)
-            patch_eval<D, T, N4, false, LUMP>(S.node, S.val, S.pids + q * kPatchIds, P.v[k],
-                                              S.contrib + q * kPatchSlots);
-    }
-    const T *gbdt2 = (sizeof(T) == 4) ? reinterpret_cast<const T *>(m.bdt2_32) : reinterpret_cast<const T *>(m.bdt2_64);
-    const T *g_bdt2 = gbdt2 + (size_t)cd.patch_off * kPatchMax;
-    for (int q = threadIdx.x + kBdRounds * blockDim.x; q < cd.n_patch; q += blockDim.x) {
-        T bd[kPatchMax];
-        load_bd(g_bdt2 + q * kPatchMax, bd);
-        patch_eval<D, T, N4, false, LUMP>(S.node, S.val, S.pids + q * kPatchIds, bd, S.contrib + q * kPatchSlots);
-    }
-}
-template <int D, typename T>
-__device__ __forceinline__ void patches_eval_pre(const MeshDev &m, const ChunkDesc &cd, const ChunkSmem<T> &S,
-                                                 const BdPrefetch<T> &P) {
-    if (m.lumped)
-        patches_eval_pre_v<D, T, true>(m, cd, S, P);
-    else
-        patches_eval_pre_v<D, T, false>(m, cd, S, P);
+template <int D, bool PRE>
+__device__ __forceinline__ void stars_eval(const MeshDev &m, const ChunkDesc &cd, const ChunkSmem<double> &S,
+                                           const StarF<D> &) {
+    for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x)
+        star_eval64<D>(star_ids(star_rec<D>(m, cd, q)), star_wt64<D>(m, cd, q), S.val, S.contrib + q * kPatchSlots);
     __syncthreads();
 }
+template <int D>
+__device__ __forceinline__ void star_prefetch(const MeshDev &m, const ChunkDesc &cd, StarF<D> &pre) {
+    if ((int)threadIdx.x < cd.n_patch) pre.load(star_rec<D>(m, cd, threadIdx.x));
+}
 
-// Sum of the contributions of local node l in incidence order.
+// Sum of contributions c[inc[k]], k in [b, e): four independent partial sums
+// in a fixed pattern (deterministic).
 template <typename T>
-__device__ __forceinline__ T node_sum(const ChunkSmem<T> &S, int l) {
-    const int b = S.incp[l], e = S.incp[l + 1];
-    // four independent partial sums (fixed pattern: deterministic)
+__device__ __forceinline__ T list_sum(const T *__restrict__ c, const uint16_t *__restrict__ inc, int b, int e) {
     T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
     int k = b;
     for (; k + 3 < e; k += 4) {
-        s0 += S.contrib[S.inc[k]];
-        s1 += S.contrib[S.inc[k + 1]];
-        s2 += S.contrib[S.inc[k + 2]];
-        s3 += S.contrib[S.inc[k + 3]];
+        s0 += c[inc[k]];
+        s1 += c[inc[k + 1]];
+        s2 += c[inc[k + 2]];
+        s3 += c[inc[k + 3]];
     }
-    for (; k < e; ++k) s0 += S.contrib[S.inc[k]];
+    for (; k < e; ++k) s0 += c[inc[k]];
     return (s0 + s1) + (s2 + s3);
 }
+// Sum of the contributions of local node l in incidence order.
+template <typename T>
+__device__ __forceinline__ T node_sum(const ChunkSmem<T> &S, int l) {
+    return list_sum(S.contrib, S.inc, S.incp[l], S.incp[l + 1]);
+}
 
-// Process chunk c.  Returns this thread's share of the mode's dot product
-// (CG: p.q, resid: r.r over interior nodes).  `phase` is the mbarrier parity
-// to wait for; it flips on return.  Block-uniform; contains __syncthreads.
+// Process chunk c (apply, residual).  Returns this thread's share of the
+// residual's r.r over interior nodes.  `phase` is the mbarrier parity to wait
+// for; it flips on return.  Block-uniform; contains __syncthreads.
 template <int D, typename T, int MODE>
 __device__ typename DotOf<T>::type process_chunk(const MeshDev &m, const VecArgs<T> &a, int c, unsigned char *smem,
-                                                 const SmemLayout &L, uint32_t &phase, T beta_cg, bool &failed) {
+                                                 const SmemLayout &L, uint32_t &phase, bool &failed) {
     using Acc = typename DotOf<T>::type;
+    constexpr bool kPre = sizeof(T) == 4;
     const ChunkDesc cd = m.chunks[c];
     const ChunkSmem<T> S = chunk_smem<T>(smem, L);
     const int n_loc = cd.n_loc, n_int = cd.n_int;
     stage_issue<T>(m, cd, S);
-    // interior input values do not depend on the staged data: fetch them
-    // while the bulk copies are in flight (masked below, once records landed)
-    T vin[4];
+    const T *mrow = chunk_mrow<T>(m, cd);
+    StarF<D> pre;
+    if (kPre) star_prefetch<D>(m, cd, pre);
+    // ---- gather the input vector (masked on Dirichlet nodes).  The element
+    // phase of a chunk whose input is zero on all its nodes (a zero first
+    // guess, a zero correction) is skipped: every contribution is then 0.
+    bool nonzero = false;
+    for (int l0 = threadIdx.x; l0 < n_loc; l0 += 4 * blockDim.x) {
+        T v[4], mr[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int l = threadIdx.x + k * blockDim.x;
-        vin[k] = T(0);
-        if (MODE != kDiag && l < n_int) {
-            const int g = cd.int_begin + l;
-            vin[k] = (MODE == kCG) ? cg_dir(a.dinv[g], a.r[g], beta_cg, a.p[g]) : a.x[g];
+        for (int k = 0; k < 4; ++k) {
+            const int l = l0 + k * blockDim.x;
+            v[k] = mr[k] = T(0);
+            if (l < n_loc) {
+                const int g = l < n_int ? cd.int_begin + l : m.sh_ids[cd.sh_off + (l - n_int)];
+                v[k] = a.x[g];
+                mr[k] = mrow[l];
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int l = l0 + k * blockDim.x;
+            if (l < n_loc) {
+                if (is_dirichlet(mr[k])) v[k] = T(0);
+                S.val[l] = v[k];
+                nonzero |= v[k] != T(0);
+            }
         }
     }
     if (!stage_wait<T>(m, S, phase)) {
         failed = true;
         return Acc();
     }
-
-    // ---- gather the input vector (masked on Dirichlet nodes).  Apply and
-    // residual skip the element phase of a chunk whose input is zero on all
-    // its nodes (a zero first guess, a zero correction): every contribution
-    // is then exactly 0.
-    bool nonzero = false;
-    if (MODE != kDiag) {
-        auto finish = [&](int l, T v) {
-            if (is_dirichlet(S.node[l].w)) v = T(0);
-            if (MODE == kCG && l < n_int) a.p[cd.int_begin + l] = v;
-            S.val[l] = v;
-            nonzero |= v != T(0);
-        };
-        auto fetch = [&](int l) -> T {
-            const int g = l < n_int ? cd.int_begin + l : S.shid[l - n_int];
-            return (MODE == kCG) ? cg_dir(a.dinv[g], a.r[g], beta_cg, a.p[g]) : a.x[g];
-        };
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int l = threadIdx.x + k * blockDim.x;
-            if (l < n_loc) finish(l, l < n_int ? vin[k] : fetch(l));
-        }
-        for (int l = threadIdx.x + 4 * blockDim.x; l < n_loc; l += blockDim.x) finish(l, fetch(l));
-    }
-    const bool work = (MODE == kApply || MODE == kResid) ? __syncthreads_or(nonzero) != 0 : true;
-    if (MODE != kDiag && !(MODE == kApply || MODE == kResid)) __syncthreads();
-
-    if (work) patches_eval<D, T, MODE == kDiag>(m, cd, S);
+    const bool work = __syncthreads_or(nonzero) != 0;
+    if (work) stars_eval<D, kPre>(m, cd, S, pre);
 
     // ---- per-node sums in incidence order
     Acc dot;
     for (int l = threadIdx.x; l < n_loc; l += blockDim.x) {
-        T s = work ? node_sum(S, l) : T(0);
-        const bool dir = is_dirichlet(S.node[l].w);
+        const T mr = mrow[l];
+        T s = work ? fma(fabs(mr), S.val[l], node_sum(S, l)) : T(0);
+        const bool dir = is_dirichlet(mr);
         if (dir) s = T(0);
         if (l < n_int) {
             const int g = cd.int_begin + l;
             if (MODE == kApply) {
                 a.y[g] = s;
-            } else if (MODE == kCG) {
-                a.y[g] = s;
-                dot.add_prod(S.val[l], s);
-            } else if (MODE == kResid) {
+            } else {
                 const T rv = dir ? T(0) : a.b[g] - s;
                 a.y[g] = rv;
                 dot.add_prod(rv, rv);
-            } else {  // diag: T == double here
-                const double dv = dir ? 0.0 : 1.0 / (double)s;
-                const_cast<double *>(m.dinv64)[g] = dv;
-                const_cast<float *>(m.dinv32)[g] = (float)dv;
             }
         } else {
             a.partial[m.sh_dest[cd.sh_off + (l - n_int)]] = s;
@@ -357,52 +280,135 @@ __device__ typename DotOf<T>::type process_chunk(const MeshDev &m, const VecArgs
     return dot;
 }
 
-// Kernel 1: one block per chunk.
+// Kernel 1 of an apply or residual: one block per chunk.
 template <int D, typename T, int MODE>
 __global__ void __launch_bounds__(256) k_chunks(MeshDev m, VecArgs<T> a) {
     extern __shared__ __align__(128) unsigned char smem[];
     const SmemLayout &L = (sizeof(T) == 4) ? m.sm32 : m.sm64;
     uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + L.bar);
     double *s_red = reinterpret_cast<double *>(smem + L.red);
-    // CG scalars are read once per block (not per thread: a same-address
-    // hot spot) and broadcast through shared memory.
     if (threadIdx.x == 0) {
-        if (MODE == kCG) {
-            s_red[0] = a.st->beta;
-            s_red[1] = (double)a.st->done;
-        }
         mbar_init(s_bar, 1);
         fence_mbar_init();
     }
     __syncthreads();
-    if (MODE == kCG && s_red[1] != 0.0) return;
-    const T beta_cg = (MODE == kCG) ? (T)s_red[0] : T(0);
-    __syncthreads();
     uint32_t phase = 0;
     bool failed = false;
-    const typename DotOf<T>::type acc = process_chunk<D, T, MODE>(m, a, blockIdx.x, smem, L, phase, beta_cg, failed);
-    if (MODE == kCG || MODE == kResid) {
+    const typename DotOf<T>::type acc = process_chunk<D, T, MODE>(m, a, blockIdx.x, smem, L, phase, failed);
+    if (MODE == kResid) {
         const double dot = block_sum(acc, s_red);
         if (threadIdx.x == 0) a.dotbuf[blockIdx.x] = dot;
     }
 }
 
-// Kernel 2: shared nodes sum their partials in slot order.  The last block to
-// finish also reduces all dot partials (kernel 1's n_first blocks, then this
-// kernel's blocks) and updates the CG scalars.
+// Star weights, row sums and the Jacobi diagonal from the mesh's geometry,
+// alpha and beta*dt^2, one block per chunk.  beta (may be null): the caller's
+// element values, stored as beta*dt^2 per element slot on the way; null: the
+// stored ones.  Row by row the diagonal is D_ii = m_i - sum_j A_ij.  Interior
+// rows are stored here (0 on Dirichlet rows), shared ones as partial sums
+// (k_shared<double, kDiag>).  A pass of the FP64 pipe (about 29 operations
+// per tetrahedron) that reads 64 bytes per tetrahedron.
+template <int D>
+__global__ void __launch_bounds__(256, 3) k_star_build(MeshDev m, const int32_t *__restrict__ elem_src,
+                                                    const double *__restrict__ beta, double dt2, double *partial) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    const ChunkSmem<double> S = chunk_smem<double>(smem, m.sm64);
+    if (threadIdx.x == 0) {
+        mbar_init(S.bar, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    const ChunkDesc cd = m.chunks[blockIdx.x];
+    stage_issue<double>(m, cd, S);
+    for (int l = threadIdx.x; l < cd.n_loc; l += blockDim.x) S.val[l] = m.alpha64[cd.node_off + l];
+    uint32_t phase = 0;
+    if (!stage_wait<double>(m, S, phase)) return;   // also the barrier for S.val
+    auto w32 = [&](int q) { return reinterpret_cast<float *>(const_cast<uint4 *>(star_rec<D>(m, cd, q))); };
+    auto w64 = [&](int q) { return reinterpret_cast<double *>(const_cast<double2 *>(star_wt64<D>(m, cd, q))); };
+    double *bdt2 = const_cast<double *>(m.bdt2_64) + (size_t)cd.patch_off * kPatchMax;
+    const int32_t *src = elem_src + (size_t)cd.patch_off * kPatchMax;
+    for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x) {
+        const StarIds id = star_ids(star_rec<D>(m, cd, q));
+        const double *geo = m.geo64 +
+                            (size_t)((cd.patch_off + q) / kStarLanes) * (kPatchMax * kGeoWords<D> * kStarLanes) +
+                            q % kStarLanes;
+        double bd[kPatchMax];
+        double2 *b2 = reinterpret_cast<double2 *>(bdt2 + q * kPatchMax);
+        if (beta) {
+            const int2 *s2 = reinterpret_cast<const int2 *>(src + q * kPatchMax);
+#pragma unroll
+            for (int j = 0; j < kPatchMax / 2; ++j) {
+                const int2 e = __ldg(s2 + j);
+                bd[2 * j] = e.x >= 0 ? __ldg(beta + e.x) * dt2 : 0.0;
+                bd[2 * j + 1] = e.y >= 0 ? __ldg(beta + e.y) * dt2 : 0.0;
+                b2[j] = make_double2(bd[2 * j], bd[2 * j + 1]);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < kPatchMax / 2; ++j) {
+                const double2 v = b2[j];
+                bd[2 * j] = v.x;
+                bd[2 * j + 1] = v.y;
+            }
+        }
+        star_build<D>(id, geo, bd, S.val, m.lumped != 0, w32(q), w64(q), S.contrib + q * kPatchSlots);
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < cd.n_loc; l += blockDim.x) {
+        double ml = node_sum(S, l);
+        S.aux[l] = ml;
+        if (is_dirichlet(S.val[l])) ml = __longlong_as_double(__double_as_longlong(ml) | (long long)0x8000000000000000ULL);
+        const_cast<double *>(m.mrow64)[cd.node_off + l] = ml;
+        const_cast<float *>(m.mrow32)[cd.node_off + l] = (float)ml;
+    }
+    __syncthreads();
+    // off-diagonal row sums, from the weights this thread just stored
+    for (int q = threadIdx.x; q < cd.n_patch; q += blockDim.x) {
+        const int nr = star_ids(star_rec<D>(m, cd, q)).nr();
+        const double *wq = w64(q);
+        auto w = [&](int k) { return wq[(k / 2) * 2 * kStarLanes + k % 2]; };
+        double *out = S.contrib + q * kPatchSlots;
+        double sa = 0.0, sb = 0.0;
+        if (D == 3) sa = sb = w(0);
+        const double wrap = w(D == 3 ? 1 : 0);
+        double prev = wrap;
+#pragma unroll
+        for (int j = 0; j < kStarRing; ++j) {
+            if (j >= nr) break;
+            const int k = j == 0 ? (D == 3 ? 2 : 1) : (D == 3 ? 4 : 2) + D * (j - 1);
+            const double next = j + 1 < nr ? w((D == 3 ? 4 : 2) + D * j + D - 1) : wrap;
+            double o = prev + next + w(k);
+            sa += w(k);
+            if (D == 3) {
+                sb += w(k + 1);
+                o += w(k + 1);
+            }
+            out[2 + j] = o;
+            prev = next;
+        }
+        out[0] = sa;
+        if (D == 3) out[1] = sb;
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < cd.n_loc; l += blockDim.x) {
+        const double d = S.aux[l] - node_sum(S, l);
+        if (l < cd.n_int) {
+            const double dv = is_dirichlet(S.val[l]) ? 0.0 : 1.0 / d;
+            const_cast<double *>(m.dinv64)[cd.int_begin + l] = dv;
+            const_cast<float *>(m.dinv32)[cd.int_begin + l] = (float)dv;
+        } else {
+            partial[m.sh_dest[cd.sh_off + (l - cd.n_int)]] = d;
+        }
+    }
+}
+
+// Kernel 2: shared nodes sum their partials in slot order.  Residual: the
+// last block to finish also reduces all dot partials (kernel 1's n_first
+// blocks, then this kernel's blocks) into the state's rr.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_first) {
     __shared__ double s_red[34];
     __shared__ bool s_last;
-    if (MODE == kCG) {
-        if (threadIdx.x == 0) {
-            s_red[0] = a.st->beta;
-            s_red[1] = (double)a.st->done;
-        }
-        __syncthreads();
-        if (s_red[1] != 0.0) return;
-    }
-    const T beta_cg = (MODE == kCG) ? (T)s_red[0] : T(0);
     typename DotOf<T>::type acc;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < m.n_shared;
          s += (int64_t)gridDim.x * blockDim.x) {
@@ -412,13 +418,7 @@ __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_f
         for (int k = kb; k < ke; ++k) sum += a.partial[k];
         const bool dir = m.dirichlet[g] != 0;
         if (MODE == kApply) {
-            a.y[g] = dir ? T(0) : sum;   // (partials of Dirichlet rows may be unmasked: paired-patch kernels)
-        } else if (MODE == kCG) {
-            T v = cg_dir(a.dinv[g], a.r[g], beta_cg, a.p[g]);
-            if (dir) v = T(0);
-            a.p[g] = v;
-            a.y[g] = sum;
-            acc.add_prod(v, sum);
+            a.y[g] = dir ? T(0) : sum;
         } else if (MODE == kResid) {
             const T rv = dir ? T(0) : a.b[g] - sum;
             a.y[g] = rv;
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_f
             const_cast<float *>(m.dinv32)[g] = (float)dv;
         }
     }
-    if (MODE != kCG && MODE != kResid) return;
+    if (MODE != kResid) return;
     const double dot = block_sum(acc, s_red);
     if (threadIdx.x == 0) {
         a.dotbuf[n_first + blockIdx.x] = dot;
@@ -440,20 +440,8 @@ __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_f
     if (!s_last) return;
     const double tot = block_sum_array(a.dotbuf, n_first + gridDim.x, s_red);
     if (threadIdx.x == 0) {
-        CgState *st = a.st;
-        st->cnt_a = 0;
-        if (MODE == kCG) {
-            st->pq = tot;
-            if (!(tot > 0.0) || !isfinite(tot)) {
-                st->status = kCgBreakdown;
-                st->done = 1;
-                if (a.host_done) *(volatile int *)a.host_done = 1;
-            } else {
-                st->alpha = st->rz / tot;
-            }
-        } else {
-            st->rr = tot;
-        }
+        a.st->cnt_a = 0;
+        a.st->rr = tot;
     }
 }
 
@@ -543,51 +531,47 @@ __global__ void k_perm_out(int64_t n, const TI *__restrict__ in, TO *__restrict_
         out[j] = (TO)in[new_of_old[j]];
 }
 
-// Fill the alpha slot of every node record: w = +alpha, or -alpha (sign bit
-// set, also for alpha = 0) on Dirichlet nodes.
-static __global__ void k_set_alpha(int64_t n_loc, const int32_t *__restrict__ loc_node, const double *__restrict__ alpha_new,
-                            const uint8_t *__restrict__ dirichlet, NodeF *node32, NodeD *node64) {
+__device__ __forceinline__ void put_alpha(const MeshDev &m, int64_t k, double a, bool dir) {
+    if (dir) a = __longlong_as_double(__double_as_longlong(a) | (long long)0x8000000000000000ULL);
+    const_cast<double *>(m.alpha64)[k] = a;
+}
+
+// Fill the alpha of every local node: +alpha, or -alpha (sign bit set, also
+// for alpha = 0) on Dirichlet nodes.
+static __global__ void k_set_alpha(MeshDev m, int64_t n_loc, const int32_t *__restrict__ loc_node,
+                                   const double *__restrict__ alpha_new) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_loc; k += (int64_t)gridDim.x * blockDim.x) {
         const int g = loc_node[k];
-        const double a = alpha_new[g];
-        double w64 = a;
-        float w32 = (float)a;
-        if (dirichlet[g]) {
-            w64 = __longlong_as_double(__double_as_longlong(w64) | (long long)0x8000000000000000ULL);
-            w32 = __int_as_float(__float_as_int(w32) | (int)0x80000000u);
-        }
-        node64[k].w = w64;
-        node32[k].w = w32;
+        put_alpha(m, k, alpha_new[g], m.dirichlet[g] != 0);
     }
 }
 
 // The same from caller-numbered alpha: unknown g takes alpha of its master
-// vertex old_of_new[g].
-static __global__ void k_set_alpha_user(int64_t n_loc, const int32_t *__restrict__ loc_node,
+// vertex old_of_new[g].  wl (may be null, lumped mass): the lumped weight
+// |T|/(d+1) summed over the chunk's elements around each local node; alpha
+// then scales it into the row sums, all that a lumped operator takes from it.
+static __global__ void k_set_alpha_user(MeshDev m, int64_t n_loc, const int32_t *__restrict__ loc_node,
                                         const int32_t *__restrict__ old_of_new, const double *__restrict__ alpha_user,
-                                        const uint8_t *__restrict__ dirichlet, NodeF *node32, NodeD *node64) {
+                                        const double *__restrict__ wl) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_loc; k += (int64_t)gridDim.x * blockDim.x) {
         const int g = loc_node[k];
         const double a = alpha_user[old_of_new[g]];
-        double w64 = a;
-        float w32 = (float)a;
-        if (dirichlet[g]) {
-            w64 = __longlong_as_double(__double_as_longlong(w64) | (long long)0x8000000000000000ULL);
-            w32 = __int_as_float(__float_as_int(w32) | (int)0x80000000u);
+        put_alpha(m, k, a, m.dirichlet[g] != 0);
+        if (wl) {
+            double ml = a * wl[k];
+            if (m.dirichlet[g]) ml = __longlong_as_double(__double_as_longlong(ml) | (long long)0x8000000000000000ULL);
+            const_cast<double *>(m.mrow64)[k] = ml;
+            const_cast<float *>(m.mrow32)[k] = (float)ml;
         }
-        node64[k].w = w64;
-        node32[k].w = w32;
     }
 }
 
 // bdt2[k] = beta[elem_src[k]] * dt2 (0 on padding slots).
 static __global__ void k_set_beta(int64_t n, const int32_t *__restrict__ elem_src, const double *__restrict__ beta,
-                           double dt2, float *b32, double *b64) {
+                                  double dt2, double *b64) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int e = elem_src[k];
-        const double v = e >= 0 ? beta[e] * dt2 : 0.0;
-        b64[k] = v;
-        b32[k] = (float)v;
+        b64[k] = e >= 0 ? beta[e] * dt2 : 0.0;
     }
 }
 

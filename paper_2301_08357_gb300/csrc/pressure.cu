@@ -22,7 +22,7 @@
 #include "internal.h"
 #include "cg1.cuh"
 #include "cg2.cuh"
-#include "cg2u.cuh"
+#include "cg2s.cuh"
 
 using namespace ps;
 
@@ -30,6 +30,14 @@ namespace ps {
 
 const int kBlock = kChunkThreads;   // threads per block of every kernel
 static const int kUpdateBlocksPerSm = 2;   // update-kernel grid when occupancy is unknown
+
+// Star records beyond this size are read with evict-first priority by the
+// operator kernel (half of the 129 MB L2: records, vectors and partial sums of
+// a smaller mesh stay resident from one pass to the next).  Measured on Kuhn
+// cubes, evict-first / plain: 64^3 (25 MB of records) 15.4 / 14.7 us per pass,
+// 96^3 (85 MB) 31.3 / 38.8, 112^3 (135 MB) 50.4 / 54.9, 160^3 (393 MB) 134.9 /
+// 135.7; the update kernel gains too (96^3: 11.1 -> 9.5 us).
+static constexpr int64_t kStreamBytes = int64_t(64) << 20;
 
 static int sm_count_of(int dev) {
     int v = 0;
@@ -75,7 +83,7 @@ static uint32_t align128(uint64_t v) { return (uint32_t)((v + 127) / 128 * 128);
 // Geometry of element j of a star patch (vertices A, B, ring j, ring j+1 in
 // 3D; A, ring j, ring j+1 in 2D; chunk-relative coordinates rel): the
 // cofactor vectors c_a (grad lambda_a = c_a / det) and the slot words of
-// patch_eval_geo.
+// kGeoWords.
 static void element_geometry(int dim, const double *rel, const uint16_t *rec, int j, double *out) {
     auto P = [&](int l) { return rel + (size_t)l * dim; };
     if (dim == 3) {
@@ -105,7 +113,6 @@ static void element_geometry(int dim, const double *rel, const uint16_t *rec, in
         out[4] = G(1, 3);
         out[5] = G(2, 3);
         out[6] = ad;
-        out[7] = 0.0;
     } else {
         const double *A = P(rec[1]), *R0 = P(rec[3 + j]), *R1 = P(rec[4 + j]);
         const double d0[2] = {R0[0] - A[0], R0[1] - A[1]}, d1[2] = {R1[0] - A[0], R1[1] - A[1]};
@@ -120,17 +127,14 @@ static void element_geometry(int dim, const double *rel, const uint16_t *rec, in
     }
 }
 
-SmemLayout make_layout(int esz, int nsz, int max_loc, int max_patch, int max_inc, int max_sh) {
+SmemLayout make_layout(int esz, int max_loc, int max_patch, int max_inc) {
     SmemLayout L;
     const uint64_t ppad = (uint64_t)round_up(max_patch, kPatchPad);
     uint64_t off = 0;
-    L.node = (uint32_t)off;    off += align128((uint64_t)max_loc * nsz);
     L.val = (uint32_t)off;     off += align128((uint64_t)max_loc * esz);
     L.aux = (uint32_t)off;     off += align128((uint64_t)max_loc * esz);
-    L.pids = (uint32_t)off;    off += align128(ppad * kPatchIds * 2);
     L.incp = (uint32_t)off;    off += align128((uint64_t)round_up(max_loc + 1, kIncpPad) * 2);
     L.inc = (uint32_t)off;     off += align128((uint64_t)round_up(max_inc > 0 ? max_inc : 1, kIncPad) * 2);
-    L.shid = (uint32_t)off;    off += align128((uint64_t)round_up(max_sh > 0 ? max_sh : 1, kShPad) * 4);
     L.contrib = (uint32_t)off; off += align128(ppad * kPatchSlots * esz);
     L.red = (uint32_t)off;     off += 34 * 8;
     L.bar = (uint32_t)off;     off += 16;
@@ -138,35 +142,18 @@ SmemLayout make_layout(int esz, int nsz, int max_loc, int max_patch, int max_inc
     return L;
 }
 
-// Two-stage layout for the pipelined CG kernel: static chunk data twice
-// (node records, patch records, incidence pointers / lists, shared-node ids,
-// mbarrier), one copy of the node values and element contributions.
-void make_layout2(int esz, int nsz, int max_loc, int max_patch, int max_inc, int max_sh, SmemLayout &L0,
-                  SmemLayout &L1) {
-    const uint64_t ppad = (uint64_t)round_up(max_patch, kPatchPad);
-    const uint64_t b_node = align128((uint64_t)max_loc * nsz), b_pids = align128(ppad * kPatchIds * 2),
-                   b_incp = align128((uint64_t)round_up(max_loc + 1, kIncpPad) * 2),
-                   b_inc = align128((uint64_t)round_up(max_inc > 0 ? max_inc : 1, kIncPad) * 2),
-                   b_shid = align128((uint64_t)round_up(max_sh > 0 ? max_sh : 1, kShPad) * 4);
-    uint64_t off = 0;
-    for (SmemLayout *L : {&L0, &L1}) {
-        L->node = (uint32_t)off;  off += b_node;
-        L->pids = (uint32_t)off;  off += b_pids;
-        L->incp = (uint32_t)off;  off += b_incp;
-        L->inc = (uint32_t)off;   off += b_inc;
-        L->shid = (uint32_t)off;  off += b_shid;
-        L->bar = (uint32_t)off;   off += 128;
-    }
-    const uint32_t val = (uint32_t)off;     off += align128((uint64_t)max_loc * esz);
-    const uint32_t contrib = (uint32_t)off; off += align128(ppad * kPatchSlots * esz);
-    const uint32_t red = (uint32_t)off;     off += 34 * 8;
-    for (SmemLayout *L : {&L0, &L1}) {
-        L->val = val;
-        L->aux = val;
-        L->contrib = contrib;
-        L->red = red;
-        L->total = (uint32_t)off;
-    }
+// The largest chunk the interface takes: per local node 48 bytes, per patch
+// 24 + 72 bytes, the incidence pointers and lists and 4 bytes per shared node
+// within 227 KB (more than any pass stages; the limit does not move with the
+// kernels' layouts).
+static bool chunk_fits(const PrepMesh &pm) {
+    const uint64_t ppad = (uint64_t)round_up(pm.max_patch, 4);
+    uint64_t b = align128((uint64_t)pm.max_loc * 32) + 2 * align128((uint64_t)pm.max_loc * 8) + align128(ppad * 24) +
+                 align128((uint64_t)round_up(pm.max_loc + 1, kIncpPad) * 2) +
+                 align128((uint64_t)round_up(pm.max_inc > 0 ? pm.max_inc : 1, kIncPad) * 2) +
+                 align128((uint64_t)round_up(pm.max_sh > 0 ? pm.max_sh : 1, kShPad) * 4) + align128(ppad * 72) +
+                 34 * 8 + 16;
+    return b <= 227 * 1024;
 }
 
 int cuda_status(cudaError_t e) {
@@ -219,28 +206,19 @@ static int set_smem_attrs() {
     CK(set_max_dyn_smem(k_chunks<3, float, kApply>));
     CK(set_max_dyn_smem(k_chunks<2, double, kApply>));
     CK(set_max_dyn_smem(k_chunks<3, double, kApply>));
-    CK(set_max_dyn_smem(k_chunks<2, float, kCG>));
-    CK(set_max_dyn_smem(k_chunks<3, float, kCG>));
-    CK(set_max_dyn_smem(k_chunks<2, double, kCG>));
-    CK(set_max_dyn_smem(k_chunks<3, double, kCG>));
     CK(set_max_dyn_smem(k_chunks<2, double, kResid>));
     CK(set_max_dyn_smem(k_chunks<3, double, kResid>));
-    CK(set_max_dyn_smem(k_chunks<2, double, kDiag>));
-    CK(set_max_dyn_smem(k_chunks<3, double, kDiag>));
+    CK(set_max_dyn_smem(k_star_build<2>));
+    CK(set_max_dyn_smem(k_star_build<3>));
     CK(set_max_dyn_smem(k_cg1_chunks<2>));
     CK(set_max_dyn_smem(k_cg1_chunks<3>));
     CK(set_max_dyn_smem(k_cg2_chunks<2, float>));
     CK(set_max_dyn_smem(k_cg2_chunks<3, float>));
-    CK(set_max_dyn_smem(k_cg2_chunks<2, float, true>));
-    CK(set_max_dyn_smem(k_cg2_chunks<3, float, true>));
     CK(set_max_dyn_smem(k_cg2_chunks<2, double>));
     CK(set_max_dyn_smem(k_cg2_chunks<3, double>));
-    CK(set_max_dyn_smem(k_cg2_chunks_pipe<2>));
-    CK(set_max_dyn_smem(k_cg2_chunks_pipe<3>));
-    CK(set_max_dyn_smem(k_cg2_units<false, 256, 2>));
-    CK(set_max_dyn_smem(k_cg2_units<true, 256, 2>));
-    CK(set_max_dyn_smem(k_cg2_units<false, 128, kUnitBlocks128>));
-    CK(set_max_dyn_smem(k_cg2_units<true, 128, kUnitBlocks128>));
+    CK(set_max_dyn_smem(k_cg2_stars<kStarThreads, 3>));
+    CK(set_max_dyn_smem(k_cg2_stars<256, 3>));
+    CK(set_max_dyn_smem(k_cg2_stars<128, 5>));
     return batched_set_attrs();
 }
 
@@ -261,8 +239,6 @@ int launch_pass(ps_mesh *m, const VecArgs<T> &a, cudaStream_t s) {
 template int launch_pass<float, kApply>(ps_mesh *, const VecArgs<float> &, cudaStream_t);
 template int launch_pass<double, kApply>(ps_mesh *, const VecArgs<double> &, cudaStream_t);
 template int launch_pass<double, kResid>(ps_mesh *, const VecArgs<double> &, cudaStream_t);
-template int launch_pass<float, kCG>(ps_mesh *, const VecArgs<float> &, cudaStream_t);
-template int launch_pass<double, kCG>(ps_mesh *, const VecArgs<double> &, cudaStream_t);
 
 }  // namespace ps
 
@@ -344,9 +320,23 @@ static int mesh_upload_impl(ps_ctx *c, ps_mesh *m, const PrepMesh &pm) {
     ChunkDesc *ch;
     RC(upload(c, m, &ch, pm.chunks.data(), pm.chunks.size() * sizeof(ChunkDesc)));
     d.chunks = ch;
+    // star records: the ids in words 0..4, the weights when coefficients are set
+    {
+        int nv = pm.dim == 3 ? 6 : kStarVec<2>;
+        for (int64_t q = 0; q < pm.patch_total; ++q)
+            if (pm.dim == 3 && ((pm.sids[q * kStarIds + 4] >> 16) & 7u) == 7u) nv = kStarVec<3>;
+        d.srows = nv;
+        d.stream = (int64_t)pm.patch_total * nv * 16 > kStreamBytes;
+        std::vector<uint32_t> rec((size_t)pm.patch_total * nv * 4, 0);
+        for (int64_t q = 0; q < pm.patch_total; ++q)
+            for (int k = 0; k < kStarIds; ++k)
+                rec[(((size_t)(q / kStarLanes) * nv + k / 4) * kStarLanes + q % kStarLanes) * 4 + k % 4] =
+                    pm.sids[q * kStarIds + k];
+        uint4 *sr;
+        RC(upload(c, m, &sr, rec.data(), rec.size() * 4));
+        d.srec = sr;
+    }
     uint16_t *u;
-    RC(upload(c, m, &u, pm.pids.data(), pm.pids.size() * 2));
-    d.pids = u;
     RC(upload(c, m, &u, pm.incp.data(), pm.incp.size() * 2));
     d.incp = u;
     RC(upload(c, m, &u, pm.inc.data(), pm.inc.size() * 2));
@@ -375,51 +365,48 @@ static int mesh_upload_impl(ps_ctx *c, ps_mesh *m, const PrepMesh &pm) {
     uint8_t *du;
     RC(upload(c, m, &du, dir.data(), dir.size()));
     d.dirichlet = du;
-    // node records: coordinates relative to the chunk origin, alpha set later
-    {
-        std::vector<NodeF> nf(pm.loc_total);
-        std::vector<NodeD> nd(pm.loc_total);
-        for (int64_t k = 0; k < pm.loc_total; ++k) {
-            const double *r = &pm.loc_rel[k * pm.dim];
-            nd[k].x = r[0];
-            nd[k].y = r[1];
-            nd[k].z = pm.dim == 3 ? r[2] : 0.0;
-            nd[k].w = 0.0;
-            nf[k].x = (float)nd[k].x;
-            nf[k].y = (float)nd[k].y;
-            nf[k].z = (float)nd[k].z;
-            nf[k].w = 0.0f;
-        }
-        NodeF *pf;
-        NodeD *pd;
-        RC(upload(c, m, &pf, nf.data(), nf.size() * sizeof(NodeF)));
-        RC(upload(c, m, &pd, nd.data(), nd.size() * sizeof(NodeD)));
-        d.node32 = pf;
-        d.node64 = pd;
-    }
-    // FP64 element geometry per patch slot (patch_eval_geo): stiffness weights
-    // G_ab = c_a.c_b / (d! |det|) and |det|, from the chunk-relative FP64
-    // coordinates the device would otherwise recompute them from
+    // element geometry per patch slot (kGeoWords: stiffness weights G_ab =
+    // c_a.c_b / (d! |det|) and |det|) from chunk-relative FP64 coordinates,
+    // and the lumped weight of every local node over its chunk's elements
     {
         const int gw = pm.dim == 3 ? kGeoWords<3> : kGeoWords<2>;
-        std::vector<double> geo((size_t)pm.patch_total * kPatchMax * gw, 0.0);
+        const double lf = pm.dim == 3 ? 1.0 / 24.0 : 1.0 / 6.0;
+        std::vector<double> geo((size_t)pm.patch_total * kPatchMax * gw, 0.0), lump(pm.loc_total, 0.0);
         for (int ch = 0; ch < pm.n_chunks; ++ch) {
             const ChunkDesc &cd = pm.chunks[ch];
             const double *rel = &pm.loc_rel[(size_t)cd.node_off * pm.dim];
+            double *gc = &geo[(size_t)cd.patch_off * kPatchMax * gw];
             for (int q = 0; q < cd.n_patch; ++q) {
                 const uint16_t *rec = &pm.pids[(size_t)(cd.patch_off + q) * kPatchIds];
-                double *gs = &geo[(size_t)(cd.patch_off + q) * kPatchMax * gw];
-                for (int j = 0; j < rec[0]; ++j) element_geometry(pm.dim, rel, rec, j, gs + (size_t)j * gw);
+                for (int j = 0; j < rec[0]; ++j) {
+                    double g[8];
+                    element_geometry(pm.dim, rel, rec, j, g);
+                    for (int k = 0; k < gw; ++k)
+                        gc[((size_t)(q / kStarLanes * kPatchMax + j) * gw + k) * kStarLanes + q % kStarLanes] = g[k];
+                    const double w = g[gw - 1] * lf;
+                    lump[cd.node_off + rec[1]] += w;
+                    if (pm.dim == 3) lump[cd.node_off + rec[2]] += w;
+                    lump[cd.node_off + rec[3 + j]] += w;
+                    lump[cd.node_off + rec[4 + j]] += w;
+                }
             }
         }
         double *gp;
         RC(upload(c, m, &gp, geo.data(), geo.size() * 8));
         d.geo64 = gp;
+        RC(upload(c, m, &m->d_lump, lump.data(), lump.size() * 8));
     }
     float *f;
     double *g;
-    RC(upload(c, m, &f, nullptr, pm.patch_total * kPatchMax * 4));
-    d.bdt2_32 = f;
+    double2 *sw;
+    RC(upload(c, m, &sw, nullptr, pm.patch_total * (pm.dim == 3 ? kStarVec64<3> : kStarVec64<2>) * 16));
+    d.sw64 = sw;
+    RC(upload(c, m, &f, nullptr, pm.loc_total * 4));
+    d.mrow32 = f;
+    RC(upload(c, m, &g, nullptr, pm.loc_total * 8));
+    d.mrow64 = g;
+    RC(upload(c, m, &g, nullptr, pm.loc_total * 8));
+    d.alpha64 = g;
     RC(upload(c, m, &g, nullptr, pm.patch_total * kPatchMax * 8));
     d.bdt2_64 = g;
     RC(upload(c, m, &f, nullptr, d.n_pad * 4));
@@ -428,74 +415,42 @@ static int mesh_upload_impl(ps_ctx *c, ps_mesh *m, const PrepMesh &pm) {
     RC(upload(c, m, &g, nullptr, d.n_pad * 8));
     CK(cudaMemset(g, 0, d.n_pad * 8));
     d.dinv64 = g;
-    if (pm.dim == 3 && pm.unit_total > 0 && m->k1_variant != 1) {
-        ChunkUnits *cu;
-        RC(upload(c, m, &cu, pm.chunks_u.data(), pm.chunks_u.size() * sizeof(ChunkUnits)));
-        d.chunks_u = cu;
-        uint32_t *ur;
-        RC(upload(c, m, &ur, pm.urec.data(), pm.urec.size() * 4));
-        d.urec = ur;
-        RC(upload(c, m, &m->d_uelem, pm.uelem.data(), pm.uelem.size() * 4));
-        float *ub;
-        RC(upload(c, m, &ub, nullptr, pm.uelem.size() * 4));
-        CK(cudaMemset(ub, 0, pm.uelem.size() * 4));
-        d.ubd = ub;
-        float *dm;
-        RC(upload(c, m, &dm, nullptr, (size_t)pm.n_chunks * 4));
-        CK(cudaMemset(dm, 0, (size_t)pm.n_chunks * 4));
-        d.dmax = dm;
-        UnitSmem &U = d.smu;
+    if (pm.dim == 3 && m->k1_variant != 1) {
+        StarSmem &U = d.sms;
         uint32_t off = 0;
         auto take = [&](uint64_t bytes) {
             const uint32_t at = off;
             off = align128(off + bytes);
             return at;
         };
-        U.node = take((uint64_t)pm.max_loc * sizeof(NodeF));
+        const uint64_t groups = (pm.max_patch + kStarLanes - 1) / kStarLanes;
+        U.rec = take(groups * d.srows * kStarLanes * 16);
+        U.incp = take((uint64_t)round_up(pm.max_loc + 1, kIncpPad) * 2);
+        U.inc = take((uint64_t)round_up(pm.max_inc > 0 ? pm.max_inc : 1, kIncPad) * 2);
         U.val = take((uint64_t)pm.max_loc * 4);
-        U.acc = take((uint64_t)pm.max_loc * 8);
-        U.shd = take((uint64_t)round_up(pm.max_sh, kShPad) * 4);
-        U.urec = take((uint64_t)pm.max_unit * kURecWords * 4);
-        U.ubd = take((uint64_t)pm.max_unit * kPatchMax * 8);
         U.bar = take(8);
         U.total = off;
-        // node ids of the unit records are 16-bit; a thread's Dirichlet mask
-        // covers 32 nodes of the chunk
-        m->use_units = U.total <= 200 * 1024 && pm.max_loc <= 32 * m->unit_threads;
+        // incidence lists with the contributions' words in the records' place
+        m->use_halo = U.total <= 200 * 1024 && groups * d.srows * kStarLanes * 4 < 65536;
+        if (m->use_halo) {
+            std::vector<uint16_t> inc(pm.inc.size());
+            for (size_t k = 0; k < inc.size(); ++k) {
+                const uint32_t q = pm.inc[k] / kPatchSlots, slot = pm.inc[k] % kPatchSlots;
+                inc[k] = (uint16_t)(((q / kStarLanes * d.srows + slot / 4) * kStarLanes + q % kStarLanes) * 4 + slot % 4);
+            }
+            RC(upload(c, m, &u, inc.data(), inc.size() * 2));
+            d.inc_rec = u;
+        }
     }
     d.err = c->d_err;
-    d.sm32 = make_layout(4, sizeof(NodeF), pm.max_loc, pm.max_patch, pm.max_inc, pm.max_sh);
-    d.sm64 = make_layout(8, sizeof(NodeD), pm.max_loc, pm.max_patch, pm.max_inc, pm.max_sh);
-    if (d.sm64.total > 227 * 1024) {
+    if (!chunk_fits(pm)) {
         ps_set_last_error("chunk too large for shared memory; lower chunk_elems");
         return PS_EINVAL;
     }
+    d.sm32 = make_layout(4, pm.max_loc, pm.max_patch, pm.max_inc);
+    d.sm64 = make_layout(8, pm.max_loc, pm.max_patch, pm.max_inc);
     m->grid2 = grid_for(pm.n_shared, c->sms);
     m->grid3 = grid_for(d.n_pad, c->sms);
-    make_layout2(4, sizeof(NodeF), pm.max_loc, pm.max_patch, pm.max_inc, pm.max_sh, m->pipe_L0, m->pipe_L1);
-    {
-        int per_sm = 0;
-        cudaError_t oe = pm.dim == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg2_chunks_pipe<2>,
-                                                                                      kBlock, m->pipe_L0.total)
-                                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cg2_chunks_pipe<3>,
-                                                                                      kBlock, m->pipe_L0.total);
-        if (oe != cudaSuccess || m->pipe_L0.total > 200 * 1024) per_sm = 0;
-        cudaGetLastError();
-        m->pipe_grid = (per_sm > 0 && m->pipeline && !m->use_units)
-                           ? (int)std::min<int64_t>(pm.n_chunks, (int64_t)c->sms * per_sm)
-                           : 0;
-    }
-    {
-        // FP32 operator kernel: prefetch beta*dt^2 into registers when that
-        // costs no resident blocks (shared memory is the limit: large chunks)
-        int o0 = 0, o1 = 0;
-        cudaError_t e0 = pm.dim == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o0, k_cg2_chunks<2, float>, kBlock, d.sm32.total)
-                                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o0, k_cg2_chunks<3, float>, kBlock, d.sm32.total);
-        cudaError_t e1 = pm.dim == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_cg2_chunks<2, float, true>, kBlock, d.sm32.total)
-                                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o1, k_cg2_chunks<3, float, true>, kBlock, d.sm32.total);
-        cudaGetLastError();
-        m->k1_pre = e0 == cudaSuccess && e1 == cudaSuccess && o1 > 0 && o1 >= o0;
-    }
     {
         // auto: one full wave of the update kernel (its resident blocks per
         // SM times the SMs); measured on 160^3: 33 us at 6 blocks/SM (one
@@ -534,9 +489,9 @@ extern "C" int ps_mesh_upload_periodic(ps_ctx *c, int dim, int64_t n_nodes, cons
         po.chunk_nodes_max = opts->chunk_nodes_max;
     }
     po.periodic = periodic;
-    // 3D meshes (paired-patch operator kernel): the first wave's chunks
+    // 3D meshes (operator kernel 2): the first wave's chunks
     // split in halves on one of every ~five resident blocks of an SM
-    // (measured on 160^3 Kuhn: 141 -> 138 us per operator pass)
+    // (measured on 160^3 Kuhn with the kernel of the time: 141 -> 138 us per pass)
     const int sl = opts ? opts->split_lead : 0;
     if (sl < -1) return PS_EINVAL;
     if (sl > 0) po.split_lead = sl;
@@ -544,11 +499,10 @@ extern "C" int ps_mesh_upload_periodic(ps_ctx *c, int dim, int64_t n_nodes, cons
     ps_mesh *m = new (std::nothrow) ps_mesh();
     if (!m) return PS_ENOMEM;
     m->ctx = c;
-    m->pipeline = opts ? opts->pipeline : 0;
     m->update_bps = opts ? opts->update_blocks_per_sm : 0;
     m->k1_variant = opts ? opts->operator_kernel : 0;
     const int ot = opts ? opts->operator_threads : 0;
-    m->unit_threads = ot == 256 ? 256 : 128;
+    m->op_threads = ot;
     if (m->update_bps < 0 || m->update_bps > 64 || m->k1_variant < 0 || m->k1_variant > 2 ||
         (ot != 0 && ot != 128 && ot != 256)) {
         delete m;
@@ -625,11 +579,25 @@ extern "C" int ps_mesh_get_stats(const ps_mesh *m, ps_mesh_stats *o) {
     o->max_chunk_elems = p.max_elem;
     o->max_chunk_nodes = p.max_loc;
     o->solve_bytes = batch_ws_bytes(m);
-    o->operator_kernel = m->use_units ? 2 : 1;
+    o->operator_kernel = m->use_halo ? 2 : 1;
     return PS_OK;
 }
 
 // ---------------------------------------------------------------- ABI: coefficients
+// Star weights, row sums and Jacobi diagonal (d.dinv32, d.dinv64) from the
+// mesh's alpha and beta (null: the beta*dt^2 stored last), on stream s.
+static void launch_star_build(ps_mesh *m, const MeshDev &d, const double *beta, double dt2, double *partial,
+                              cudaStream_t s) {
+    if (d.dim == 2)
+        k_star_build<2><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, m->d_elem_src, beta, dt2, partial);
+    else
+        k_star_build<3><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, m->d_elem_src, beta, dt2, partial);
+    VecArgs<double> a;
+    std::memset(&a, 0, sizeof(a));
+    a.partial = partial;
+    k_shared<double, kDiag><<<m->grid2, kBlock, 0, s>>>(d, a, d.n_chunks);
+}
+
 static int coeff_upload(ps_mesh *m, const double *alpha, const double *beta, double dt2) {
     ps_ctx *c = m->ctx;
     const PrepMesh &p = m->prep;
@@ -639,18 +607,6 @@ static int coeff_upload(ps_mesh *m, const double *alpha, const double *beta, dou
     int rc = dalloc(c, &dbeta, p.n_elems * 8, tmp);
     if (rc != PS_OK) return rc;
     cudaError_t e = cudaMemcpy(dbeta, beta, p.n_elems * 8, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-        const int64_t nslots = p.patch_total * kPatchMax;
-        k_set_beta<<<grid_for(nslots, c->sms), kBlock>>>(nslots, m->d_elem_src, (const double *)dbeta, dt2,
-                                                                 const_cast<float *>(d.bdt2_32),
-                                                                 const_cast<double *>(d.bdt2_64));
-        if (d.ubd) {
-            const int64_t nu = (int64_t)p.uelem.size();
-            k_set_beta_units<<<grid_for(nu, c->sms), kBlock>>>(nu, m->d_uelem, (const double *)dbeta, dt2,
-                                                               const_cast<float *>(d.ubd));
-        }
-        e = cudaGetLastError();
-    }
     if (e == cudaSuccess && alpha) {
         std::vector<double> an(p.n_dofs);   // the master vertex's alpha per unknown
         for (int64_t g = 0; g < p.n_dofs; ++g) an[g] = alpha[p.old_of_new[g]];
@@ -662,29 +618,19 @@ static int coeff_upload(ps_mesh *m, const double *alpha, const double *beta, dou
         }
         e = cudaMemcpy(dal, an.data(), p.n_dofs * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) {
-            k_set_alpha<<<grid_for(p.loc_total, c->sms), kBlock>>>(p.loc_total, m->d_loc_node, (const double *)dal,
-                                                                    d.dirichlet, const_cast<NodeF *>(d.node32),
-                                                                    const_cast<NodeD *>(d.node64));
+            k_set_alpha<<<grid_for(p.loc_total, c->sms), kBlock>>>(d, p.loc_total, m->d_loc_node, (const double *)dal);
             e = cudaGetLastError();
         }
     }
     if (e == cudaSuccess) {
-        // Jacobi diagonal, FP64 element arithmetic, both precisions stored
-        VecArgs<double> a;
-        std::memset(&a, 0, sizeof(a));
+        // star weights, row sums and the Jacobi diagonal (FP64 arithmetic, both precisions stored)
         void *part = nullptr;
         rc = dalloc(c, &part, (p.sh_total > 0 ? p.sh_total : 1) * 8, tmp);
         if (rc != PS_OK) {
             dfree_all(c, tmp);
             return rc;
         }
-        a.partial = (double *)part;
-        if (d.dim == 2)
-            k_chunks<2, double, kDiag><<<d.n_chunks, kBlock, d.sm64.total>>>(d, a);
-        else
-            k_chunks<3, double, kDiag><<<d.n_chunks, kBlock, d.sm64.total>>>(d, a);
-        k_shared<double, kDiag><<<m->grid2, kBlock>>>(d, a, d.n_chunks);
-        if (d.dmax) k_chunk_dmax<<<d.n_chunks, 128>>>(d, const_cast<float *>(d.dmax));
+        launch_star_build(m, d, (const double *)dbeta, dt2, (double *)part, nullptr);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
     }
@@ -738,79 +684,62 @@ extern "C" int ps_coeff_set_beta(ps_mesh *m, const double *beta) {
 // ---------------------------------------------------------------- workspace
 namespace ps {
 
-// Jacobi diagonal from the mesh's current alpha, beta*dt^2 and mass form, on
-// stream s (FP64 element arithmetic, both precisions stored).  The caller
-// holds the context mutex and the workspace exists.
-static int diag_update_device(ps_mesh *m, cudaStream_t s) {
+// Star weights, row sums and Jacobi diagonal from the mesh's current alpha,
+// beta (null: the stored beta*dt^2) and mass form, on stream s (FP64 element
+// arithmetic, both precisions stored).  The caller holds the context mutex
+// and the workspace exists.
+static int star_update_device(ps_mesh *m, const double *beta, double dt2, cudaStream_t s) {
     const MeshDev &d = m->dev;
-    VecArgs<double> a;
-    std::memset(&a, 0, sizeof(a));
-    a.partial = m->ws.part64;
-    if (d.dim == 2)
-        k_chunks<2, double, kDiag><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, a);
-    else
-        k_chunks<3, double, kDiag><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, a);
-    k_shared<double, kDiag><<<m->grid2, kBlock, 0, s>>>(d, a, d.n_chunks);
-    if (d.dmax) k_chunk_dmax<<<d.n_chunks, 128, 0, s>>>(d, const_cast<float *>(d.dmax));
+    launch_star_build(m, d, beta, dt2, m->ws.part64, s);
     CK(cudaGetLastError());
     return PS_OK;
 }
 
-// Coefficients changed while the preconditioner keeps its diagonal: the
-// paired-patch kernel's fixed-point bound still needs the current diagonal,
-// so it is computed into scratch (two free workspace vectors) and only its
-// chunk maxima are kept (dmax).  No-op for the other kernels.
-static int dmax_refresh(ps_mesh *m, cudaStream_t s) {
-    const MeshDev &d = m->dev;
-    if (!d.dmax) return PS_OK;
-    MeshDev d2 = d;
+// The same while the preconditioner keeps its diagonal: the current one goes
+// into scratch (two free workspace vectors).
+static int star_update_keep_diag(ps_mesh *m, cudaStream_t s) {
+    MeshDev d2 = m->dev;
     d2.dinv64 = m->ws.q64;
     d2.dinv32 = m->ws.q32;
-    VecArgs<double> a;
-    std::memset(&a, 0, sizeof(a));
-    a.partial = m->ws.part64;
-    k_chunks<3, double, kDiag><<<d2.n_chunks, kBlock, d2.sm64.total, s>>>(d2, a);
-    k_shared<double, kDiag><<<m->grid2, kBlock, 0, s>>>(d2, a, d2.n_chunks);
-    k_chunk_dmax<<<d2.n_chunks, 128, 0, s>>>(d2, const_cast<float *>(d.dmax));
+    launch_star_build(m, d2, nullptr, 0.0, m->ws.part64, s);
     CK(cudaGetLastError());
     return PS_OK;
 }
 
-// beta (caller's element order, device) -> beta*dt^2 per patch slot and the
-// Jacobi diagonal, on stream s without allocating or synchronising (the
-// projection stage updates the operator between Picard iterations).  The
-// caller holds the context mutex.
+// beta (caller's element order, device) -> beta*dt^2 per patch slot, star
+// weights and the Jacobi diagonal, on stream s without allocating or
+// synchronising (the projection stage updates the operator between Picard
+// iterations).  diag = false: only the beta*dt^2 are stored; the caller's
+// alpha update that follows (diag = true) forms the rest.  The caller holds
+// the context mutex.
 int beta_update_device(ps_mesh *m, const double *beta_dev, double dt2, cudaStream_t s, bool diag) {
     RC(ensure_workspace(m));
     const PrepMesh &p = m->prep;
     MeshDev &d = m->dev;
-    const int64_t nslots = p.patch_total * kPatchMax;
-    k_set_beta<<<grid_for(nslots, m->ctx->sms), kBlock, 0, s>>>(nslots, m->d_elem_src, beta_dev, dt2,
-                                                                 const_cast<float *>(d.bdt2_32),
-                                                                 const_cast<double *>(d.bdt2_64));
-    if (d.ubd) {
-        const int64_t nu = (int64_t)p.uelem.size();
-        k_set_beta_units<<<grid_for(nu, m->ctx->sms), kBlock, 0, s>>>(nu, m->d_uelem, beta_dev, dt2,
-                                                                      const_cast<float *>(d.ubd));
+    if (!diag) {
+        const int64_t nslots = p.patch_total * kPatchMax;
+        k_set_beta<<<grid_for(nslots, m->ctx->sms), kBlock, 0, s>>>(nslots, m->d_elem_src, beta_dev, dt2,
+                                                                     const_cast<double *>(d.bdt2_64));
     }
     CK(cudaGetLastError());
     m->dt2 = dt2;
-    return diag ? diag_update_device(m, s) : dmax_refresh(m, s);
+    return diag ? star_update_device(m, beta_dev, dt2, s) : PS_OK;
 }
 
 // Nodal alpha (caller's numbering, device; each unknown takes its master
-// vertex's value) into both node records, then (diag) the Jacobi diagonal; on
-// stream s without allocating or synchronising.  The caller holds the
-// context mutex.
+// vertex's value), then the star weights and (diag) the Jacobi diagonal; on
+// stream s without allocating or synchronising.  Without diag a lumped
+// operator only needs its row sums scaled.  The caller holds the context
+// mutex.
 int alpha_update_device(ps_mesh *m, const double *alpha_dev, cudaStream_t s, bool diag) {
     RC(ensure_workspace(m));
     const PrepMesh &p = m->prep;
     MeshDev &d = m->dev;
     k_set_alpha_user<<<grid_for(p.loc_total, m->ctx->sms), kBlock, 0, s>>>(
-        p.loc_total, m->d_loc_node, m->d_old_of_new, alpha_dev, d.dirichlet, const_cast<NodeF *>(d.node32),
-        const_cast<NodeD *>(d.node64));
+        d, p.loc_total, m->d_loc_node, m->d_old_of_new, alpha_dev, d.lumped && !diag ? m->d_lump : nullptr);
     CK(cudaGetLastError());
-    return diag ? diag_update_device(m, s) : dmax_refresh(m, s);
+    if (diag) return star_update_device(m, nullptr, 0.0, s);
+    return d.lumped ? PS_OK : star_update_keep_diag(m, s);
 }
 
 int ensure_workspace(ps_mesh *m) {
@@ -855,8 +784,8 @@ int ensure_workspace(ps_mesh *m) {
     WA(s32b, float, np);
     WA(part32b, float, sh);
     WA(dots1, double, 3 * m->dev.n_chunks + 8);
-    if (m->use_units) WA(halo32, float2, sh);
-    if (m->use_units) WA(pqu, float2, m->dev.n_chunks + 8);
+    if (m->use_halo) WA(halo32, float2, sh);
+    if (m->use_halo) WA(pqu, float2, m->dev.n_chunks + 8);
 #undef WA
     if (rc != PS_OK) {
         dfree_all(c, w.allocs);
@@ -890,19 +819,19 @@ static Cg2Args<T> cg2_args(ps_mesh *m) {
         a.partial = (T *)w.part64;
     }
     a.pq = (typename PartOf<T>::type *)w.pq2;
-    if (sizeof(T) == 4 && m->use_units) a.pq = (typename PartOf<T>::type *)w.pqu;
+    if (sizeof(T) == 4 && m->use_halo) a.pq = (typename PartOf<T>::type *)w.pqu;
     a.z2 = (typename PartOf<T>::type *)w.z3;
     a.g3 = m->g3c;
     a.st = w.st;
-    a.halo = (sizeof(T) == 4 && m->use_units) ? w.halo32 : nullptr;
+    a.halo = (sizeof(T) == 4 && m->use_halo) ? w.halo32 : nullptr;
     return a;
 }
 
-// The paired-patch kernel's chunk shares of p.Ap back to their "unset"
+// k_cg2_stars' chunk shares of p.Ap back to their "unset"
 // pattern, on stream s: at the start of every CG run and before a diagnostic
 // launch, so that no share written after an interrupted launch can be taken
 // for a later one.
-static cudaError_t reset_unit_shares(ps_mesh *m, cudaStream_t s) {
+static cudaError_t reset_shares(ps_mesh *m, cudaStream_t s) {
     if (!m->ws.pqu) return cudaSuccess;
     return cudaMemsetAsync(m->ws.pqu, 0xff, ((size_t)m->dev.n_chunks + 8) * sizeof(float2), s);
 }
@@ -912,18 +841,14 @@ static cudaError_t reset_unit_shares(ps_mesh *m, cudaStream_t s) {
 // 15-55% slower than 256-thread blocks capped at 64 registers.)
 static void launch_k1_f32(ps_mesh *m, const Cg2Args<float> &a, cudaStream_t s) {
     const MeshDev &d = m->dev;
-    if (m->use_units) {
+    if (m->use_halo) {
         const int g = d.n_chunks + 1;   // the chunks and the completion block
-        if (m->unit_threads == 128) {
-            if (d.lumped) k_cg2_units<true, 128, kUnitBlocks128><<<g, 128, d.smu.total, s>>>(d, a);
-            else k_cg2_units<false, 128, kUnitBlocks128><<<g, 128, d.smu.total, s>>>(d, a);
-        } else {
-            if (d.lumped) k_cg2_units<true, 256, 2><<<g, 256, d.smu.total, s>>>(d, a);
-            else k_cg2_units<false, 256, 2><<<g, 256, d.smu.total, s>>>(d, a);
-        }
-    } else if (m->k1_pre) {
-        if (d.dim == 2) k_cg2_chunks<2, float, true><<<d.n_chunks, kBlock, d.sm32.total, s>>>(d, a);
-        else k_cg2_chunks<3, float, true><<<d.n_chunks, kBlock, d.sm32.total, s>>>(d, a);
+        if (m->op_threads == 128)
+            k_cg2_stars<128, 5><<<g, 128, d.sms.total, s>>>(d, a);
+        else if (m->op_threads == 256)
+            k_cg2_stars<256, 3><<<g, 256, d.sms.total, s>>>(d, a);
+        else
+            k_cg2_stars<kStarThreads, 3><<<g, kStarThreads, d.sms.total, s>>>(d, a);
     } else {
         if (d.dim == 2) k_cg2_chunks<2, float><<<d.n_chunks, kBlock, d.sm32.total, s>>>(d, a);
         else k_cg2_chunks<3, float><<<d.n_chunks, kBlock, d.sm32.total, s>>>(d, a);
@@ -973,15 +898,7 @@ static int enqueue_cg_iters(ps_mesh *m, int iters, bool fused, cudaStream_t s) {
     const Cg2Args<T> a = cg2_args<T>(m);
     const SmemLayout &L = sizeof(T) == 4 ? m->dev.sm32 : m->dev.sm64;
     for (int k = 0; k < iters; ++k) {
-        if (sizeof(T) == 4 && m->pipe_grid > 0) {
-            const Cg2Args<float> &af = reinterpret_cast<const Cg2Args<float> &>(a);
-            if (m->dev.dim == 2)
-                k_cg2_chunks_pipe<2><<<m->pipe_grid, kBlock, m->pipe_L0.total, s>>>(m->dev, af, m->pipe_L0,
-                                                                                     m->pipe_L1);
-            else
-                k_cg2_chunks_pipe<3><<<m->pipe_grid, kBlock, m->pipe_L0.total, s>>>(m->dev, af, m->pipe_L0,
-                                                                                     m->pipe_L1);
-        } else if (sizeof(T) == 4)
+        if (sizeof(T) == 4)
             launch_k1_f32(m, reinterpret_cast<const Cg2Args<float> &>(a), s);
         else if (m->dev.dim == 2)
             k_cg2_chunks<2, T><<<m->dev.n_chunks, kBlock, L.total, s>>>(m->dev, a);
@@ -1008,7 +925,7 @@ static int run_cg_until_done(ps_mesh *m, int gi, bool jac, bool fused, cudaStrea
     Workspace &w = m->ws;
     fused = fused && sizeof(T) == 4;
     const int kind = (sizeof(T) == 4 ? 0 : 1) + (jac ? 0 : 2) + (fused ? 4 : 0);
-    const int per_iter = fused ? 1 : (sizeof(T) == 4 && m->use_units ? 3 : 2);
+    const int per_iter = fused ? 1 : (sizeof(T) == 4 && m->use_halo ? 3 : 2);
     if (gi <= 0) {
         const int batch = 15;
         for (;;) {
@@ -1218,7 +1135,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
                 m->launches += 2;
             } else {
                 Cg2Args<float> a = cg2_args<float>(m);
-                CK(reset_unit_shares(m, s));
+                CK(reset_shares(m, s));
                 k_cg2_start<float><<<m->g3c, kBlock, 0, s>>>(m->dev, a, w.r64, scale, w.x32, it_k * it_k, 1,
                                                              max_it - used);
                 m->launches += 1;
@@ -1374,7 +1291,7 @@ extern "C" int ps_debug_cg_apply(ps_mesh *m, const void *x, void *y, double *pap
     hs.rz = 1.0;
     CK(cudaMemcpyAsync(w.st, &hs, sizeof(hs), cudaMemcpyHostToDevice, s));
     const Cg2Args<float> ca = cg2_args<float>(m);
-    CK(reset_unit_shares(m, s));
+    CK(reset_shares(m, s));
     if (ca.halo)
         k_halo_gather<<<grid_for(m->prep.sh_total, m->ctx->sms), kBlock, 0, s>>>(m->prep.sh_total,
                                                                                 m->dev.sh_ids, ca, 0);
@@ -1447,7 +1364,7 @@ extern "C" int ps_debug_prepare(int dim, int64_t n_nodes, const double *coords, 
         stats->chunk_node_refs = pm.loc_total;
         stats->max_chunk_elems = pm.max_elem;
         stats->max_chunk_nodes = pm.max_loc;
-        SmemLayout l64 = make_layout(8, sizeof(NodeD), pm.max_loc, pm.max_patch, pm.max_inc, pm.max_sh);
+        SmemLayout l64 = make_layout(8, pm.max_loc, pm.max_patch, pm.max_inc);
         stats->reserved[0] = pm.n_patches;
         stats->reserved[1] = pm.inc_total;
         stats->device_bytes = l64.total;  // shared memory per block of the FP64 pass
@@ -1476,7 +1393,7 @@ extern "C" int ps_profile_kernel(ps_mesh *m, int which, int reps, void *stream, 
     hs.first = 1;
     hs.free_run = 1;     // the fused pass never stops
     CK(cudaMemcpyAsync(w.st, &hs, sizeof(hs), cudaMemcpyHostToDevice, s));
-    CK(reset_unit_shares(m, s));
+    CK(reset_shares(m, s));
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -1484,14 +1401,7 @@ extern "C" int ps_profile_kernel(ps_mesh *m, int which, int reps, void *stream, 
         switch (which) {
             case 0: {
                 Cg2Args<float> a = cg2_args<float>(m);
-                if (m->pipe_grid > 0) {
-                    if (d.dim == 2)
-                        k_cg2_chunks_pipe<2><<<m->pipe_grid, kBlock, m->pipe_L0.total, s>>>(d, a, m->pipe_L0, m->pipe_L1);
-                    else
-                        k_cg2_chunks_pipe<3><<<m->pipe_grid, kBlock, m->pipe_L0.total, s>>>(d, a, m->pipe_L0, m->pipe_L1);
-                } else {
-                    launch_k1_f32(m, a, s);
-                }
+                launch_k1_f32(m, a, s);
                 break;
             }
             case 1: {
@@ -1574,7 +1484,7 @@ extern "C" int ps_mesh_set_mass(ps_mesh *m, int mass) {
     free_graphs(m);
     if (!m->coeff_ok) return PS_OK;
     RC(ensure_workspace(m));
-    RC(ps::diag_update_device(m, nullptr));
+    RC(ps::star_update_device(m, nullptr, 0.0, nullptr));
     CK(cudaDeviceSynchronize());
     return PS_OK;
 }
