@@ -123,8 +123,10 @@ typedef struct {
                              /* inner iteration (one-reduction PCG): fewer launches */
                              /* and reductions, more vector traffic per pass; FP64  */
                              /* mode falls back to two kernels;                     */
-                             /* PS_ENGINE_AUTO: FUSED for meshes of at most 200,000 */
-                             /* nodes (where it measured faster), else GRAPH;       */
+                             /* PS_ENGINE_AUTO: one cooperative kernel per inner    */
+                             /* solve (or FP64 CG run) when the mesh's vectors fit  */
+                             /* the SMs' shared memory, else FUSED for meshes of at */
+                             /* most 200,000 nodes and GRAPH above;                 */
                              /* PS_ENGINE_PERSISTENT (mixed mode) runs the batched  */
                              /* persistent engine on a batch of one, which gives    */
                              /* bitwise the result the mesh gets in any batch       */

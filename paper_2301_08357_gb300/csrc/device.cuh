@@ -357,6 +357,60 @@ __device__ __forceinline__ void star_eval(const StarF<D> &S, const float *__rest
         default: star_eval_nr<D, 2>(S, id, s_val, out); break;
     }
 }
+// One code path for every star but the closed one of six: seven ring nodes,
+// the ones past nr with zero weights (whatever node their id names) and
+// contributions nobody reads; the edge (r_{nr-1}, r_0) is added at the end.
+// For kernels that run all their phases in a loop, where the instruction
+// cache pays for every variant.
+template <int D, typename T, typename W>
+__device__ __forceinline__ void star_eval_any(const W &S, const StarIds &id, const T *__restrict__ s_val,
+                                              T *__restrict__ out) {
+    constexpr int w0 = D == 3 ? 2 : 1;
+    const int nr = id.nr();
+    const T va = node_value(s_val, id.a());
+    T vb = T(0), oa = T(0), ob = T(0);
+    if (D == 3) {
+        vb = node_value(s_val, id.b());
+        oa = S.weight(0) * (vb - va);
+        ob = -oa;
+    }
+    T pv = T(0), po = T(0);
+#pragma unroll
+    for (int j = 0; j < kStarRing; ++j) {
+        const int w = j == 0 ? w0 : w0 + (D - 1) + D * (j - 1);
+        const T v = node_value(s_val, id.ring(j));
+        T d = v - va;
+        oa = fma(S.weight(w), d, oa);
+        T o = -(S.weight(w) * d);
+        if (D == 3) {
+            d = v - vb;
+            ob = fma(S.weight(w + 1), d, ob);
+            o = fma(-S.weight(w + 1), d, o);
+        }
+        if (j > 0) {
+            d = v - pv;
+            out[2 + j - 1] = fma(S.weight(w + D - 1), d, po);
+            o = fma(-S.weight(w + D - 1), d, o);
+        }
+        pv = v;
+        po = o;
+    }
+    out[2 + kStarRing - 1] = po;
+    out[0] = oa;
+    if (D == 3) out[1] = ob;
+    const T wrap = S.weight(D == 3 ? 1 : 0);
+    if (wrap != T(0)) {
+        const int last = nr - 1;
+        uint32_t w = id.w[1];
+        if (last >= 2) w = id.w[2];
+        if (last >= 4) w = id.w[3];
+        if (last >= 6) w = id.w[4];
+        const uint32_t off = last & 1 ? w >> 16 : w & 0xffffu;
+        const T f = wrap * (node_value(s_val, id.ring(0)) - node_value(s_val, off));
+        out[2 + last] += f;
+        out[2] -= f;
+    }
+}
 __device__ __forceinline__ StarIds star_ids(const uint4 *__restrict__ rec) {
     const uint4 q = __ldg(rec);
     return StarIds{{q.x, q.y, q.z, q.w, __ldg(reinterpret_cast<const uint32_t *>(rec + kStarLanes))}};

@@ -10,6 +10,7 @@
 #include "../../include/pressure.h"
 #include "mesh_prep.h"
 #include "ops.cuh"
+#include "solo.h"
 
 struct ps_mesh;
 
@@ -116,6 +117,8 @@ struct ps_mesh {
     bool alpha_newton = false;         // alpha last set by the general-EOS Newton iteration
     double dt2 = 0.0;
     ps::Workspace ws;
+    ps::Solo *solo = nullptr;   // on-chip CG (solo.cu); null: the mesh does not fit
+    double *d_lump_tot = nullptr;      // [n_pad] lumped weight of each unknown
     void *batch_ws = nullptr;   // owned by batched.cu
     void *proj = nullptr;       // owned by projection.cu
     std::vector<double> coords_host;   // [n_nodes * dim], caller's numbering

@@ -44,6 +44,8 @@ struct MeshDev {
     const double2 *sw64;     // FP64 star weights
     const float *mrow32;     // [loc_total] row sums of the chunk's patches, sign bit set on Dirichlet nodes
     const double *mrow64;
+    const float *mtot32;     // [n_pad] the same summed over all chunks, per unknown
+    const double *mtot64;
     const uint16_t *incp, *inc;
     const int32_t *sh_ids, *shr_ptr, *sh_dest;
     const int4 *sh_info;     // [sh_total] node id, partial range [begin, end), owner flag
@@ -306,11 +308,13 @@ __global__ void __launch_bounds__(256) k_chunks(MeshDev m, VecArgs<T> a) {
 // element values, stored as beta*dt^2 per element slot on the way; null: the
 // stored ones.  Row by row the diagonal is D_ii = m_i - sum_j A_ij.  Interior
 // rows are stored here (0 on Dirichlet rows), shared ones as partial sums
-// (k_shared<double, kDiag>).  A pass of the FP64 pipe (about 29 operations
+// (k_shared<double, kDiag>), the diagonal's n_part of them and then the row
+// sums' (per unknown).  A pass of the FP64 pipe (about 29 operations
 // per tetrahedron) that reads 64 bytes per tetrahedron.
 template <int D>
 __global__ void __launch_bounds__(256, 3) k_star_build(MeshDev m, const int32_t *__restrict__ elem_src,
-                                                    const double *__restrict__ beta, double dt2, double *partial) {
+                                                    const double *__restrict__ beta, double dt2, double *partial,
+                                                    int64_t n_part) {
     extern __shared__ __align__(128) unsigned char smem[];
     const ChunkSmem<double> S = chunk_smem<double>(smem, m.sm64);
     if (threadIdx.x == 0) {
@@ -360,6 +364,12 @@ __global__ void __launch_bounds__(256, 3) k_star_build(MeshDev m, const int32_t 
         if (is_dirichlet(S.val[l])) ml = __longlong_as_double(__double_as_longlong(ml) | (long long)0x8000000000000000ULL);
         const_cast<double *>(m.mrow64)[cd.node_off + l] = ml;
         const_cast<float *>(m.mrow32)[cd.node_off + l] = (float)ml;
+        if (l < cd.n_int) {
+            const_cast<double *>(m.mtot64)[cd.int_begin + l] = ml;
+            const_cast<float *>(m.mtot32)[cd.int_begin + l] = (float)ml;
+        } else {
+            partial[n_part + m.sh_dest[cd.sh_off + (l - cd.n_int)]] = fabs(ml);
+        }
     }
     __syncthreads();
     // off-diagonal row sums, from the weights this thread just stored
@@ -427,6 +437,12 @@ __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_f
             const double dv = dir ? 0.0 : 1.0 / (double)sum;
             const_cast<double *>(m.dinv64)[g] = dv;
             const_cast<float *>(m.dinv32)[g] = (float)dv;
+            // the row sums' partials follow the diagonal's (n_first slots)
+            double mt = 0.0;
+            for (int k = kb; k < ke; ++k) mt += (double)a.partial[n_first + k];
+            if (dir) mt = __longlong_as_double(__double_as_longlong(mt) | (long long)0x8000000000000000ULL);
+            const_cast<double *>(m.mtot64)[g] = mt;
+            const_cast<float *>(m.mtot32)[g] = (float)mt;
         }
     }
     if (MODE != kResid) return;
@@ -548,11 +564,19 @@ static __global__ void k_set_alpha(MeshDev m, int64_t n_loc, const int32_t *__re
 
 // The same from caller-numbered alpha: unknown g takes alpha of its master
 // vertex old_of_new[g].  wl (may be null, lumped mass): the lumped weight
-// |T|/(d+1) summed over the chunk's elements around each local node; alpha
-// then scales it into the row sums, all that a lumped operator takes from it.
+// |T|/(d+1) summed over the chunk's elements around each local node (wl_tot:
+// over all elements, per unknown); alpha then scales it into the row sums, all that a lumped operator takes from it.
 static __global__ void k_set_alpha_user(MeshDev m, int64_t n_loc, const int32_t *__restrict__ loc_node,
                                         const int32_t *__restrict__ old_of_new, const double *__restrict__ alpha_user,
-                                        const double *__restrict__ wl) {
+                                        const double *__restrict__ wl, const double *__restrict__ wl_tot) {
+    if (wl)
+        for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < m.n_nodes;
+             g += (int64_t)gridDim.x * blockDim.x) {
+            double mt = alpha_user[old_of_new[g]] * wl_tot[g];
+            if (m.dirichlet[g]) mt = __longlong_as_double(__double_as_longlong(mt) | (long long)0x8000000000000000ULL);
+            const_cast<double *>(m.mtot64)[g] = mt;
+            const_cast<float *>(m.mtot32)[g] = (float)mt;
+        }
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_loc; k += (int64_t)gridDim.x * blockDim.x) {
         const int g = loc_node[k];
         const double a = alpha_user[old_of_new[g]];

@@ -219,7 +219,8 @@ static int set_smem_attrs() {
     CK(set_max_dyn_smem(k_cg2_stars<kStarThreads, 3>));
     CK(set_max_dyn_smem(k_cg2_stars<256, 3>));
     CK(set_max_dyn_smem(k_cg2_stars<128, 5>));
-    return batched_set_attrs();
+    RC(batched_set_attrs());
+    return solo_set_attrs();
 }
 
 // Launch kernel 1 + kernel 2 of one operator pass (mode MODE, type T).
@@ -395,16 +396,24 @@ static int mesh_upload_impl(ps_ctx *c, ps_mesh *m, const PrepMesh &pm) {
         RC(upload(c, m, &gp, geo.data(), geo.size() * 8));
         d.geo64 = gp;
         RC(upload(c, m, &m->d_lump, lump.data(), lump.size() * 8));
+        std::vector<double> tot(d.n_pad, 0.0);
+        for (int64_t k = 0; k < pm.loc_total; ++k) tot[pm.loc_node[k]] += lump[k];
+        RC(upload(c, m, &m->d_lump_tot, tot.data(), tot.size() * 8));
     }
     float *f;
     double *g;
     double2 *sw;
     RC(upload(c, m, &sw, nullptr, pm.patch_total * (pm.dim == 3 ? kStarVec64<3> : kStarVec64<2>) * 16));
+    CK(cudaMemset(sw, 0, pm.patch_total * (pm.dim == 3 ? kStarVec64<3> : kStarVec64<2>) * 16));   // (unused weights stay 0)
     d.sw64 = sw;
     RC(upload(c, m, &f, nullptr, pm.loc_total * 4));
     d.mrow32 = f;
     RC(upload(c, m, &g, nullptr, pm.loc_total * 8));
     d.mrow64 = g;
+    RC(upload(c, m, &f, nullptr, d.n_pad * 4));
+    d.mtot32 = f;
+    RC(upload(c, m, &g, nullptr, d.n_pad * 8));
+    d.mtot64 = g;
     RC(upload(c, m, &g, nullptr, pm.loc_total * 8));
     d.alpha64 = g;
     RC(upload(c, m, &g, nullptr, pm.patch_total * kPatchMax * 8));
@@ -515,7 +524,9 @@ extern "C" int ps_mesh_upload_periodic(ps_ctx *c, int dim, int64_t n_nodes, cons
         return PS_EINVAL;
     }
     int rc = mesh_upload_impl(c, m, m->prep);
+    if (rc == PS_OK) rc = solo_upload(m);
     if (rc != PS_OK) {
+        solo_release(m);
         dfree_all(c, m->allocs);
         delete m;
         return rc;
@@ -556,6 +567,7 @@ extern "C" void ps_mesh_free(ps_mesh *m) {
     free_workspace(m);
     batched_release_mesh(m);
     projection_release(m);
+    solo_release(m);
     dfree_all(c, m->allocs);
     c->meshes.erase(m);
     delete m;
@@ -586,16 +598,18 @@ extern "C" int ps_mesh_get_stats(const ps_mesh *m, ps_mesh_stats *o) {
 // ---------------------------------------------------------------- ABI: coefficients
 // Star weights, row sums and Jacobi diagonal (d.dinv32, d.dinv64) from the
 // mesh's alpha and beta (null: the beta*dt^2 stored last), on stream s.
+// partial: scratch of two values per shared slot.
 static void launch_star_build(ps_mesh *m, const MeshDev &d, const double *beta, double dt2, double *partial,
                               cudaStream_t s) {
+    const int64_t n_part = m->prep.sh_total;
     if (d.dim == 2)
-        k_star_build<2><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, m->d_elem_src, beta, dt2, partial);
+        k_star_build<2><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, m->d_elem_src, beta, dt2, partial, n_part);
     else
-        k_star_build<3><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, m->d_elem_src, beta, dt2, partial);
+        k_star_build<3><<<d.n_chunks, kBlock, d.sm64.total, s>>>(d, m->d_elem_src, beta, dt2, partial, n_part);
     VecArgs<double> a;
     std::memset(&a, 0, sizeof(a));
     a.partial = partial;
-    k_shared<double, kDiag><<<m->grid2, kBlock, 0, s>>>(d, a, d.n_chunks);
+    k_shared<double, kDiag><<<m->grid2, kBlock, 0, s>>>(d, a, (int)n_part);
 }
 
 static int coeff_upload(ps_mesh *m, const double *alpha, const double *beta, double dt2) {
@@ -625,7 +639,7 @@ static int coeff_upload(ps_mesh *m, const double *alpha, const double *beta, dou
     if (e == cudaSuccess) {
         // star weights, row sums and the Jacobi diagonal (FP64 arithmetic, both precisions stored)
         void *part = nullptr;
-        rc = dalloc(c, &part, (p.sh_total > 0 ? p.sh_total : 1) * 8, tmp);
+        rc = dalloc(c, &part, (p.sh_total > 0 ? p.sh_total : 1) * 16, tmp);
         if (rc != PS_OK) {
             dfree_all(c, tmp);
             return rc;
@@ -736,7 +750,8 @@ int alpha_update_device(ps_mesh *m, const double *alpha_dev, cudaStream_t s, boo
     const PrepMesh &p = m->prep;
     MeshDev &d = m->dev;
     k_set_alpha_user<<<grid_for(p.loc_total, m->ctx->sms), kBlock, 0, s>>>(
-        d, p.loc_total, m->d_loc_node, m->d_old_of_new, alpha_dev, d.lumped && !diag ? m->d_lump : nullptr);
+        d, p.loc_total, m->d_loc_node, m->d_old_of_new, alpha_dev, d.lumped && !diag ? m->d_lump : nullptr,
+        m->d_lump_tot);
     CK(cudaGetLastError());
     if (diag) return star_update_device(m, nullptr, 0.0, s);
     return d.lumped ? PS_OK : star_update_keep_diag(m, s);
@@ -770,7 +785,7 @@ int ensure_workspace(ps_mesh *m) {
     WA(p32, float, np);
     WA(q32, float, np);
     WA(part32, float, sh);
-    WA(part64, double, sh);
+    WA(part64, double, 2 * sh);
     WA(dot1, double, m->dev.n_chunks + m->grid2 + 8);
     WA(dot2, double, 2 * m->grid3 + 8);
     WA(st, CgState, 1);
@@ -1091,21 +1106,26 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
     int rc = PS_OK;
     if (o.mode == PS_MODE_FP64) {
         const int max_restarts = o.max_outer > 0 ? o.max_outer : 40;
+        const bool solo = o.engine == PS_ENGINE_AUTO && m->solo && m->solo->fp64;
         for (;;) {
             rc = true_residual(m, s, &rr);
             if (rc != PS_OK) break;
             ++outer;
             if (rr <= stop_abs2) { status = PS_OK; break; }
             if (used >= max_it || outer > max_restarts) { status = PS_ENOTCONV; break; }
-            {
+            if (solo) {
+                if ((rc = solo_run<double>(m, 1.0, stop_abs2, max_it - used, true, s)) != PS_OK) break;
+            } else {
                 Cg2Args<double> a = cg2_args<double>(m);
                 k_cg2_start<double><<<m->g3c, kBlock, 0, s>>>(m->dev, a, nullptr, 1.0, nullptr, stop_abs2, 0,
                                                               max_it - used);
                 m->launches += 1;
             }
             if ((rc = cuda_status(cudaGetLastError())) != PS_OK) break;
-            if ((rc = run_cg_until_done<double>(m, gi, jac, false, s)) != PS_OK) break;
+            if (!solo && (rc = run_cg_until_done<double>(m, gi, jac, false, s)) != PS_OK) break;
             RC(read_state(m, s, &h));
+            if (solo) solo_end(*m->solo, h.done != 0, h.iters);
+            if (solo && !h.done) { rc = PS_ETIMEOUT; break; }
             used += h.iters;
             if (h.status == kCgBreakdown) { status = PS_EBREAKDOWN; rc = PS_OK; break; }
         }
@@ -1116,6 +1136,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
         // the fused pass is ~30% faster at 35K nodes, equal near 250K, ~20%
         // slower at 900K (its larger vector traffic sits in the latency-bound
         // chunk pass)
+        const bool solo = o.engine == PS_ENGINE_AUTO && m->solo && m->solo->fp32;
         const bool fused = o.engine == PS_ENGINE_FUSED ||
                            (o.engine == PS_ENGINE_AUTO && m->dev.n_nodes <= kFusedMaxNodes);
         for (;;) {
@@ -1128,7 +1149,10 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
             // inner reduction: itol, or only what the outer tolerance still
             // needs (with a factor 10 of margin) when that is less
             const double it_k = inner_reduction(itol, tol, bb, rr);
-            if (fused) {
+            if (solo) {
+                rc = solo_run<float>(m, scale, it_k * it_k, max_it - used, m->dev.n_nodes > kFusedMaxNodes, s);
+                if (rc != PS_OK) break;
+            } else if (fused) {
                 const CG1Vec v = cg1_vec(m);
                 k_cg1_init_state<<<1, 32, 0, s>>>(w.st, it_k * it_k, max_it - used);
                 k_cg1_start<<<g3, kBlock, 0, s>>>(np, m->prep.sh_total, v, w.r64, scale);
@@ -1146,10 +1170,13 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
                 }
             }
             if ((rc = cuda_status(cudaGetLastError())) != PS_OK) break;
-            if ((rc = run_cg_until_done<float>(m, gi, jac, fused, s)) != PS_OK) break;
+            if (!solo && (rc = run_cg_until_done<float>(m, gi, jac, fused, s)) != PS_OK) break;
             RC(read_state(m, s, &h));
+            if (solo) solo_end(*m->solo, h.done != 0, h.iters);
+            if (solo && !h.done) { rc = PS_ETIMEOUT; break; }
             used += h.iters;
             if (h.status == kCgBreakdown) { status = PS_EBREAKDOWN; rc = PS_OK; break; }
+            if (solo) continue;    // (the correction is added already)
             if (fused)
                 k_cg1_correct<<<g3, kBlock, 0, s>>>(np, w.x64, cg1_vec(m), w.st, 1.0 / scale);
             else
@@ -1159,6 +1186,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
         }
     }
     m->dev = saved;
+    if (rc == PS_ETIMEOUT) check_dev_err(m->ctx);
     if (rc != PS_OK) return rc;
     RC(check_dev_err(m->ctx));
     info->iters_outer = outer;
@@ -1349,6 +1377,11 @@ extern "C" int ps_debug_prepare(int dim, int64_t n_nodes, const double *coords, 
         return PS_EINVAL;
     }
     err = validate_prep(pm, conn);
+    if (err.empty() && pm.max_loc <= 16383) {
+        SoloPrep sp;
+        build_solo(pm, 152, sp);
+        if (sp.max_loc <= 16383 && sp.max_star * kPatchSlots <= 65535) err = validate_solo(pm, sp);
+    }
     if (!err.empty()) {
         ps_set_last_error(err.c_str());
         return PS_ESTATE;

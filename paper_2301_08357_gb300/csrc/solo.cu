@@ -1,0 +1,717 @@
+// On-chip CG of one mesh: see solo.h.
+//
+// A mesh of up to a few hundred thousand nodes spends a CG iteration of
+// separate kernels waiting: for launches, for chains of dependent loads (chunk
+// descriptor, ids, vectors, partial sums) and for grid reductions.  Here one
+// cooperative kernel runs the whole inner solve.  Each block owns a contiguous
+// range of star patches and keeps in shared memory, for the unknowns they
+// touch, every CG vector, the incidence lists and the contributions, and in
+// registers the first stars' weights; per iteration it exchanges only
+//   * the partial sums of the unknowns it shares with other blocks, and
+//   * its shares of the three dot products,
+// through L2.  The recurrences are the one-reduction form of cg1.cuh
+// (Chronopoulos and Gear), so there is one exchange per iteration: a block
+// stores its shares into every block's own list, each block waits for its
+// list, sums it in block order and advances the scalars (the same words in
+// the same order, so all take the same decision); the others' partial sums
+// travel, and are read, at the same time.  Every word exchanged carries the iteration's tag
+// beside 32 bits of its value, so a reader knows a word by itself: no fence,
+// no barrier counter, no clearing between iterations.  Two buffers suffice: a
+// block overwrites a word of iteration k in iteration k + 2, after it has seen
+// every block's share of k + 1, which that block stored after its last read of
+// iteration k.  One list per reader costs n^2 words, but a list that all
+// blocks poll took 4 us to arrive (150 readers of the same lines), and a
+// reducing block in between two hops of 1.7 us.
+// Results are bitwise reproducible (fixed orders).  Every wait is bounded; on
+// expiry the error flag is set and the kernel ends.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "../../include/pressure.h"
+#include "internal.h"
+#include "cg1.cuh"
+
+namespace ps {
+
+// ---------------------------------------------------------------- host layout
+constexpr int kSoloResident = 2;   // stars per thread whose FP32 record stays in registers
+static SoloSmem solo_smem(const SoloPrep &p, int esz) {
+    SoloSmem L;
+    uint64_t off = 0;
+    auto take = [&](uint64_t bytes) {
+        const uint64_t at = off;
+        off += (bytes + 15) / 16 * 16;
+        return (uint32_t)at;
+    };
+    const uint64_t v = (uint64_t)p.max_loc * esz;
+    L.val = take(v);
+    L.r = take(v);
+    L.s = take(v);
+    L.p = take(v);
+    L.x = take(v);
+    L.di = take(v);
+    L.m = take(v);
+    L.w = take(v);
+    L.contrib = take(((uint64_t)p.max_star * kPatchSlots + 1) * esz);
+    L.goff = take(((uint64_t)p.max_loc / 32 + 2) * 4);
+    L.ell = take((uint64_t)p.max_ell * 4);
+    L.sh = take((uint64_t)p.max_sh * 16);
+    L.total = (uint32_t)std::min<uint64_t>(off, UINT32_MAX);
+    return L;
+}
+
+// ---------------------------------------------------------------- kernel
+template <typename T>
+struct SoloArgs {
+    const SoloBlock *blocks;
+    const uint4 *ids4;
+    const uint32_t *ids1;
+    const int32_t *gid;
+    const uint32_t *goff, *ell;
+    const int4 *sh;
+    const uint4 *srec;
+    int srows;
+    const double2 *sw64;
+    const T *dinv, *mtot;
+    uint2 *part0, *part1;       // [n_slots * kWords] partial sums, two buffers
+    int n_slots;
+    const double *r64;
+    double *x64;
+    double scale, inv_scale, tol2;
+    int relative, nan_breaks;
+    long long max_iters;
+    uint4 *exch;                // [2 buffers][reader][3 products][writer], two tagged words each
+    uint32_t tag0;              // tag of the first iteration
+    CgState *st;
+    int *err;
+    SoloSmem L;
+};
+
+// What blocks exchange travels in 8-byte words {32 bits of the value, tag}: a
+// word is read and written as a whole, and it is valid when its tag is the
+// iteration's.  No word has to be ordered against another, so neither side
+// needs a fence.
+__device__ __forceinline__ void st_tagged(uint2 *p, uint32_t v, uint32_t tag) {
+    const unsigned long long w = (unsigned long long)v | (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ uint2 ld_tagged(const uint2 *p) {
+    unsigned long long w;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+    return make_uint2((uint32_t)w, (uint32_t)(w >> 32));
+}
+// Two words at once (each valid by its own tag).
+__device__ __forceinline__ void st_pair(uint4 *p, uint32_t v0, uint32_t v1, uint32_t tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | v0), "l"(t | v1) : "memory");
+}
+__device__ __forceinline__ uint4 ld_pair(const uint4 *p) {
+    unsigned long long a, b;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+}
+// A wait's budget: false once it has given up.
+struct Spin {
+    uint32_t polls = 0;
+    bool ok = true;
+    __device__ __forceinline__ bool again() {
+        if (++polls > kGridSpinLimit) ok = false;
+        if (polls > 4096u) __nanosleep(64);
+        return ok;
+    }
+};
+// A value of type T in kWords words per entry; word k of entry e of n at
+// [k * n + e].
+template <typename T> struct Tagged;
+template <> struct Tagged<float> {
+    static constexpr int kWords = 1;
+    static __device__ __forceinline__ void put(uint2 *p, int, int e, float v, uint32_t tag) {
+        st_tagged(p + e, __float_as_uint(v), tag);
+    }
+    static __device__ __forceinline__ float of(const uint2 *w) { return __uint_as_float(w[0].x); }
+};
+template <> struct Tagged<double> {
+    static constexpr int kWords = 2;
+    static __device__ __forceinline__ void put(uint2 *p, int n, int e, double v, uint32_t tag) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+        st_tagged(p + e, (uint32_t)b, tag);
+        st_tagged(p + n + e, (uint32_t)(b >> 32), tag);
+    }
+    static __device__ __forceinline__ double of(const uint2 *w) { return __hiloint2double((int)w[1].x, (int)w[0].x); }
+};
+
+// A dot product's share: a float pair (unevaluated sum) for FP32 vectors, a
+// double for FP64 ones; two words either way.  FP64 additions cost an SM 16
+// cycles per warp, so pairs stay in FP32 until the totals.
+template <typename T> struct Share;
+template <> struct Share<float> {
+    using type = float2;
+    static __device__ __forceinline__ float2 zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ float2 add(float2 a, float2 b) {
+        DotF t;
+        t.hi = a.x;
+        t.lo = a.y;
+        t.merge(b.x, b.y);
+        return make_float2(t.hi, t.lo);
+    }
+    static __device__ __forceinline__ float2 of(const DotF &a) { return make_float2(a.hi, a.lo); }
+    static __device__ __forceinline__ float2 shfl(float2 a, int o) {
+        return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+    }
+    static __device__ __forceinline__ float2 bcast(float2 a, int l) {
+        return make_float2(__shfl_sync(0xffffffffu, a.x, l), __shfl_sync(0xffffffffu, a.y, l));
+    }
+    static __device__ __forceinline__ uint2 bits(float2 a) { return make_uint2(__float_as_uint(a.x), __float_as_uint(a.y)); }
+    static __device__ __forceinline__ float2 from(uint32_t x, uint32_t y) {
+        return make_float2(__uint_as_float(x), __uint_as_float(y));
+    }
+    static __device__ __forceinline__ double total(float2 a) { return (double)a.x + (double)a.y; }
+    static __device__ __forceinline__ bool finite(float2 a) { return isfinite(a.x) && isfinite(a.y); }
+};
+template <> struct Share<double> {
+    using type = double;
+    static __device__ __forceinline__ double zero() { return 0.0; }
+    static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+    static __device__ __forceinline__ double of(const DotD &a) { return a.v; }
+    static __device__ __forceinline__ double shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+    static __device__ __forceinline__ double bcast(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+    static __device__ __forceinline__ uint2 bits(double a) {
+        return make_uint2((uint32_t)__double2loint(a), (uint32_t)__double2hiint(a));
+    }
+    static __device__ __forceinline__ double from(uint32_t x, uint32_t y) { return __hiloint2double((int)y, (int)x); }
+    static __device__ __forceinline__ double total(double a) { return a; }
+    static __device__ __forceinline__ bool finite(double a) { return isfinite(a); }
+};
+template <typename T>
+__device__ __forceinline__ typename Share<T>::type warp_share(typename Share<T>::type v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = Share<T>::add(v, Share<T>::shfl(v, o));
+    return v;
+}
+// Three warp sums at once: after two exchanges each lane carries one product
+// (lane / 8 = 0: a, 1: b, 2: c), which three more add up -- six additions per
+// lane instead of fifteen.  Lanes 0, 8 and 16 hold the results.
+template <typename T>
+__device__ __forceinline__ typename Share<T>::type warp_share3(typename Share<T>::type a, typename Share<T>::type b,
+                                                               typename Share<T>::type c, int lane) {
+    using Sh = Share<T>;
+    const bool up = lane & 16;
+    // lanes of the lower half keep a and b, those of the upper half c
+    typename Sh::type k0 = Sh::add(up ? c : a, Sh::shfl(up ? a : c, 16));
+    typename Sh::type k1 = Sh::add(up ? Sh::zero() : b, Sh::shfl(up ? b : Sh::zero(), 16));
+    const bool odd = lane & 8;
+    typename Sh::type v = Sh::add(odd ? k1 : k0, Sh::shfl(odd ? k0 : k1, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v = Sh::add(v, Sh::shfl(v, o));
+    return v;
+}
+// Positive (not 0, not NaN), from the sign and exponent word.
+__device__ __forceinline__ bool positive(double v) {
+    const int h = __double2hiint(v);
+    return h > 0 && h <= 0x7ff00000;
+}
+
+template <typename T>
+__device__ __forceinline__ T fma_rn(T a, T b, T c);
+template <>
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+template <>
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// The scalars of a run, advanced once per iteration by one warp of every
+// block from the same totals.
+template <typename T>
+struct SoloScalars {
+    using Sh = Share<T>;
+    double rz = 0.0, ra = 0.0, rr0 = 0.0, stop_rr = 0.0;   // gamma; gamma * alpha
+    long long iters = 0;
+    int status = kCgRunning;
+    // t: gamma, delta, rho of iteration `it` in every lane.  quot: alpha in
+    // lane 0, beta in lane 1.  Returns 1 if the run ends.
+    __device__ __forceinline__ int advance(const SoloArgs<T> &A, int it, const typename Sh::type (&t)[3], int lane,
+                                           double &quot) {
+        const double g = Sh::total(t[0]), d = Sh::total(t[1]), rho = Sh::total(t[2]);
+        int done = 0;
+        // alpha' = g / (d - beta g / alpha) = g (rz alpha) / (d (rz alpha) - g g), beta = g / rz
+        const double num = it == 0 || lane == 1 ? g : g * ra;
+        const double den = it == 0 ? d : lane == 1 ? rz : d * ra - g * g;
+        quot = num / den;
+        if (it == 0) {
+            rr0 = rho;
+            stop_rr = A.relative ? A.tol2 * rho : A.tol2;
+            if (A.nan_breaks && !Sh::finite(t[2])) {
+                done = 1;
+                status = kCgBreakdown;
+            } else if (!(rho > 0.0) || (!A.relative && rho <= stop_rr)) {
+                done = 1;
+                status = kCgConverged;
+            } else if (!positive(d) || !Sh::finite(t[0]) || !Sh::finite(t[1])) {
+                done = 1;
+                status = kCgBreakdown;
+            }
+        } else {
+            iters += 1;
+            const bool pos = __shfl_sync(0xffffffffu, positive(den) ? 1 : 0, 0) && positive(ra);
+            if (!Sh::finite(t[0]) || !Sh::finite(t[1]) || !Sh::finite(t[2]) || !pos) {
+                done = 1;
+                status = kCgBreakdown;
+            } else if (rho <= stop_rr) {
+                done = 1;
+                status = kCgConverged;
+            } else if (iters >= A.max_iters) {
+                done = 1;
+                status = kCgMaxIter;
+            }
+        }
+        if (done && lane == 0 && blockIdx.x == 0) {
+            A.st->iters = iters;
+            A.st->status = status;
+            A.st->rr = rho;
+            A.st->rr0 = rr0;
+            A.st->done = 1;
+        }
+        return done;
+    }
+    __device__ __forceinline__ void next(const typename Sh::type (&t)[3], double quot) {
+        rz = Sh::total(t[0]);
+        ra = rz * __shfl_sync(0xffffffffu, quot, 0);
+    }
+};
+// What a finished run tells the blocks.
+enum SoloEnd : int { kSoloRuns = 0, kSoloKeep = 1, kSoloDrop = 2 };
+
+// Sum of a block's (up to) 16 warp sums in a fixed order.
+template <typename T>
+__device__ __forceinline__ typename Share<T>::type sum16(const typename Share<T>::type *v) {
+    using Sh = Share<T>;
+    typename Sh::type a[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll 1
+    for (int w = 4; w < 16; w += 4)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a[k] = Sh::add(a[k], v[w + k]);
+    return Sh::add(Sh::add(a[0], a[1]), Sh::add(a[2], a[3]));
+}
+
+// The loop of the kernel below is kept small on purpose (no unrolling, one copy
+// of the star arithmetic): each of its phases runs once per iteration, and
+// with 40 KB of loop the instruction fetches took longer than the phases
+// (301 x 301 squares: 15k cycles per iteration).
+// Measured per iteration, with the kernels it replaces: 301 x 301 squares 5.8 us
+// (fused pass 16), 64^3 Kuhn 10.2 (operator, update and halo kernels 28), FP64
+// 64 x 64 squares 9.8 (25), FP64 40^3 24 (68).  Bound, 301 x 301 squares: 5.4k of
+// 11.9k cycles are the exchange (a word from one SM's store to another's poll
+// takes 1.7 us on this part, the rest overlaps or adds sums), 3.1k the scalars
+// (dependent FP64 operations), 3.5k the update, stars and node sums; 64^3: 4.5k
+// of 21k the stars (half their records stream from L2), 4.5k the node sums;
+// FP64 40^3: 14.6k the stars, at the FP64 pipe's rate.
+template <int D, typename T>
+__global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
+    constexpr bool F32 = sizeof(T) == 4;
+    constexpr int RES = F32 ? kSoloResident : 1;
+    constexpr int kW = Tagged<T>::kWords;
+    extern __shared__ __align__(128) unsigned char smem[];
+    // (done: set when the run ends, by this thread, and not after a wait's limit)
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.st->done = 0;
+    T *val = reinterpret_cast<T *>(smem + A.L.val), *sr = reinterpret_cast<T *>(smem + A.L.r),
+      *ss = reinterpret_cast<T *>(smem + A.L.s), *sp = reinterpret_cast<T *>(smem + A.L.p),
+      *sx = reinterpret_cast<T *>(smem + A.L.x), *sdi = reinterpret_cast<T *>(smem + A.L.di),
+      *sm = reinterpret_cast<T *>(smem + A.L.m), *sw = reinterpret_cast<T *>(smem + A.L.w),
+      *contrib = reinterpret_cast<T *>(smem + A.L.contrib);
+    uint32_t *goff = reinterpret_cast<uint32_t *>(smem + A.L.goff), *ell = reinterpret_cast<uint32_t *>(smem + A.L.ell);
+    int4 *sh = reinterpret_cast<int4 *>(smem + A.L.sh);
+    using Sh = Share<T>;
+    using ST = typename Sh::type;
+    __shared__ ST s_red[3][16];   // warps' sums; entries past the last warp stay 0
+    __shared__ ST s_seg[3][kSoloMaxBlocks / 32];
+    __shared__ T s_alpha, s_beta;
+    __shared__ int s_end;
+    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = NT >> 5;
+    const int G = gridDim.x, n_seg = (G + 31) / 32;
+    const SoloBlock B = A.blocks[blockIdx.x];
+    const int n_sh = B.n_loc - B.n_int;
+    // ---- the block's part of the mesh and of the residual
+    for (int l = tid; l < B.n_loc; l += NT) {
+        const int g = A.gid[B.node0 + l];
+        sr[l] = (T)(A.r64[g] * A.scale);
+        sdi[l] = A.dinv[g];
+        sm[l] = A.mtot[g];
+        val[l] = ss[l] = sp[l] = sx[l] = sw[l] = T(0);
+    }
+    for (int k = tid; k <= (B.n_loc + 31) / 32; k += NT) goff[k] = A.goff[B.goff0 + k];
+    for (int k = tid; k < B.n_ell; k += NT) ell[k] = A.ell[B.ell0 + k];
+    for (int k = tid; k < n_sh; k += NT) sh[k] = A.sh[B.sh0 + k];
+    auto load_star = [&](StarF<D> &S, int q) {
+        const int s = B.star0 + q;
+        const uint4 id = __ldg(A.ids4 + s);
+        const uint32_t id4 = __ldg(A.ids1 + s);
+        if (D == 3) S.v[kStarVec<D> - 1] = make_uint4(0u, 0u, 0u, 0u);
+        S.load(A.srec + (size_t)(s / kStarLanes) * (A.srows * kStarLanes) + s % kStarLanes);
+        S.v[0] = id;
+        S.v[1].x = id4;
+    };
+    auto eval_star = [&](const StarF<D> &S, T *out) {
+        if constexpr (F32) {
+            const StarIds id = S.ids();
+            if (id.nr() == 6) star_eval_nr<D, 6>(S, id, val, out);
+            else if (id.nr()) star_eval_any<D>(S, id, val, out);
+        }
+    };
+    StarF<D> res[RES];
+    if (F32) {
+#pragma unroll
+        for (int k = 0; k < RES; ++k) {
+            res[k].v[1].x = 0u;
+            if (tid + k * NT < B.n_star) load_star(res[k], tid + k * NT);
+        }
+    }
+    SoloScalars<T> sc;
+    if (tid < 48) s_red[tid / 16][tid % 16] = Sh::zero();
+    if (tid == 0) {
+        s_alpha = s_beta = T(0);
+        s_end = 0;
+        contrib[B.n_star * kPatchSlots] = T(0);   // the lists' padding
+    }
+    __syncthreads();
+    Spin spin;
+    for (int it = 0;; ++it) {
+        const uint32_t tag = A.tag0 + (uint32_t)it;
+        // ---- update
+        const T al = s_alpha, be = s_beta;
+#pragma unroll 1
+        for (int l = tid; l < B.n_loc; l += NT) {
+            const T di = sdi[l], r = sr[l];
+            const T s2 = fma_rn(be, ss[l], sw[l]);
+            const T r2 = fma_rn(-al, s2, r);
+            const T p2 = fma_rn(be, sp[l], di * r);
+            ss[l] = s2;
+            sr[l] = r2;
+            sp[l] = p2;
+            sx[l] = fma_rn(al, p2, sx[l]);
+            val[l] = di * r2;
+        }
+        __syncthreads();
+        // ---- stars
+        if constexpr (F32) {
+#pragma unroll 1
+            for (int q = tid, k = 0; q < B.n_star; q += NT, ++k) {
+                StarF<D> S = k == 0 ? res[0] : res[1];
+                if (k >= RES) load_star(S, q);
+                eval_star(S, contrib + q * kPatchSlots);
+            }
+        } else {
+#pragma unroll 1
+            for (int q = tid; q < B.n_star; q += NT) {
+                const int s = B.star0 + q;
+                const uint4 i4 = __ldg(A.ids4 + s);
+                const StarIds id{{i4.x, i4.y, i4.z, i4.w, __ldg(A.ids1 + s)}};
+                const double2 *wt =
+                    A.sw64 + (size_t)(s / kStarLanes) * (kStarVec64<D> * kStarLanes) + s % kStarLanes;
+                T *out = contrib + q * kPatchSlots;
+                if (id.nr() == 6) {
+                    star_eval64_nr<D, 6>(wt, id, val, out);
+                } else if (id.nr()) {
+                    StarD<D, 7> S;
+                    S.load(wt);
+                    star_eval_any<D>(S, id, val, out);
+                }
+            }
+        }
+        __syncthreads();
+        // ---- node sums and the shares of gamma = r.u, delta = u.A u, rho = r.r
+        uint2 *part = (it & 1) ? A.part1 : A.part0;
+        typename DotOf<T>::type dg, dd, dr;
+#pragma unroll 1
+        for (int l = tid; l < B.n_loc; l += NT) {
+            T c0 = T(0), c1 = T(0);
+#pragma unroll 2
+            for (uint32_t o = goff[l >> 5] + lane, e = goff[(l >> 5) + 1]; o < e; o += 32) {
+                const uint32_t w = ell[o];
+                c0 += contrib[w & 0xffffu];
+                c1 += contrib[w >> 16];
+            }
+            const T c = c0 + c1;
+            const T u = val[l], mr = sm[l], r = sr[l];
+            T w = fma_rn(fabs(mr), u, c);
+            bool own = true;
+            if (l < B.n_int) {
+                sw[l] = is_dirichlet(mr) ? T(0) : w;
+            } else {
+                // (a shared unknown's owner carries its row-sum term and its own products)
+                const int4 si = sh[l - B.n_int];
+                Tagged<T>::put(part, A.n_slots, si.z, c, tag);
+                own = si.w != 0;
+                if (!own) w = c;
+            }
+            dd.add_prod(u, w);       // (u = 0 on Dirichlet nodes)
+            const T ro = own ? r : T(0);
+            dg.add_prod(ro, u);
+            dr.add_prod(ro, ro);
+        }
+        {
+            const ST v = warp_share3<T>(Sh::of(dg), Sh::of(dd), Sh::of(dr), lane);
+            if ((lane & 7) == 0 && lane < 24) s_red[lane >> 3][wid] = v;
+        }
+        __syncthreads();
+        if (G > 1) {
+            // every block's share to every block: a reader's words lie
+            // together and have no other reader
+            uint4 *exch = A.exch + (size_t)(it & 1) * 3 * G * G;
+#pragma unroll 1
+            for (int t = tid; t < 3 * G; t += NT) {
+                const int dst = t / 3, q = t - 3 * dst;
+                const uint2 b = Sh::bits(sum16<T>(s_red[q]));
+                st_pair(exch + (size_t)(3 * dst + q) * G + blockIdx.x, b.x, b.y, tag);
+            }
+            // the shared unknowns' partials, which travel beside the shares
+#pragma unroll 1
+            for (int j = tid; j < n_sh; j += NT) {
+                const int l = B.n_int + j;
+                const int4 si = sh[j];
+                // eight partials' loads are in flight together (a corner of
+                // several blocks has that many); one not there yet is polled
+                T w = T(0);
+#pragma unroll 1
+                for (int k0 = si.x; k0 < si.y; k0 += 8) {
+                    uint2 f[8 * kW];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+#pragma unroll
+                        for (int h = 0; h < kW; ++h) {
+                            f[k * kW + h] = make_uint2(0u, tag);
+                            if (k0 + k < si.y) f[k * kW + h] = ld_tagged(part + h * A.n_slots + k0 + k);
+                        }
+                    bool all = true;
+#pragma unroll
+                    for (int k = 0; k < 8 * kW; ++k) all = all && f[k].y == tag;
+                    if (all) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) w += Tagged<T>::of(f + k * kW);
+                    } else if (spin.again()) {
+                        k0 -= 8;
+                    }
+                }
+                const T mr = sm[l];
+                sw[l] = is_dirichlet(mr) ? T(0) : fma_rn(mr, val[l], w);
+            }
+            const uint4 *mine = exch + (size_t)3 * blockIdx.x * G;
+#pragma unroll 1
+            for (int sg = wid; sg < 3 * n_seg; sg += nw) {
+                const int q = sg / n_seg, b = (sg - q * n_seg) * 32 + lane;
+                ST v = Sh::zero();
+                if (b < G) {
+                    const uint4 *w = mine + q * G + b;
+                    uint4 x = ld_pair(w);
+                    while ((x.y != tag || x.w != tag) && spin.again()) x = ld_pair(w);
+                    v = Sh::from(x.x, x.z);
+                }
+                __syncwarp();
+                v = warp_share<T>(v);
+                if (lane == 0) s_seg[q][sg - q * n_seg] = v;
+            }
+        } else if (tid < 3) {
+            s_seg[tid][0] = sum16<T>(s_red[tid]);
+        }
+        __syncthreads();
+        if (wid == 0) {
+            // lane 8 q + k: segment k of product q
+            const int q = lane >> 3, k = lane & 7;
+            ST v = q < 3 && k < n_seg ? s_seg[q][k] : Sh::zero();
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) v = Sh::add(v, Sh::shfl(v, o));
+            const ST t[3] = {Sh::bcast(v, 0), Sh::bcast(v, 8), Sh::bcast(v, 16)};
+            double quot;
+            const int done = sc.advance(A, it, t, lane, quot);
+            if (lane == 0) {
+                s_alpha = (T)quot;
+                s_end = !done ? kSoloRuns : sc.status == kCgBreakdown ? kSoloDrop : kSoloKeep;
+            }
+            if (lane == 1 && it > 0) s_beta = (T)quot;
+            sc.next(t, quot);
+        }
+        const bool ok = __syncthreads_and(spin.ok) != 0;
+        if (!ok) {
+            if (tid == 0) atomicOr(A.err, kErrGridTimeout);
+            return;
+        }
+        if (s_end) break;
+    }
+    if (s_end == kSoloDrop) return;
+    for (int l = tid; l < B.n_loc; l += NT)
+        if (l < B.n_int || sh[l - B.n_int].w) {
+            const int g = A.gid[B.node0 + l];
+            A.x64[g] += (double)sx[l] * A.inv_scale;
+        }
+}
+
+// ---------------------------------------------------------------- host side
+static int solo_rc(cudaError_t e) {
+    if (e == cudaSuccess) return PS_OK;
+    ps_set_last_error(cudaGetErrorString(e));
+    return cuda_status(e);
+}
+
+template <typename F>
+static cudaError_t solo_attr(F *func) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, (const void *)func);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void *)func, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 optin - (int)fa.sharedSizeBytes);
+    return e;
+}
+
+int solo_set_attrs() {
+    cudaError_t e = solo_attr(k_solo_cg<2, float>);
+    if (e == cudaSuccess) e = solo_attr(k_solo_cg<3, float>);
+    if (e == cudaSuccess) e = solo_attr(k_solo_cg<2, double>);
+    if (e == cudaSuccess) e = solo_attr(k_solo_cg<3, double>);
+    return solo_rc(e);
+}
+
+int solo_upload(ps_mesh *m) {
+    const PrepMesh &pm = m->prep;
+    ps_ctx *c = m->ctx;
+    // even the lists of a larger mesh cannot fit (a star and its share of a
+    // block's nodes take over 80 bytes of FP32 shared memory)
+    if (pm.n_patches * 80 > (int64_t)std::min(c->sms, kSoloMaxBlocks) * 227 * 1024) return PS_OK;
+    SoloPrep sp;
+    build_solo(pm, c->sms, sp);
+    if (sp.max_loc * 4 > 65535 || (int64_t)sp.max_star * kPatchSlots > 65535) return PS_OK;
+    Solo *S = new Solo();
+    S->n_blocks = (int)sp.blocks.size();
+    S->n_slots = sp.n_slots;
+    S->sm32 = solo_smem(sp, 4);
+    S->sm64 = solo_smem(sp, 8);
+    S->threads = sp.max_star <= 128 ? 128 : sp.max_star <= 256 ? 256 : 512;
+    // one block per SM: cooperative launch needs them all resident
+    auto fits = [&](auto *k, uint32_t bytes) {
+        int per = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, S->threads, bytes);
+        cudaGetLastError();
+        return e == cudaSuccess && (int64_t)per * c->sms >= S->n_blocks;
+    };
+    const uint32_t lim = 226 * 1024;
+    if (pm.dim == 2) {
+        S->fp32 = S->sm32.total <= lim && fits(k_solo_cg<2, float>, S->sm32.total);
+        S->fp64 = S->sm64.total <= lim && fits(k_solo_cg<2, double>, S->sm64.total);
+    } else {
+        S->fp32 = S->sm32.total <= lim && fits(k_solo_cg<3, float>, S->sm32.total);
+        S->fp64 = S->sm64.total <= lim && fits(k_solo_cg<3, double>, S->sm64.total);
+    }
+    if (!S->fp32 && !S->fp64) {
+        delete S;
+        return PS_OK;
+    }
+    std::vector<uint32_t> i4((size_t)pm.patch_total * 4), i1((size_t)pm.patch_total);
+    for (int64_t q = 0; q < pm.patch_total; ++q) {
+        for (int k = 0; k < 4; ++k) i4[q * 4 + k] = sp.ids[q * kStarIds + k];
+        i1[q] = sp.ids[q * kStarIds + 4];
+    }
+    int rc = PS_OK;
+    auto up = [&](auto **dst, const void *src, size_t bytes) {
+        void *p = nullptr;
+        if (rc == PS_OK) rc = dalloc(c, &p, bytes, m->allocs);
+        if (rc == PS_OK && bytes) rc = solo_rc(cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice));
+        *dst = reinterpret_cast<std::remove_reference_t<decltype(*dst)>>(p);
+    };
+    up(&S->blocks, sp.blocks.data(), sp.blocks.size() * sizeof(SoloBlock));
+    up(&S->ids4, i4.data(), i4.size() * 4);
+    up(&S->ids1, i1.data(), i1.size() * 4);
+    up(&S->gid, sp.gid.data(), sp.gid.size() * 4);
+    up(&S->goff, sp.goff.data(), sp.goff.size() * 4);
+    up(&S->ell, sp.ell.data(), sp.ell.size() * 4);
+    up(&S->sh, sp.sh.data(), sp.sh.size() * 4);
+    if (rc != PS_OK) {
+        delete S;       // (the arrays belong to the mesh's allocations)
+        return rc;
+    }
+    m->solo = S;
+    return PS_OK;
+}
+
+void solo_release(ps_mesh *m) {
+    delete m->solo;
+    m->solo = nullptr;
+}
+
+template <typename T>
+int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, cudaStream_t s) {
+    constexpr bool F32 = sizeof(T) == 4;
+    Solo &S = *m->solo;
+    Workspace &w = m->ws;
+    const size_t part_bytes = (size_t)std::max(S.n_slots, 1) * 2 * Tagged<double>::kWords * sizeof(uint2);
+    const size_t exch_bytes = (size_t)6 * S.n_blocks * S.n_blocks * sizeof(uint4);
+    cudaError_t e = cudaSuccess;
+    if (!S.exch) {
+        void *p = nullptr;
+        int rc = dalloc(m->ctx, &p, part_bytes, w.allocs);
+        if (rc != PS_OK) return rc;
+        S.part = p;
+        rc = dalloc(m->ctx, &p, exch_bytes, w.allocs);
+        if (rc != PS_OK) return rc;
+        S.exch = (uint4 *)p;
+        S.tag = 0;
+    }
+    // tags of a run: tag + 1 .. tag + its iterations + 1 (never reused before
+    // the words are cleared; a run that gave up leaves tag = 0)
+    if (S.tag == 0 || S.tag > 0x40000000u || max_iters > 0x20000000) {
+        e = cudaMemsetAsync(S.part, 0, part_bytes, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(S.exch, 0, exch_bytes, s);
+        if (e != cudaSuccess) return solo_rc(e);
+        S.tag = 1;
+    }
+    SoloArgs<T> A;
+    std::memset(&A, 0, sizeof(A));
+    A.blocks = S.blocks;
+    A.ids4 = S.ids4;
+    A.ids1 = S.ids1;
+    A.gid = S.gid;
+    A.goff = S.goff;
+    A.ell = S.ell;
+    A.sh = S.sh;
+    A.srec = m->dev.srec;
+    A.srows = m->dev.srows;
+    A.sw64 = m->dev.sw64;
+    A.dinv = F32 ? (const T *)m->dev.dinv32 : (const T *)m->dev.dinv64;
+    A.mtot = F32 ? (const T *)m->dev.mtot32 : (const T *)m->dev.mtot64;
+    A.part0 = (uint2 *)S.part;
+    A.part1 = A.part0 + (size_t)S.n_slots * Tagged<T>::kWords;
+    A.n_slots = S.n_slots;
+    A.r64 = w.r64;
+    A.x64 = w.x64;
+    A.scale = scale;
+    A.inv_scale = 1.0 / scale;
+    A.tol2 = tol2;
+    A.relative = F32 ? 1 : 0;
+    A.nan_breaks = nan_breaks ? 1 : 0;
+    A.max_iters = std::min(max_iters, (long long)0x20000000);
+    A.exch = S.exch;
+    A.tag0 = S.tag + 1;
+    A.st = w.st;
+    A.err = m->ctx->d_err;
+    A.L = F32 ? S.sm32 : S.sm64;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(S.n_blocks);
+    cfg.blockDim = dim3(F32 ? S.threads : std::min(S.threads, 256));
+    cfg.dynamicSmemBytes = A.L.total;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void *args[] = {&A};
+    const void *k = m->dev.dim == 2 ? (const void *)k_solo_cg<2, T> : (const void *)k_solo_cg<3, T>;
+    m->launches += 1;
+    return solo_rc(cudaLaunchKernelExC(&cfg, k, args));
+}
+template int solo_run<float>(ps_mesh *, double, double, long long, bool, cudaStream_t);
+template int solo_run<double>(ps_mesh *, double, double, long long, bool, cudaStream_t);
+
+}  // namespace ps

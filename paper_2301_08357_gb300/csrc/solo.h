@@ -1,0 +1,48 @@
+// On-chip CG of one mesh (solo.cu): the inner solve of ps_pressure_solve in
+// one cooperative kernel whose blocks keep their part of every CG vector in
+// shared memory from the first iteration to the last.
+#pragma once
+#include "ops.cuh"
+#include "solo_prep.h"
+
+struct ps_mesh;
+
+namespace ps {
+
+// Offsets of a block's arrays in shared memory.
+struct SoloSmem {
+    uint32_t val, r, s, p, x, di, m, w, contrib, goff, ell, sh, total;
+};
+
+// Device copy, owned by the mesh (null: the mesh does not fit).
+struct Solo {
+    int n_blocks = 0, n_slots = 0;
+    int threads = 0;               // FP32 kernel (the FP64 one: at most 256)
+    SoloBlock *blocks = nullptr;
+    uint4 *ids4 = nullptr;
+    uint32_t *ids1 = nullptr;
+    int32_t *gid = nullptr;
+    uint32_t *goff = nullptr, *ell = nullptr;
+    int4 *sh = nullptr;
+    SoloSmem sm32, sm64;
+    bool fp32 = false, fp64 = false;   // which precisions fit
+    // workspace, allocated by the first solve
+    void *part = nullptr;              // partial sums, two buffers of tagged words
+    uint4 *exch = nullptr;             // dot-product shares, two buffers of tagged words
+    uint32_t tag = 0;                  // last tag used (0: the words are to be cleared)
+};
+
+int solo_set_attrs();
+int solo_upload(ps_mesh *m);
+void solo_release(ps_mesh *m);
+// One inner run from the residual r64 (times scale) in the mesh's workspace:
+// x64 += the correction found / scale; the CG state receives the iteration
+// count and status.  T = float: relative reduction tol2 of r.r; double: stop
+// at r.r <= tol2.
+template <typename T>
+int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, cudaStream_t s);
+// After the run's state is on the host: iters of it (done) or no end (a wait
+// gave up).
+inline void solo_end(Solo &S, bool done, long long iters) { S.tag = done ? S.tag + (uint32_t)iters + 2u : 0u; }
+
+}  // namespace ps
