@@ -286,7 +286,7 @@ int ps_pressure_apply(ps_mesh *mesh, const void *x_dev, void *y_dev, int precisi
  * allocator already holds the memory they may use, or an allocation would
  * synchronise the device inside a time-critical loop).  The paper has no
  * counterpart: this is a deployment variant of the same operator.
- * Scratch (permuted copies of x and y, shared-node partial sums) lives in one
+ * Scratch (shared-node partial sums) lives in one
  * file-scope device array of 16 MiB that every GPU loading the library holds
  * until exit; meshes needing more (about 2 x n_nodes x 4 or 8 bytes plus the
  * partial sums) are rejected with PS_EINVAL and a ps_last_error message.  The

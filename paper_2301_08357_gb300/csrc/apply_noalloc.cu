@@ -6,9 +6,9 @@
 // has already reserved the device memory it is allowed to use (a fresh
 // cudaMalloc would fail or push it over its budget), or a solver loop that
 // must not let an allocation implicitly synchronise the device between time
-// steps.  ps_pressure_apply allocates its workspace (permuted copies of x and
-// y, partial sums of shared nodes) on first use; this variant instead carves
-// that scratch out of one file-scope __device__ array, which every GPU that
+// steps.  ps_pressure_apply allocates the mesh's solver workspace (its scratch
+// among it: partial sums of shared nodes) on first use; this variant instead
+// carves that scratch out of one file-scope __device__ array, which every GPU that
 // loads the library holds until the process exits.
 //
 // The array's host-side name is only a stand-in; the device address is looked
@@ -80,6 +80,9 @@ extern "C" int ps_pressure_apply_noalloc(ps_mesh *m, const void *x, void *y, int
     const size_t esz = prec == PS_F32 ? 4 : 8;
     const int64_t np = m->dev.n_pad;
     const int64_t sh = m->prep.sh_total > 0 ? m->prep.sh_total : 1;
+    // the documented limit: room for permuted copies of x and y beside the
+    // partial sums (only the latter are used: the kernels read x and write y
+    // in the caller's numbering)
     const size_t need = 2 * align256((size_t)np * esz) + align256((size_t)sh * esz);
     if (need > kScratchBytes) {
         char msg[160];
@@ -98,39 +101,7 @@ extern "C" int ps_pressure_apply_noalloc(ps_mesh *m, const void *x, void *y, int
     void *base = nullptr;
     int rc = scratch_address(m->ctx->device, &base);
     if (rc != PS_OK) return rc;
-    unsigned char *b = static_cast<unsigned char *>(base);
-    void *xi = b;
-    void *yi = b + align256((size_t)np * esz);
-    void *part = b + 2 * align256((size_t)np * esz);
     cudaStream_t s = (cudaStream_t)stream;
-    const int64_t n = m->dev.n_nodes, nu = m->prep.n_nodes;   // unknowns, caller's vertices
-    const int g = grid_for(n, m->ctx->sms), gu = grid_for(nu, m->ctx->sms);
-    if (prec == PS_F32) {
-        k_perm_in<float, float><<<g, kChunkThreads, 0, s>>>(n, (const float *)x, (float *)xi, m->d_old_of_new, m->dev.dirichlet);
-        VecArgs<float> a;
-        std::memset(&a, 0, sizeof(a));
-        a.x = (const float *)xi;
-        a.y = (float *)yi;
-        a.partial = (float *)part;
-        rc = launch_pass<float, kApply>(m, a, s);
-        if (rc != PS_OK) return rc;
-        k_perm_out<float, float><<<gu, kChunkThreads, 0, s>>>(nu, (const float *)yi, (float *)y, m->d_new_of_old);
-    } else {
-        k_perm_in<double, double><<<g, kChunkThreads, 0, s>>>(n, (const double *)x, (double *)xi, m->d_old_of_new,
-                                                    m->dev.dirichlet);
-        VecArgs<double> a;
-        std::memset(&a, 0, sizeof(a));
-        a.x = (const double *)xi;
-        a.y = (double *)yi;
-        a.partial = (double *)part;
-        rc = launch_pass<double, kApply>(m, a, s);
-        if (rc != PS_OK) return rc;
-        k_perm_out<double, double><<<gu, kChunkThreads, 0, s>>>(nu, (const double *)yi, (double *)y, m->d_new_of_old);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) {
-        ps_set_last_error(cudaGetErrorString(e));
-        return PS_ECUDA;
-    }
-    return PS_OK;
+    if (prec == PS_F32) return launch_apply<float>(m, (const float *)x, (float *)y, (float *)base, s);
+    return launch_apply<double>(m, (const double *)x, (double *)y, (double *)base, s);
 }

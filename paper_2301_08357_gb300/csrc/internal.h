@@ -62,6 +62,9 @@ int grid_for(int64_t n, int dev_sms);
 int cuda_status(cudaError_t e);
 SmemLayout make_layout(int esz, int max_loc, int max_patch, int max_inc);
 int ensure_workspace(ps_mesh *m);
+// y = A x in the caller's numbering: two launches, partial sums in `part`.
+template <typename T>
+int launch_apply(ps_mesh *m, const T *x, T *y, T *part, cudaStream_t s);
 template <typename T, int MODE>
 int launch_pass(ps_mesh *m, const VecArgs<T> &a, cudaStream_t s);
 
@@ -105,6 +108,7 @@ struct ps_mesh {
     ps::MeshDev dev;
     std::vector<ps::DevAlloc> allocs;
     int32_t *d_loc_node = nullptr, *d_elem_src = nullptr;
+    int32_t *d_loc_user = nullptr;     // caller's vertex of every local node's unknown
     int32_t *d_old_of_new = nullptr, *d_new_of_old = nullptr;
     int32_t *d_slave_ptr = nullptr, *d_slave = nullptr;   // merged periodic vertices (null: none)
     int grid2 = 1, grid3 = 1, g3c = 1;

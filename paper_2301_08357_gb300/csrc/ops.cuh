@@ -83,6 +83,10 @@ struct VecArgs {
     T *partial;      // [sh_total] partial sums of shared local nodes
     double *dotbuf;  // resid: per-block dot partials
     CgState *st;     // resid: receives r.r
+    // apply in the caller's numbering (null: x and y in the internal one): the
+    // caller's vertex of every local node and of every unknown, and the
+    // vertices merged into an unknown
+    const int32_t *loc_user, *old_of_new, *slave_ptr, *slave;
 };
 
 __device__ __forceinline__ float cg_dir(float dinv, float r, float beta, float p) {
@@ -237,7 +241,9 @@ __device__ typename DotOf<T>::type process_chunk(const MeshDev &m, const VecArgs
             const int l = l0 + k * blockDim.x;
             v[k] = mr[k] = T(0);
             if (l < n_loc) {
-                const int g = l < n_int ? cd.int_begin + l : m.sh_ids[cd.sh_off + (l - n_int)];
+                const int g = MODE == kApply && a.loc_user ? a.loc_user[cd.node_off + l]
+                              : l < n_int                  ? cd.int_begin + l
+                                                           : m.sh_ids[cd.sh_off + (l - n_int)];
                 v[k] = a.x[g];
                 mr[k] = mrow[l];
             }
@@ -269,7 +275,7 @@ __device__ typename DotOf<T>::type process_chunk(const MeshDev &m, const VecArgs
         if (l < n_int) {
             const int g = cd.int_begin + l;
             if (MODE == kApply) {
-                a.y[g] = s;
+                a.y[a.loc_user ? a.loc_user[cd.node_off + l] : g] = s;
             } else {
                 const T rv = dir ? T(0) : a.b[g] - s;
                 a.y[g] = rv;
@@ -428,7 +434,10 @@ __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_f
         for (int k = kb; k < ke; ++k) sum += a.partial[k];
         const bool dir = m.dirichlet[g] != 0;
         if (MODE == kApply) {
-            a.y[g] = dir ? T(0) : sum;
+            const T v = dir ? T(0) : sum;
+            a.y[a.old_of_new ? a.old_of_new[g] : g] = v;
+            if (a.slave_ptr)
+                for (int k = a.slave_ptr[g]; k < a.slave_ptr[g + 1]; ++k) a.y[a.slave[k]] = v;
         } else if (MODE == kResid) {
             const T rv = dir ? T(0) : a.b[g] - sum;
             a.y[g] = rv;
