@@ -130,12 +130,13 @@ typedef struct {
                              /* PS_ENGINE_PERSISTENT (mixed mode) runs the batched  */
                              /* persistent engine on a batch of one, which gives    */
                              /* bitwise the result the mesh gets in any batch       */
-    int32_t grid_spin_limit; /* diagnostic: polls of the persistent kernel's grid   */
-                             /* barrier before it gives up and the call returns     */
-                             /* PS_ETIMEOUT (batched, persistent and served solves; */
-                             /* 0 = 2^26 polls, each at least 32 ns apart)          */
-    int32_t batch_threads;   /* batched / persistent / served solves: threads per   */
-                             /* block of the persistent kernel (0 = 256, 128, 256)  */
+    int32_t grid_spin_limit; /* diagnostic: polls of a wait between the blocks of a */
+                             /* batch's kernels before it gives up and the call     */
+                             /* returns PS_ETIMEOUT (batched, persistent and served */
+                             /* solves; 0 = 2^26 polls)                             */
+    int32_t batch_threads;   /* batched / persistent / served solves, meshes too    */
+                             /* large for the on-chip kernel: threads per block of  */
+                             /* the persistent kernel (0 = 256, 128, 256)           */
     int32_t batch_order;     /* their task order per pass: 0 = the (mesh, chunk)    */
                              /* list in mesh order, static round robin over blocks; */
                              /* 1 = only the chunks of meshes still running,        */
@@ -417,14 +418,16 @@ int ps_projection_step_eos(ps_mesh *mesh, const ps_eos_opts *opts, const double 
                            double *p_dev, double *wun_dev, double *h_dev, double *rhok_dev,
                            double *newton_res_host, ps_solve_info *info, void *stream);
 
-/* ---- batched solve: many independent meshes in one persistent kernel ----
+/* ---- batched solve: many independent meshes in one kernel ----
  *   meshes  [n] mesh handles of one context (distinct, coefficients set)
  *   b_dev   [n] device pointers, each [n_nodes_i] double, caller numbering
  *   x_dev   [n] device pointers, each [n_nodes_i] double (in: guess, out: sol)
  *   infos   [n] per-mesh results, may be NULL
- * Mixed precision only: every FP32 inner PCG iteration of all unconverged
- * meshes runs inside one cooperative persistent kernel (grid barriers with a
- * bounded spin), FP64 residuals and updates between epochs; the launch
+ * Mixed precision only: the FP32 inner solves of all unconverged meshes run
+ * side by side in one cooperative kernel, each mesh on thread blocks of its
+ * own and at its own pace (meshes whose vectors exceed the SMs' shared memory:
+ * chunk by chunk in a second one, grid barriers between their iterations; all
+ * waits bounded), FP64 residuals and updates between epochs; the launch
  * sequence is captured in a CUDA graph when opts->graph_iters >= 0.
  * Each mesh's arithmetic and reduction order do not depend on which other
  * meshes share the batch.  Returns PS_OK if all converged, else the first
@@ -445,7 +448,9 @@ int ps_batch_solve(ps_mesh *const *meshes, int n, const double *const *b_dev,
  * alone in the single-solve engine between epochs instead. */
 typedef struct {
     int32_t max_slots;        /* requests in flight at once (0 = 64)                */
-    int32_t epoch_iters;      /* inner iterations per epoch (0 = 64)                */
+    int32_t epoch_iters;      /* inner iterations per epoch (0 = 64) of meshes too
+                                 large for the on-chip kernel; the others' inner
+                                 solves run to their end                            */
     size_t hbm_budget_bytes;  /* cap on workspaces of in-flight requests (0 = ctx)  */
     ps_solve_opts opts;       /* solver options for every request                   */
     int32_t single_nodes;     /* requests of cases whose mesh has at least this many
@@ -486,7 +491,7 @@ int ps_server_release(ps_server *srv, ps_ticket ticket);
 
 typedef struct {
     int64_t submitted, completed, failed, in_flight, queued;
-    int64_t epochs;           /* persistent-kernel epochs launched                  */
+    int64_t epochs;           /* epochs launched                                    */
     int64_t peak_in_flight;
     int64_t bytes_in_use;
     double busy_seconds;

@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(256) k_b_resid2(const BMesh *meshes, const int
             in.first = 1;
             in.free_run = 0;
             in.cnt_a = in.cnt_b = 0;
-            st->phase = kPhInnerInit;
+            st->phase = M.solo ? kPhSolo : kPhInnerInit;
         }
     }
 }
@@ -458,6 +458,12 @@ static int ensure_batch_ws(ps_mesh *m) {
         delete w;
         return rc;
     }
+    rc = solo_batch_layout(m, w->allocs, &w->solo);
+    if (rc != PS_OK) {
+        dfree_all(m->ctx, w->allocs);
+        delete w;
+        return rc;
+    }
     m->batch_ws = w;
     return PS_OK;
 }
@@ -467,20 +473,22 @@ int64_t batch_ws_bytes(const ps_mesh *m) {
     // FP64 x b r p q, FP32 x r p q (two buffers each), s (two), D^-1 copies
     // of the unpreconditioned mode, partial sums, per-chunk dots
     const int64_t np = m->dev.n_pad, sh = m->prep.sh_total;
-    return np * (5 * 8 + 12 * 4) + sh * 16 + (int64_t)m->dev.n_chunks * 48;
+    // and the on-chip layout: ids, lists and exchanged words
+    return np * (5 * 8 + 12 * 4) + sh * 16 + (int64_t)m->dev.n_chunks * 48 + m->prep.patch_total * 64;
 }
 
 void batched_release_mesh(ps_mesh *m) {
     if (!m->batch_ws) return;
     BatchMeshWs *w = static_cast<BatchMeshWs *>(m->batch_ws);
     dfree_all(m->ctx, w->allocs);
+    if (w->solo != m->solo) delete w->solo;
     delete w;
     m->batch_ws = nullptr;
 }
 
 // A plan buffer of at least `bytes` (grown by half again when it is too
 // small; the contents are not kept).
-static int plan_buf(ps_ctx *ctx, DevAlloc &a, size_t bytes) {
+int plan_buf(ps_ctx *ctx, DevAlloc &a, size_t bytes) {
     if (a.p && a.bytes >= bytes) return PS_OK;
     if (a.p) {
         cudaFree(a.p);
@@ -497,7 +505,7 @@ void batch_plan_free(BatchPlan &plan) {
     if (plan.graph) cudaGraphExecDestroy(plan.graph);
     if (plan.cap) cudaStreamDestroy(plan.cap);
     if (plan.ctx) {
-        for (DevAlloc *a : {&plan.buf_st, &plan.buf_meshes, &plan.buf_t[0], &plan.buf_t[1], &plan.buf_t[2]})
+        for (DevAlloc *a : {&plan.buf_st, &plan.buf_meshes, &plan.buf_t[0], &plan.buf_t[1], &plan.buf_t[2], &plan.buf_solo})
             if (a->p) {
                 cudaFree(a->p);
                 plan.ctx->bytes -= (int64_t)a->bytes;
@@ -546,6 +554,7 @@ int batch_plan_build(ps_ctx *ctx, ps_mesh *const *meshes, int n, int epoch_iters
     plan.epoch_iters = epoch_iters > 0 ? epoch_iters : 256;
     std::vector<int2> t1, t2, t3;
     plan.h_meshes.resize(n);
+    plan.chunked = false;
     int rc = plan_buf(ctx, plan.buf_st, (size_t)n * sizeof(BState) + 4096);
     if (rc != PS_OK) return rc;
     plan.d_st = (BState *)plan.buf_st.p;
@@ -590,6 +599,8 @@ int batch_plan_build(ps_ctx *ctx, ps_mesh *const *meshes, int n, int epoch_iters
         B.n_segs = w->n_segs;
         B.n_vt = w->n_vt;
         B.st = plan.d_st + i;
+        B.solo = w->solo;
+        plan.chunked = plan.chunked || !w->solo;
         for (int c = 0; c < m->dev.n_chunks; ++c) t1.push_back(make_int2(i, c));
         for (int sg = 0; sg < w->n_segs; ++sg) t2.push_back(make_int2(i, sg));
         for (int v = 0; v < w->n_vt; ++v) t3.push_back(make_int2(i, v));
@@ -619,6 +630,8 @@ int batch_plan_build(ps_ctx *ctx, ps_mesh *const *meshes, int n, int epoch_iters
     }
     if (e != cudaSuccess) return cuda_rc(e);
     std::memset(plan.h_st, 0, (size_t)n * sizeof(BState));
+    rc = solo_plan_build(plan, s);
+    if (rc != PS_OK) return rc;
     plan.L32 = max_layout(plan.meshes, false);
     plan.L64 = max_layout(plan.meshes, true);
     // scalar cache (alpha, beta; parity) per mesh, then the compacted order's
@@ -671,14 +684,11 @@ int batch_upload_states(BatchPlan &plan, cudaStream_t s) {
     return cuda_rc(e);
 }
 
-// Enqueue one epoch on stream s (also used under stream capture).
-static int epoch_enqueue(BatchPlan &plan, cudaStream_t s) {
+// The inner solves of the meshes that are not solved on chip.
+static int pcg_enqueue(BatchPlan &plan, cudaStream_t s) {
     const int n = (int)plan.meshes.size();
     unsigned int *bar = plan_bar(plan);
     int *active = (int *)(bar + 128);
-    k_b_vec<kPrepare><<<plan.n_t3, 256, 0, s>>>(plan.d_meshes, plan.d_t3, active);
-    k_b_resid1<<<plan.n_t1, 256, plan.L64.total, s>>>(plan.d_meshes, plan.d_t1, plan.L64);
-    k_b_resid2<<<plan.n_t2, 256, 0, s>>>(plan.d_meshes, plan.d_t2);
     k_b_vec<kInnerInit><<<plan.n_t3, 256, 0, s>>>(plan.d_meshes, plan.d_t3, active);
     int rc = cuda_rc(cudaGetLastError());
     if (rc != PS_OK) return rc;
@@ -709,6 +719,21 @@ static int epoch_enqueue(BatchPlan &plan, cudaStream_t s) {
     rc = cuda_rc(cudaLaunchKernelExC(&cfg, (const void *)k_batch_pcg, args));
     if (rc != PS_OK) return rc;
     k_b_vec<kCorrect><<<plan.n_t3, 256, 0, s>>>(plan.d_meshes, plan.d_t3, active);
+    return cuda_rc(cudaGetLastError());
+}
+
+// Enqueue one epoch on stream s (also used under stream capture).
+static int epoch_enqueue(BatchPlan &plan, cudaStream_t s) {
+    const int n = (int)plan.meshes.size();
+    unsigned int *bar = plan_bar(plan);
+    int *active = (int *)(bar + 128);
+    k_b_vec<kPrepare><<<plan.n_t3, 256, 0, s>>>(plan.d_meshes, plan.d_t3, active);
+    k_b_resid1<<<plan.n_t1, 256, plan.L64.total, s>>>(plan.d_meshes, plan.d_t1, plan.L64);
+    k_b_resid2<<<plan.n_t2, 256, 0, s>>>(plan.d_meshes, plan.d_t2);
+    int rc = cuda_rc(cudaGetLastError());
+    if (rc == PS_OK) rc = solo_plan_enqueue(plan, s);
+    if (rc == PS_OK && plan.chunked) rc = pcg_enqueue(plan, s);
+    if (rc != PS_OK) return rc;
     k_b_vec<kFinish><<<plan.n_t3, 256, 0, s>>>(plan.d_meshes, plan.d_t3, active);
     rc = cuda_rc(cudaGetLastError());
     if (rc != PS_OK) return rc;
@@ -741,7 +766,9 @@ int batch_epoch(BatchPlan &plan, cudaStream_t s) {
             }
         }
     }
-    int rc;
+    int rc = PS_OK;
+    if (plan.tag_high > 0x40000000) rc = solo_plan_clear(plan, s);
+    if (rc != PS_OK) return rc;
     if (plan.graph)
         rc = cuda_rc(cudaGraphLaunch(plan.graph, s));
     else
@@ -755,9 +782,13 @@ int batch_epoch(BatchPlan &plan, cudaStream_t s) {
     if (herr) {
         cudaMemset(plan.ctx->d_err, 0, sizeof(int));
         cudaMemset(plan_bar(plan), 0, 1024);
+        solo_plan_clear(plan, s);
         ps_set_last_error("batch epoch: a bounded device wait timed out");
         return PS_ETIMEOUT;
     }
+    long long most = 0;
+    for (size_t i = 0; i < plan.meshes.size(); ++i) most = std::max(most, plan.h_st[i].in.iters);
+    plan.tag_high += most + 2;
     return PS_OK;
 }
 
@@ -812,7 +843,7 @@ int batch_solve_locked(ps_mesh *const *meshes, int n, const double *const *b_dev
             ps_solve_info tmp;
             batch_info(plan, i, &tmp);
             tmp.seconds = secs;
-            tmp.kernel_launches = ep * (plan.graph ? 7 : 7);
+            tmp.kernel_launches = ep * (4 + (plan.chunked ? 3 : 0) + (int64_t)plan.launches.size());
             if (infos) infos[i] = tmp;
             if (tmp.status != PS_OK && first_err == PS_OK) first_err = tmp.status;
         }

@@ -4,7 +4,8 @@
 //     a task list covering every mesh of the batch;
 //   * the FP32 inner solves run in one cooperative persistent kernel whose
 //     blocks walk the (mesh, chunk) task list once per CG iteration, with one
-//     grid barrier per iteration.
+//     grid barrier per iteration; meshes that fit on chip (solo.h) run theirs
+//     in the on-chip kernel instead, side by side and each at its own pace.
 // The inner solver is the fused one-reduction PCG pass of cg1.cuh
 // (Chronopoulos and Gear): each chunk updates its nodes from the previous
 // pass's double-buffered vectors, applies A, and contributes its share of
@@ -33,7 +34,8 @@ enum BPhase : int {
     kPhInner = 4,      // FP32 one-reduction PCG in the persistent kernel
     kPhCorrect = 5,    // x64 += d32 * ||r64||
     kPhOutput = 6,     // x back to the caller's numbering
-    kPhDone = 7
+    kPhDone = 7,
+    kPhSolo = 8        // the inner solve of a mesh on chip (solo.cu), instead of phases 3 to 5
 };
 
 struct BState {
@@ -60,6 +62,7 @@ struct BMesh {
     int n_segs, n_vt;
     int64_t n_part;                // partial-sum slots (sh_total)
     BState *st;
+    const Solo *solo;              // host side; null on either: the persistent kernel's mesh
 };
 
 // Host-side batch plan: device arrays of meshes and task lists, the per-mesh
@@ -89,6 +92,16 @@ struct BatchPlan {
     uint32_t spin_limit = kGridSpinLimit;   // grid-barrier polls before giving up
     int threads = 256;                      // threads per block of the persistent kernel
     int order = 0;                          // task order (PcgArgs::order)
+    // meshes solved on chip (solo.h): launches, and their buffer (jobs, block
+    // list, tags and exchanged words)
+    DevAlloc buf_solo{nullptr, 0};
+    std::vector<SoloLaunch> launches;
+    void *d_jobs = nullptr, *zero_at = nullptr;
+    int2 *d_list = nullptr;
+    int *d_ptr = nullptr;
+    size_t zero_bytes = 0;
+    long long tag_high = 0;                 // no tag used so far is above
+    bool chunked = true;                    // some mesh is the persistent kernel's
 };
 
 // Per-mesh batch workspace beyond ps_mesh::ws (FP64 reduction partials).
@@ -96,7 +109,10 @@ struct BatchMeshWs {
     std::vector<DevAlloc> allocs;
     double *dots64 = nullptr, *vdots = nullptr;
     int n_segs = 0, n_vt = 0;
+    Solo *solo = nullptr;          // layout on chip (null: none; may be the mesh's own)
 };
+
+int plan_buf(ps_ctx *ctx, DevAlloc &a, size_t bytes);
 
 // Build (or rebuild) the plan for `n` distinct meshes of one context
 // (workspaces allocated on first use); states start in kPhIdle.  A rebuild
@@ -110,9 +126,10 @@ void batch_plan_free(BatchPlan &plan);
 // at the next batch_upload_states.
 void batch_arm(BatchPlan &plan, int i, const double *b_user, double *x_user, const ps_solve_opts &o);
 int batch_upload_states(BatchPlan &plan, cudaStream_t s);
-// One epoch: prepare / residual / inner-init / persistent PCG (<= epoch_iters
-// iterations) / correct / output for every mesh in the matching phase, then
-// the states are copied to plan.h_st.  Synchronises the stream.
+// One epoch: prepare / residual / on-chip inner solves (to their end) /
+// inner-init / persistent PCG (<= epoch_iters iterations) / correct / output for
+// every mesh in the matching phase, then the states are copied to plan.h_st.
+// Synchronises the stream.
 int batch_epoch(BatchPlan &plan, cudaStream_t s);
 // Fill a solve info from a finished mesh's state.
 void batch_info(const BatchPlan &plan, int i, ps_solve_info *info);

@@ -1129,7 +1129,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
     int rc = PS_OK;
     if (o.mode == PS_MODE_FP64) {
         const int max_restarts = o.max_outer > 0 ? o.max_outer : 40;
-        const bool solo = o.engine == PS_ENGINE_AUTO && m->solo && m->solo->fp64;
+        const bool solo = o.engine == PS_ENGINE_AUTO && m->solo && m->solo->fp64 && solo_ready(m);
         for (;;) {
             rc = true_residual(m, s, &rr);
             if (rc != PS_OK) break;
@@ -1159,7 +1159,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
         // the fused pass is ~30% faster at 35K nodes, equal near 250K, ~20%
         // slower at 900K (its larger vector traffic sits in the latency-bound
         // chunk pass)
-        const bool solo = o.engine == PS_ENGINE_AUTO && m->solo && m->solo->fp32;
+        const bool solo = o.engine == PS_ENGINE_AUTO && m->solo && m->solo->fp32 && solo_ready(m);
         const bool fused = o.engine == PS_ENGINE_FUSED ||
                            (o.engine == PS_ENGINE_AUTO && m->dev.n_nodes <= kFusedMaxNodes);
         for (;;) {
@@ -1380,9 +1380,11 @@ extern "C" int ps_debug_prepare(int dim, int64_t n_nodes, const double *coords, 
     }
     err = validate_prep(pm, conn);
     if (err.empty() && pm.max_loc <= 16383) {
-        SoloPrep sp;
-        build_solo(pm, 152, sp);
-        if (sp.max_loc <= 16383 && sp.max_star * kPatchSlots <= 65535) err = validate_solo(pm, sp);
+        for (int stars : {kSoloStars, kSoloBatchStars}) {
+            SoloPrep sp;
+            build_solo(pm, 152, stars, sp);
+            if (err.empty() && sp.max_loc <= 16383 && sp.max_star * kPatchSlots <= 65535) err = validate_solo(pm, sp);
+        }
     }
     if (!err.empty()) {
         ps_set_last_error(err.c_str());

@@ -27,10 +27,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "../../include/pressure.h"
 #include "internal.h"
+#include "batched.h"
 #include "cg1.cuh"
 
 namespace ps {
@@ -81,6 +83,8 @@ struct SoloArgs {
     double *x64;
     double scale, inv_scale, tol2;
     int relative, nan_breaks;
+    int drop;                   // 1: a breakdown leaves x64 alone, 0: it keeps the last iterate
+    uint32_t spin_limit;        // polls of a wait before it gives up
     long long max_iters;
     uint4 *exch;                // [2 buffers][reader][3 products][writer], two tagged words each
     uint32_t tag0;              // tag of the first iteration
@@ -114,10 +118,11 @@ __device__ __forceinline__ uint4 ld_pair(const uint4 *p) {
 }
 // A wait's budget: false once it has given up.
 struct Spin {
-    uint32_t polls = 0;
+    uint32_t limit, polls = 0;
     bool ok = true;
+    __device__ __forceinline__ explicit Spin(uint32_t l) : limit(l) {}
     __device__ __forceinline__ bool again() {
-        if (++polls > kGridSpinLimit) ok = false;
+        if (++polls >= limit) ok = false;
         if (polls > 4096u) __nanosleep(64);
         return ok;
     }
@@ -230,8 +235,8 @@ struct SoloScalars {
     int status = kCgRunning;
     // t: gamma, delta, rho of iteration `it` in every lane.  quot: alpha in
     // lane 0, beta in lane 1.  Returns 1 if the run ends.
-    __device__ __forceinline__ int advance(const SoloArgs<T> &A, int it, const typename Sh::type (&t)[3], int lane,
-                                           double &quot) {
+    __device__ __forceinline__ int advance(const SoloArgs<T> &A, int bid, int it, const typename Sh::type (&t)[3],
+                                           int lane, double &quot) {
         const double g = Sh::total(t[0]), d = Sh::total(t[1]), rho = Sh::total(t[2]);
         int done = 0;
         // alpha' = g / (d - beta g / alpha) = g (rz alpha) / (d (rz alpha) - g g), beta = g / rz
@@ -265,7 +270,7 @@ struct SoloScalars {
                 status = kCgMaxIter;
             }
         }
-        if (done && lane == 0 && blockIdx.x == 0) {
+        if (done && lane == 0 && bid == 0) {
             A.st->iters = iters;
             A.st->status = status;
             A.st->rr = rho;
@@ -306,14 +311,16 @@ __device__ __forceinline__ typename Share<T>::type sum16(const typename Share<T>
 // (dependent FP64 operations), 3.5k the update, stars and node sums; 64^3: 4.5k
 // of 21k the stars (half their records stream from L2), 4.5k the node sums;
 // FP64 40^3: 14.6k the stars, at the FP64 pipe's rate.
+// bid, G: this block's number among the mesh's G blocks.  The run's end, or
+// kSoloRuns after a wait's limit.
 template <int D, typename T>
-__global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
+__device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bid, const int G) {
+    extern __shared__ __align__(128) unsigned char smem[];
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int RES = F32 ? kSoloResident : 1;
     constexpr int kW = Tagged<T>::kWords;
-    extern __shared__ __align__(128) unsigned char smem[];
     // (done: set when the run ends, by this thread, and not after a wait's limit)
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.st->done = 0;
+    if (bid == 0 && threadIdx.x == 0) A.st->done = 0;
     T *val = reinterpret_cast<T *>(smem + A.L.val), *sr = reinterpret_cast<T *>(smem + A.L.r),
       *ss = reinterpret_cast<T *>(smem + A.L.s), *sp = reinterpret_cast<T *>(smem + A.L.p),
       *sx = reinterpret_cast<T *>(smem + A.L.x), *sdi = reinterpret_cast<T *>(smem + A.L.di),
@@ -328,8 +335,8 @@ __global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
     __shared__ T s_alpha, s_beta;
     __shared__ int s_end;
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = NT >> 5;
-    const int G = gridDim.x, n_seg = (G + 31) / 32;
-    const SoloBlock B = A.blocks[blockIdx.x];
+    const int n_seg = (G + 31) / 32;
+    const SoloBlock B = A.blocks[bid];
     const int n_sh = B.n_loc - B.n_int;
     // ---- the block's part of the mesh and of the residual
     for (int l = tid; l < B.n_loc; l += NT) {
@@ -374,7 +381,7 @@ __global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
         contrib[B.n_star * kPatchSlots] = T(0);   // the lists' padding
     }
     __syncthreads();
-    Spin spin;
+    Spin spin(A.spin_limit);
     for (int it = 0;; ++it) {
         const uint32_t tag = A.tag0 + (uint32_t)it;
         // ---- update
@@ -462,7 +469,7 @@ __global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
             for (int t = tid; t < 3 * G; t += NT) {
                 const int dst = t / 3, q = t - 3 * dst;
                 const uint2 b = Sh::bits(sum16<T>(s_red[q]));
-                st_pair(exch + (size_t)(3 * dst + q) * G + blockIdx.x, b.x, b.y, tag);
+                st_pair(exch + (size_t)(3 * dst + q) * G + bid, b.x, b.y, tag);
             }
             // the shared unknowns' partials, which travel beside the shares
 #pragma unroll 1
@@ -495,7 +502,7 @@ __global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
                 const T mr = sm[l];
                 sw[l] = is_dirichlet(mr) ? T(0) : fma_rn(mr, val[l], w);
             }
-            const uint4 *mine = exch + (size_t)3 * blockIdx.x * G;
+            const uint4 *mine = exch + (size_t)3 * bid * G;
 #pragma unroll 1
             for (int sg = wid; sg < 3 * n_seg; sg += nw) {
                 const int q = sg / n_seg, b = (sg - q * n_seg) * 32 + lane;
@@ -522,10 +529,10 @@ __global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
             for (int o = 4; o > 0; o >>= 1) v = Sh::add(v, Sh::shfl(v, o));
             const ST t[3] = {Sh::bcast(v, 0), Sh::bcast(v, 8), Sh::bcast(v, 16)};
             double quot;
-            const int done = sc.advance(A, it, t, lane, quot);
+            const int done = sc.advance(A, bid, it, t, lane, quot);
             if (lane == 0) {
                 s_alpha = (T)quot;
-                s_end = !done ? kSoloRuns : sc.status == kCgBreakdown ? kSoloDrop : kSoloKeep;
+                s_end = !done ? kSoloRuns : sc.status == kCgBreakdown && A.drop ? kSoloDrop : kSoloKeep;
             }
             if (lane == 1 && it > 0) s_beta = (T)quot;
             sc.next(t, quot);
@@ -533,16 +540,76 @@ __global__ void __launch_bounds__(512, 1) k_solo_cg(SoloArgs<T> A) {
         const bool ok = __syncthreads_and(spin.ok) != 0;
         if (!ok) {
             if (tid == 0) atomicOr(A.err, kErrGridTimeout);
-            return;
+            return kSoloRuns;
         }
         if (s_end) break;
     }
-    if (s_end == kSoloDrop) return;
+    if (s_end == kSoloDrop) return kSoloDrop;
     for (int l = tid; l < B.n_loc; l += NT)
         if (l < B.n_int || sh[l - B.n_int].w) {
             const int g = A.gid[B.node0 + l];
             A.x64[g] += (double)sx[l] * A.inv_scale;
         }
+    return kSoloKeep;
+}
+
+template <int D, typename T>
+__global__ void __launch_bounds__(512, 1) k_solo_cg(const __grid_constant__ SoloArgs<T> A) {
+    solo_run_block<D, T>(A, blockIdx.x, gridDim.x);
+}
+
+// The same for the meshes of a batch that are in their inner solve.  A thread
+// block runs the mesh blocks of its part of the list in order; meshes exchange
+// nothing with each other, so a mesh's arithmetic does not depend on the others.
+// All lists hold the meshes in one order and all thread blocks are resident, so
+// the first unfinished mesh always has its blocks running.
+struct SoloJob {
+    SoloArgs<float> A;          // (scale, tolerance, cap and tag are the state's)
+    BState *bst;
+    uint32_t *tag;              // last tag used
+    int dim, G;
+};
+// Two blocks of 256 threads share an SM at 128 registers, so one mesh's exchange
+// overlaps the other's arithmetic.  16 meshes, half 2D of up to 167,000
+// triangles, half 3D of up to 329,000 tetrahedra: 12.8 ms with a pass over all
+// meshes' chunks per iteration, 5.3 here (a 2D mesh of 167,000 triangles takes
+// 8 us per iteration beside the others, and it is what the call waits for).
+constexpr int kSoloBatchThreads = 256;
+__global__ void __launch_bounds__(512, 1) k_solo_batch(const SoloJob *jobs, const int2 *list, const int *ptr) {
+    __shared__ __align__(16) SoloJob J;
+    __shared__ int s_run;
+#pragma unroll 1
+    for (int k = ptr[blockIdx.x], e = ptr[blockIdx.x + 1]; k < e; ++k) {
+        const int2 me = list[k];            // job, block of the mesh
+        __syncthreads();                    // (the previous run's shared memory)
+        static_assert(sizeof(SoloJob) % 4 == 0, "word copy");
+        for (int w = threadIdx.x; w < (int)(sizeof(SoloJob) / 4); w += blockDim.x)
+            reinterpret_cast<uint32_t *>(&J)[w] = reinterpret_cast<const uint32_t *>(jobs + me.x)[w];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            // (the phase changes at the end of the run, which every block of
+            // the mesh takes part in: all have read it by then)
+            const BState *st = J.bst;
+            s_run = st->phase == kPhSolo;
+            J.A.scale = st->scale;
+            J.A.inv_scale = 1.0 / st->scale;
+            J.A.tol2 = st->in.tol2;
+            J.A.max_iters = min(st->in.max_iters, (long long)0x20000000);
+            J.A.tag0 = *J.tag + 1u;
+        }
+        __syncthreads();
+        if (!s_run) continue;
+        const int end = J.dim == 3 ? solo_run_block<3, float>(J.A, me.y, J.G)
+                                   : solo_run_block<2, float>(J.A, me.y, J.G);
+        if (end == kSoloRuns) return;       // a wait gave up: the others' will
+        if (me.y == 0 && threadIdx.x == 0) {
+            BState *st = J.bst;
+            const long long iters = st->in.iters;   // (this thread wrote it)
+            st->iters_total += iters;
+            st->phase = kPhResid;
+            *J.tag = J.A.tag0 + (uint32_t)iters + 1u;
+        }
+    }
 }
 
 // ---------------------------------------------------------------- host side
@@ -570,52 +637,53 @@ int solo_set_attrs() {
     if (e == cudaSuccess) e = solo_attr(k_solo_cg<3, float>);
     if (e == cudaSuccess) e = solo_attr(k_solo_cg<2, double>);
     if (e == cudaSuccess) e = solo_attr(k_solo_cg<3, double>);
+    if (e == cudaSuccess) e = solo_attr(k_solo_batch);
     return solo_rc(e);
 }
 
-int solo_upload(ps_mesh *m) {
-    const PrepMesh &pm = m->prep;
-    ps_ctx *c = m->ctx;
-    // even the lists of a larger mesh cannot fit (a star and its share of a
-    // block's nodes take over 80 bytes of FP32 shared memory)
-    if (pm.n_patches * 80 > (int64_t)std::min(c->sms, kSoloMaxBlocks) * 227 * 1024) return PS_OK;
-    SoloPrep sp;
-    build_solo(pm, c->sms, sp);
-    if (sp.max_loc * 4 > 65535 || (int64_t)sp.max_star * kPatchSlots > 65535) return PS_OK;
+// Resident blocks of a kernel on the device.
+template <typename F>
+static int64_t solo_resident(F *k, int threads, uint32_t bytes, int sms) {
+    int per = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, threads, bytes);
+    cudaGetLastError();
+    return e == cudaSuccess ? (int64_t)per * sms : 0;
+}
+constexpr uint32_t kSoloSmemMax = 226 * 1024;
+
+// A mesh too large even for its lists alone (a star and its share of a
+// block's nodes take over 80 bytes of FP32 shared memory).
+static bool solo_too_large(const ps_mesh *m) {
+    return m->prep.n_patches * 80 > (int64_t)std::min(m->ctx->sms, kSoloMaxBlocks) * 227 * 1024;
+}
+
+// Blocks of about `stars` stars; null: a block's lists exceed 16 bits.
+static Solo *solo_sizes(const ps_mesh *m, int stars, SoloPrep &sp) {
+    build_solo(m->prep, m->ctx->sms, stars, sp);
+    if (sp.max_loc * 4 > 65535 || (int64_t)sp.max_star * kPatchSlots > 65535) return nullptr;
     Solo *S = new Solo();
     S->n_blocks = (int)sp.blocks.size();
     S->n_slots = sp.n_slots;
     S->sm32 = solo_smem(sp, 4);
     S->sm64 = solo_smem(sp, 8);
     S->threads = sp.max_star <= 128 ? 128 : sp.max_star <= 256 ? 256 : 512;
-    // one block per SM: cooperative launch needs them all resident
-    auto fits = [&](auto *k, uint32_t bytes) {
-        int per = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, S->threads, bytes);
-        cudaGetLastError();
-        return e == cudaSuccess && (int64_t)per * c->sms >= S->n_blocks;
-    };
-    const uint32_t lim = 226 * 1024;
-    if (pm.dim == 2) {
-        S->fp32 = S->sm32.total <= lim && fits(k_solo_cg<2, float>, S->sm32.total);
-        S->fp64 = S->sm64.total <= lim && fits(k_solo_cg<2, double>, S->sm64.total);
-    } else {
-        S->fp32 = S->sm32.total <= lim && fits(k_solo_cg<3, float>, S->sm32.total);
-        S->fp64 = S->sm64.total <= lim && fits(k_solo_cg<3, double>, S->sm64.total);
-    }
-    if (!S->fp32 && !S->fp64) {
-        delete S;
-        return PS_OK;
-    }
+    return S;
+}
+
+// Device copy of a layout into `owner`.  Where the context has no room for it
+// the mesh goes without: *ok = false, PS_OK.
+static int solo_arrays(ps_mesh *m, const SoloPrep &sp, Solo *S, std::vector<DevAlloc> &owner, bool *ok) {
+    const PrepMesh &pm = m->prep;
     std::vector<uint32_t> i4((size_t)pm.patch_total * 4), i1((size_t)pm.patch_total);
     for (int64_t q = 0; q < pm.patch_total; ++q) {
         for (int k = 0; k < 4; ++k) i4[q * 4 + k] = sp.ids[q * kStarIds + k];
         i1[q] = sp.ids[q * kStarIds + 4];
     }
     int rc = PS_OK;
+    std::vector<DevAlloc> mine;
     auto up = [&](auto **dst, const void *src, size_t bytes) {
         void *p = nullptr;
-        if (rc == PS_OK) rc = dalloc(c, &p, bytes, m->allocs);
+        if (rc == PS_OK) rc = dalloc(m->ctx, &p, bytes, mine);
         if (rc == PS_OK && bytes) rc = solo_rc(cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice));
         *dst = reinterpret_cast<std::remove_reference_t<decltype(*dst)>>(p);
     };
@@ -626,12 +694,33 @@ int solo_upload(ps_mesh *m) {
     up(&S->goff, sp.goff.data(), sp.goff.size() * 4);
     up(&S->ell, sp.ell.data(), sp.ell.size() * 4);
     up(&S->sh, sp.sh.data(), sp.sh.size() * 4);
-    if (rc != PS_OK) {
-        delete S;       // (the arrays belong to the mesh's allocations)
-        return rc;
+    *ok = rc == PS_OK;
+    if (*ok) owner.insert(owner.end(), mine.begin(), mine.end());
+    else dfree_all(m->ctx, mine);
+    if (rc == PS_ENOMEM) {
+        cudaGetLastError();
+        rc = PS_OK;
     }
-    m->solo = S;
-    return PS_OK;
+    return rc;
+}
+
+int solo_upload(ps_mesh *m) {
+    if (solo_too_large(m)) return PS_OK;
+    SoloPrep sp;
+    Solo *S = solo_sizes(m, kSoloStars, sp);
+    if (!S) return PS_OK;
+    // one block per SM: cooperative launch needs them all resident
+    auto fits = [&](auto *k, uint32_t bytes) {
+        return bytes <= kSoloSmemMax && solo_resident(k, S->threads, bytes, m->ctx->sms) >= S->n_blocks;
+    };
+    const bool d2 = m->prep.dim == 2;
+    S->fp32 = d2 ? fits(k_solo_cg<2, float>, S->sm32.total) : fits(k_solo_cg<3, float>, S->sm32.total);
+    S->fp64 = d2 ? fits(k_solo_cg<2, double>, S->sm64.total) : fits(k_solo_cg<3, double>, S->sm64.total);
+    bool ok = S->fp32 || S->fp64;
+    const int rc = ok ? solo_arrays(m, sp, S, m->allocs, &ok) : PS_OK;
+    if (ok) m->solo = S;
+    else delete S;
+    return rc;
 }
 
 void solo_release(ps_mesh *m) {
@@ -639,32 +728,35 @@ void solo_release(ps_mesh *m) {
     m->solo = nullptr;
 }
 
+// Bytes of the exchanged words: partial sums (two buffers of 8 bytes per FP32
+// word) and shares, each from a line of its own (the words of a block that share
+// lines with others arrive later: 301 x 301 squares +2.5% per solve).
 template <typename T>
-int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, cudaStream_t s) {
-    constexpr bool F32 = sizeof(T) == 4;
+static size_t solo_part_bytes(const Solo &S) {
+    return ((size_t)std::max(S.n_slots, 1) * 2 * Tagged<T>::kWords * sizeof(uint2) + 255) / 256 * 256;
+}
+static size_t solo_exch_bytes(const Solo &S) {
+    return ((size_t)6 * S.n_blocks * S.n_blocks * sizeof(uint4) + 255) / 256 * 256;
+}
+
+bool solo_ready(ps_mesh *m) {
     Solo &S = *m->solo;
-    Workspace &w = m->ws;
-    const size_t part_bytes = (size_t)std::max(S.n_slots, 1) * 2 * Tagged<double>::kWords * sizeof(uint2);
-    const size_t exch_bytes = (size_t)6 * S.n_blocks * S.n_blocks * sizeof(uint4);
-    cudaError_t e = cudaSuccess;
-    if (!S.exch) {
-        void *p = nullptr;
-        int rc = dalloc(m->ctx, &p, part_bytes, w.allocs);
-        if (rc != PS_OK) return rc;
-        S.part = p;
-        rc = dalloc(m->ctx, &p, exch_bytes, w.allocs);
-        if (rc != PS_OK) return rc;
-        S.exch = (uint4 *)p;
-        S.tag = 0;
+    if (S.exch) return true;
+    void *p = nullptr;
+    if (dalloc(m->ctx, &p, solo_part_bytes<double>(S) + solo_exch_bytes(S), m->ws.allocs) != PS_OK) {
+        cudaGetLastError();
+        return false;
     }
-    // tags of a run: tag + 1 .. tag + its iterations + 1 (never reused before
-    // the words are cleared; a run that gave up leaves tag = 0)
-    if (S.tag == 0 || S.tag > 0x40000000u || max_iters > 0x20000000) {
-        e = cudaMemsetAsync(S.part, 0, part_bytes, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(S.exch, 0, exch_bytes, s);
-        if (e != cudaSuccess) return solo_rc(e);
-        S.tag = 1;
-    }
+    S.part = p;
+    S.exch = (uint4 *)((char *)p + solo_part_bytes<double>(S));
+    S.tag = 0;
+    return true;
+}
+
+// What a run reads of the mesh, and its exchanged words.
+template <typename T>
+static SoloArgs<T> solo_args(const ps_mesh *m, const Solo &S, void *part, uint4 *exch) {
+    constexpr bool F32 = sizeof(T) == 4;
     SoloArgs<T> A;
     std::memset(&A, 0, sizeof(A));
     A.blocks = S.blocks;
@@ -679,22 +771,39 @@ int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool na
     A.sw64 = m->dev.sw64;
     A.dinv = F32 ? (const T *)m->dev.dinv32 : (const T *)m->dev.dinv64;
     A.mtot = F32 ? (const T *)m->dev.mtot32 : (const T *)m->dev.mtot64;
-    A.part0 = (uint2 *)S.part;
+    A.part0 = (uint2 *)part;
     A.part1 = A.part0 + (size_t)S.n_slots * Tagged<T>::kWords;
     A.n_slots = S.n_slots;
-    A.r64 = w.r64;
-    A.x64 = w.x64;
+    A.r64 = m->ws.r64;
+    A.x64 = m->ws.x64;
+    A.relative = F32 ? 1 : 0;
+    A.drop = F32 ? 1 : 0;
+    A.spin_limit = kGridSpinLimit;
+    A.exch = exch;
+    A.st = m->ws.st;
+    A.err = m->ctx->d_err;
+    A.L = F32 ? S.sm32 : S.sm64;
+    return A;
+}
+
+template <typename T>
+int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, cudaStream_t s) {
+    constexpr bool F32 = sizeof(T) == 4;
+    Solo &S = *m->solo;
+    // tags of a run: tag + 1 .. tag + its iterations + 1 (never reused before
+    // the words are cleared; a run that gave up leaves tag = 0)
+    if (S.tag == 0 || S.tag > 0x40000000u || max_iters > 0x20000000) {
+        const cudaError_t e = cudaMemsetAsync(S.part, 0, solo_part_bytes<double>(S) + solo_exch_bytes(S), s);
+        if (e != cudaSuccess) return solo_rc(e);
+        S.tag = 1;
+    }
+    SoloArgs<T> A = solo_args<T>(m, S, S.part, S.exch);
     A.scale = scale;
     A.inv_scale = 1.0 / scale;
     A.tol2 = tol2;
-    A.relative = F32 ? 1 : 0;
     A.nan_breaks = nan_breaks ? 1 : 0;
     A.max_iters = std::min(max_iters, (long long)0x20000000);
-    A.exch = S.exch;
     A.tag0 = S.tag + 1;
-    A.st = w.st;
-    A.err = m->ctx->d_err;
-    A.L = F32 ? S.sm32 : S.sm64;
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(S.n_blocks);
@@ -713,5 +822,145 @@ int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool na
 }
 template int solo_run<float>(ps_mesh *, double, double, long long, bool, cudaStream_t);
 template int solo_run<double>(ps_mesh *, double, double, long long, bool, cudaStream_t);
+
+// ---------------------------------------------------------------- batches
+int solo_batch_layout(ps_mesh *m, std::vector<DevAlloc> &owner, Solo **out) {
+    *out = nullptr;
+    if (solo_too_large(m)) return PS_OK;
+    const int64_t cap = std::min(m->ctx->sms, kSoloMaxBlocks);
+    if (m->prep.n_patches > cap * kSoloBatchStars) {
+        // every SM either way: the layout of the mesh alone
+        if (m->solo && m->solo->fp32 &&
+            solo_resident(k_solo_batch, m->solo->threads, m->solo->sm32.total, m->ctx->sms) >= m->solo->n_blocks)
+            *out = m->solo;
+        return PS_OK;
+    }
+    SoloPrep sp;
+    Solo *S = solo_sizes(m, kSoloBatchStars, sp);
+    if (!S) return PS_OK;
+    S->threads = kSoloBatchThreads;
+    bool ok = S->sm32.total <= kSoloSmemMax &&
+              solo_resident(k_solo_batch, kSoloBatchThreads, S->sm32.total, m->ctx->sms) >= S->n_blocks;
+    const int rc = ok ? solo_arrays(m, sp, S, owner, &ok) : PS_OK;
+    if (ok) *out = S;
+    else delete S;
+    return rc;
+}
+
+int solo_plan_build(BatchPlan &plan, cudaStream_t s) {
+    plan.launches.clear();
+    // longest runs (iterations ~ nodes per side) first, the larger blocks of
+    // the meshes laid out for a solve alone after the others
+    std::vector<int> order;
+    for (size_t i = 0; i < plan.meshes.size(); ++i)
+        if (plan.h_meshes[i].solo) order.push_back((int)i);
+    if (order.empty()) return PS_OK;
+    auto threads = [&](int i) { return plan.h_meshes[i].solo->threads; };
+    auto side = [&](int i) {
+        const PrepMesh &p = plan.meshes[i]->prep;
+        return std::pow((double)p.n_nodes, 1.0 / p.dim);
+    };
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return threads(a) != threads(b) ? threads(a) < threads(b) : side(a) > side(b);
+    });
+    std::vector<SoloJob> jobs(order.size());
+    std::vector<int2> list;
+    std::vector<int> ptr;
+    size_t words = 0;
+    for (size_t j0 = 0, j1; j0 < order.size(); j0 = j1) {
+        SoloLaunch w{(int)ptr.size(), 0, threads(order[j0]), 0u};
+        for (j1 = j0; j1 < order.size() && threads(order[j1]) == w.threads; ++j1)
+            w.smem = std::max(w.smem, plan.h_meshes[order[j1]].solo->sm32.total);
+        const int64_t room = solo_resident(k_solo_batch, w.threads, w.smem, plan.ctx->sms);
+        // a mesh takes the thread blocks that are free first
+        std::vector<std::vector<int2>> mine(room);
+        std::vector<std::pair<double, int>> free(room);   // when, which
+        for (int64_t k = 0; k < room; ++k) free[k] = {0.0, (int)k};
+        for (size_t j = j0; j < j1; ++j) {
+            const Solo &S = *plan.h_meshes[order[j]].solo;
+            if (S.n_blocks > room) {
+                ps_set_last_error("batch: a mesh's blocks are not resident together");
+                return PS_EINVAL;
+            }
+            std::partial_sort(free.begin(), free.begin() + S.n_blocks, free.end());
+            const double end = free[S.n_blocks - 1].first + side(order[j]);
+            for (int k = 0; k < S.n_blocks; ++k) {
+                mine[free[k].second].push_back(make_int2((int)j, k));
+                free[k].first = end;
+            }
+            words += solo_part_bytes<float>(S) + solo_exch_bytes(S);
+        }
+        for (const auto &v : mine) {
+            if (v.empty()) continue;
+            ptr.push_back((int)list.size());
+            list.insert(list.end(), v.begin(), v.end());
+            w.blocks++;
+        }
+        ptr.push_back((int)list.size());
+        plan.launches.push_back(w);
+    }
+    // jobs, block lists, then what starts at zero: tags and words
+    auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
+    const size_t at_list = pad(jobs.size() * sizeof(SoloJob)), at_ptr = at_list + pad(list.size() * sizeof(int2)),
+                 at_tag = at_ptr + pad(ptr.size() * 4), at_words = at_tag + pad(jobs.size() * 4);
+    int rc = plan_buf(plan.ctx, plan.buf_solo, at_words + words);
+    if (rc != PS_OK) return rc;
+    char *base = (char *)plan.buf_solo.p, *next = base + at_words;
+    for (size_t j = 0; j < order.size(); ++j) {
+        const ps_mesh *m = plan.meshes[order[j]];
+        const Solo &S = *plan.h_meshes[order[j]].solo;
+        SoloJob &J = jobs[j];
+        std::memset(&J, 0, sizeof(J));
+        J.A = solo_args<float>(m, S, next, (uint4 *)(next + solo_part_bytes<float>(S)));
+        next += solo_part_bytes<float>(S) + solo_exch_bytes(S);
+        J.A.drop = 0;      // (the batch's correction follows a breakdown too)
+        J.A.spin_limit = plan.spin_limit;
+        J.bst = plan.d_st + order[j];
+        J.A.st = &J.bst->in;
+        J.tag = (uint32_t *)(base + at_tag) + j;
+        J.dim = m->dev.dim;
+        J.G = S.n_blocks;
+    }
+    plan.d_jobs = base;
+    plan.d_list = (int2 *)(base + at_list);
+    plan.d_ptr = (int *)(base + at_ptr);
+    plan.zero_at = base + at_tag;
+    plan.zero_bytes = at_words + words - at_tag;
+    // pageable sources: staged by the runtime before the calls return
+    rc = solo_rc(cudaMemcpyAsync(base, jobs.data(), jobs.size() * sizeof(SoloJob), cudaMemcpyHostToDevice, s));
+    if (rc == PS_OK)
+        rc = solo_rc(cudaMemcpyAsync(plan.d_list, list.data(), list.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+    if (rc == PS_OK) rc = solo_rc(cudaMemcpyAsync(plan.d_ptr, ptr.data(), ptr.size() * 4, cudaMemcpyHostToDevice, s));
+    return rc == PS_OK ? solo_plan_clear(plan, s) : rc;
+}
+
+int solo_plan_clear(BatchPlan &plan, cudaStream_t s) {
+    plan.tag_high = 0;
+    if (plan.launches.empty()) return PS_OK;
+    return solo_rc(cudaMemsetAsync(plan.zero_at, 0, plan.zero_bytes, s));
+}
+
+int solo_plan_enqueue(BatchPlan &plan, cudaStream_t s) {
+    for (const SoloLaunch &w : plan.launches) {
+        cudaLaunchConfig_t cfg;
+        std::memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3(w.blocks);
+        cfg.blockDim = dim3(w.threads);
+        cfg.dynamicSmemBytes = w.smem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const SoloJob *jobs = (const SoloJob *)plan.d_jobs;
+        const int2 *list = plan.d_list;
+        const int *ptr = plan.d_ptr + w.first;
+        void *args[] = {&jobs, &list, &ptr};
+        const int rc = solo_rc(cudaLaunchKernelExC(&cfg, (const void *)k_solo_batch, args));
+        if (rc != PS_OK) return rc;
+    }
+    return PS_OK;
+}
 
 }  // namespace ps

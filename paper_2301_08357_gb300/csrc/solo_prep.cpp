@@ -7,15 +7,11 @@
 
 namespace ps {
 
-// Stars per block of a small mesh (larger ones use every SM): fewer leave
-// threads idle, more lengthen the FP64 pass (57 FP64 operations per star at
-// two per clock and SM).
-constexpr int kSoloStars = 64;
-void build_solo(const PrepMesh &m, int sms, SoloPrep &o) {
+void build_solo(const PrepMesh &m, int sms, int stars, SoloPrep &o) {
     o = SoloPrep();
     const int n_groups = (int)(m.patch_total / kStarLanes);
     sms = std::min(sms, kSoloMaxBlocks);
-    const int64_t G = std::max<int64_t>(1, std::min<int64_t>(sms, (m.n_patches + kSoloStars - 1) / kSoloStars));
+    const int64_t G = std::max<int64_t>(1, std::min<int64_t>(sms, (m.n_patches + stars - 1) / stars));
     // groups -> blocks by real stars
     std::vector<int> chunk_of(n_groups, 0), real(n_groups, 0);
     for (int c = 0; c < m.n_chunks; ++c)

@@ -10,6 +10,16 @@
 namespace ps {
 
 constexpr int kSoloMaxBlocks = 160;
+// Stars per block of a mesh solved alone (larger meshes use every SM): fewer
+// leave threads idle, more lengthen the FP64 pass (57 FP64 operations per star
+// at two per clock and SM).
+constexpr int kSoloStars = 64;
+// Of a mesh in a batch, where the blocks of many meshes share the SMs: with the
+// padding of the groups about two per thread, which stay in registers.  More
+// are more per second but a longer iteration, and the meshes with the most
+// iterations set the time (16 meshes, half 2D of up to 167,000 triangles: 320
+// in 2D 6.0 ms, 448 5.3, 672 6.8; 896 in 3D 7.3).
+constexpr int kSoloBatchStars = 448;
 
 // One block's part of the mesh: a contiguous range of star groups and the
 // unknowns they touch (interior: touched by this block alone; shared after
@@ -38,7 +48,7 @@ struct SoloPrep {
     int n_slots = 0;               // partial sums
     int max_star = 0, max_loc = 0, max_ell = 0, max_sh = 0;
 };
-void build_solo(const PrepMesh &m, int sms, SoloPrep &out);
+void build_solo(const PrepMesh &m, int sms, int stars_per_block, SoloPrep &out);
 // Checks what the kernel relies on: every star's ids name its unknowns in its
 // block's numbering, every contribution is in the list of its node exactly
 // once and all other entries are the zero slot, shared unknowns' partial slots

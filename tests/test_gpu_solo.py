@@ -86,3 +86,51 @@ def test_on_chip_matches_two_kernels(env, name, make, how, mode, precond):
         assert st == (P.PS_ENOTCONV if two[1].iters_inner > 2 else P.PS_OK) and info.iters_inner <= 2
     finally:
         P.ps_mesh_free(m)
+
+
+def test_batch_on_chip(env):
+    """Every form at once, with enough blocks for more than one launch and one
+    mesh that does not fit on chip: each solution meets the oracle's residual
+    and is bitwise the one of the mesh alone."""
+    P, torch, ctx = env
+    forms = FORMS + [("square_150_%d" % k, lambda: S.make_c1(150), {}) for k in range(18)] + [
+        ("cube_44", lambda: S.make_c2(44), {}), ("cube_72", lambda: S.make_c2(72), {})]
+    ms, cases, As = [], [], []
+    try:
+        for name, make, how in forms:
+            case = make()
+            master = case.extra["master"] if how.get("periodic") else None
+            m = P.ps_mesh_upload(ctx, case.dim, case.coords, case.conn, case.dirichlet, periodic=master,
+                                 chunk_elems=how.get("chunk_elems", 1536))
+            ms.append(m)
+            P.ps_coeff_set(m, case.alpha, case.beta, case.dt2)
+            args = (case.dim, case.coords, case.conn, case.dirichlet)
+            if how.get("lumped"):
+                P.ps_mesh_set_mass(m, P.PS_MASS_LUMPED)
+                A = LumpedMatrix(*args, case.alpha, case.beta, case.dt2)
+            elif master is not None:
+                A = PeriodicMatrix(*args, master, case.alpha, case.beta, case.dt2)
+            else:
+                A = oracle.PressureMatrix.from_case(case)
+            cases.append(case)
+            As.append(A)
+        bs = [torch.as_tensor(c.b, device="cuda") for c in cases]
+        xs = [torch.zeros_like(b) for b in bs]
+        opts = P.make_opts(tol=1e-10)
+        st, infos = P.ps_batch_solve(ms, bs, xs, opts)
+        assert st == P.PS_OK
+        for f, c, A, x in zip(forms, cases, As, xs):
+            assert A.residual(c.b, x.cpu().numpy()) <= 1.05e-10, f[0]
+        for k in (0, 1, 5, 8, 10, 12, len(ms) - 2, len(ms) - 1):
+            x = torch.zeros_like(bs[k])
+            st, info = P.ps_batch_solve([ms[k]], [bs[k]], [x], opts)
+            assert st == P.PS_OK and torch.equal(x, xs[k]), forms[k][0]
+            assert info[0].iters_inner == infos[k].iters_inner
+        # a cap on the iterations is reported for the meshes that need more
+        xs = [torch.zeros_like(b) for b in bs]
+        st, capped = P.ps_batch_solve(ms, bs, xs, P.make_opts(tol=1e-10, max_iters=3))
+        for i, c in zip(infos, capped):
+            assert c.iters_inner <= 3 and c.status == (P.PS_OK if i.iters_inner <= 3 else P.PS_ENOTCONV)
+    finally:
+        for m in ms:
+            P.ps_mesh_free(m)
