@@ -134,3 +134,30 @@ def test_batch_on_chip(env):
     finally:
         for m in ms:
             P.ps_mesh_free(m)
+
+
+@pytest.mark.parametrize("make", [lambda: S.shuffle_case(S.make_c1(13)), lambda: S.shuffle_case(S.make_c2(5))],
+                         ids=["square", "cube"])
+def test_infinite_entry_reaches_its_neighbours_only(env, make):
+    """An infinite or NaN value reaches the rows its element matrices couple it
+    to, and no others (2D stars of every size share one code path; an open
+    star's two ends are no neighbours)."""
+    P, torch, ctx = env
+    c = make()
+    m = P.ps_mesh_upload(ctx, c.dim, c.coords, c.conn, c.dirichlet)
+    try:
+        P.ps_coeff_set(m, c.alpha, c.beta, c.dt2)
+        rng = np.random.default_rng(3)
+        for bad in (np.inf, np.nan):
+            for v in rng.choice(np.flatnonzero(c.dirichlet == 0), 24, replace=False):
+                x = rng.standard_normal(c.n_nodes)
+                x[v] = bad
+                near = np.zeros(c.n_nodes, bool)
+                near[np.unique(c.conn[(c.conn == v).any(axis=1)])] = True
+                for prec, dt in ((P.PS_F64, torch.float64), (P.PS_F32, torch.float32)):
+                    xd = torch.as_tensor(x, dtype=dt, device="cuda")
+                    y = torch.empty_like(xd)
+                    P.ps_pressure_apply(m, xd, y, prec)
+                    assert np.all(np.isfinite(y.cpu().numpy()[~near]))
+    finally:
+        P.ps_mesh_free(m)
