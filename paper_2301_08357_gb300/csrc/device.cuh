@@ -77,6 +77,15 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return false;
 }
 
+// ---------------------------------------------------------------- dependent launches
+// Between two kernels of one stream, the second launched with
+// cudaLaunchAttributeProgrammaticStreamSerialization: once every block of the
+// first has passed grid_dep_launch the second's blocks may start, and
+// grid_dep_wait holds them until the first has ended and its writes are
+// visible.  Without the attribute both do nothing.
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- completion counter
 // "Last block" detection: every block publishes its partial result with a
 // plain store, then increments a device-scope counter with acquire-release
@@ -432,7 +441,7 @@ __device__ __forceinline__ void star_eval64(const StarIds &id, const double2 *__
     if (D == 2) {
         // A 2D chunk has stars of every size in one warp: a variant and its
         // loads per size ran one after another (64 x 64 squares, apply in a
-        // graph: 10.6 us per size, 8.3 as six and others, 7.3 as one).
+        // graph: 10.6 us per size, 8.3 as six and others, 7.4 as one).
         StarD<D, kStarRing> S;
         S.load(wt);
         star_eval_any<D, true>(S, id, s_val, out);

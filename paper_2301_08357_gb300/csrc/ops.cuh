@@ -295,6 +295,7 @@ __global__ void __launch_bounds__(256) k_chunks(MeshDev m, VecArgs<T> a) {
     const SmemLayout &L = (sizeof(T) == 4) ? m.sm32 : m.sm64;
     uint64_t *s_bar = reinterpret_cast<uint64_t *>(smem + L.bar);
     double *s_red = reinterpret_cast<double *>(smem + L.red);
+    grid_dep_launch();   // (k_shared's blocks may start once every block here has)
     if (threadIdx.x == 0) {
         mbar_init(s_bar, 1);
         fence_mbar_init();
@@ -426,11 +427,20 @@ __global__ void __launch_bounds__(256) k_shared(MeshDev m, VecArgs<T> a, int n_f
     __shared__ double s_red[34];
     __shared__ bool s_last;
     typename DotOf<T>::type acc;
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < m.n_shared;
-         s += (int64_t)gridDim.x * blockDim.x) {
+    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int kb = 0, ke = 0;
+    if (s < m.n_shared) {
+        kb = m.shr_ptr[s];
+        ke = m.shr_ptr[s + 1];
+    }
+    grid_dep_wait();     // kernel 1 has ended: its partial sums are there
+    for (; s < m.n_shared; s += (int64_t)gridDim.x * blockDim.x) {
         const int64_t g = m.n_int + s;
         T sum = T(0);
-        const int kb = m.shr_ptr[s], ke = m.shr_ptr[s + 1];
+        if (s >= (int64_t)gridDim.x * blockDim.x) {
+            kb = m.shr_ptr[s];
+            ke = m.shr_ptr[s + 1];
+        }
         for (int k = kb; k < ke; ++k) sum += a.partial[k];
         const bool dir = m.dirichlet[g] != 0;
         if (MODE == kApply) {
