@@ -51,13 +51,7 @@ UNIT = "DOF-iter/s"
 # stands, keyed by (kernel, workload), with the capture it came from.  An
 # entry is removed whenever the kernel changes; missing means not captured
 # (the line then reports null).
-TRAFFIC = {
-    ("k_cg2_units<false,128,5>", "c3_3d_kuhn_160^3_stiff_warm_tets24576000_nodes4173281"): {
-        "bytes": 345454336 + 28280064,
-        "source": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum (1 pass, cold L2), third launch of "
-                  "`python bench.py --workload c3 --steps 1 --warmup 2 --launch-list --no-clocks`; "
-                  "profiles/k_cg2_units_kuhn128.md"},
-}
+TRAFFIC = {}
 
 
 def parse():
@@ -297,8 +291,10 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 
 
 def fp64_flops(stats, lumped, cg):
-    """Algorithmic FP64 flops of one FP64 operator pass with the precomputed
-    element geometry (an FMA counts 2): per element the stiffness differences
+    """Algorithmic FP64 flops of one FP64 operator pass element by element, with
+    precomputed element geometry (the passes over star patches do about a
+    quarter of them, so a fraction of the FP64 peak above 1 is possible; an FMA
+    counts 2): per element the stiffness differences
     (3D 24, 2D 13) and the mass term (consistent 3D 47 / 2D 35, lumped 4(d+1)+1),
     3 accumulations; per node the incidence sums E(d+1)/N plus 3 (residual and
     its dot) or 4 (CG direction and p.Ap)."""
