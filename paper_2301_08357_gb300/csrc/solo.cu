@@ -116,11 +116,14 @@ __device__ __forceinline__ uint4 ld_pair(const uint4 *p) {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
     return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
 }
-// A wait's budget: false once it has given up.
+// A wait's budget: false once it has given up.  begin() before every wait (a
+// budget spent over a whole run ended healthy long runs, and after its first
+// 4,096 polls every later one slept).
 struct Spin {
     uint32_t limit, polls = 0;
     bool ok = true;
     __device__ __forceinline__ explicit Spin(uint32_t l) : limit(l) {}
+    __device__ __forceinline__ void begin() { polls = 0; }
     __device__ __forceinline__ bool again() {
         if (++polls >= limit) ok = false;
         if (polls > 4096u) __nanosleep(64);
@@ -384,6 +387,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
     Spin spin(A.spin_limit);
     for (int it = 0;; ++it) {
         const uint32_t tag = A.tag0 + (uint32_t)it;
+        spin.begin();   // (an iteration's words are waited for together)
         // ---- update
         const T al = s_alpha, be = s_beta;
 #pragma unroll 1
