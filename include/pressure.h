@@ -130,10 +130,12 @@ typedef struct {
                              /* PS_ENGINE_PERSISTENT (mixed mode) runs the batched  */
                              /* persistent engine on a batch of one, which gives    */
                              /* bitwise the result the mesh gets in any batch       */
-    int32_t grid_spin_limit; /* diagnostic: polls of a wait between the blocks of a */
-                             /* batch's kernels before it gives up and the call     */
-                             /* returns PS_ETIMEOUT (batched, persistent and served */
-                             /* solves; 0 = 2^26 polls)                             */
+    int32_t grid_spin_limit; /* diagnostic: polls of a wait between the running     */
+                             /* blocks of a batch's kernels before it gives up and  */
+                             /* the call returns PS_ETIMEOUT (batched, persistent   */
+                             /* and served solves; 0 = 2^26 polls).  Blocks that    */
+                             /* wait for others to finish an earlier mesh have the  */
+                             /* default limit and count from the last sign of life  */
     int32_t batch_threads;   /* batched / persistent / served solves, meshes too    */
                              /* large for the on-chip kernel: threads per block of  */
                              /* the persistent kernel (0 = 256, 128, 256)           */

@@ -85,6 +85,7 @@ struct SoloArgs {
     int relative, nan_breaks;
     int drop;                   // 1: a breakdown leaves x64 alone, 0: it keeps the last iterate
     uint32_t spin_limit;        // polls of a wait before it gives up
+    uint32_t *beat;             // in a batch: counts its runs' iterations by 256 and their ends (null: a run alone)
     long long max_iters;
     uint4 *exch;                // [2 buffers][reader][3 products][writer], two tagged words each
     uint32_t tag0;              // tag of the first iteration
@@ -116,15 +117,33 @@ __device__ __forceinline__ uint4 ld_pair(const uint4 *p) {
     asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
     return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
 }
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
 // A wait's budget: false once it has given up.  begin() before every wait (a
 // budget spent over a whole run ended healthy long runs, and after its first
 // 4,096 polls every later one slept).
+// queued: the first wait of a run in a batch, which lasts until thread blocks that
+// still run earlier meshes come to this one.  That may be many runs, so the wait
+// has the default limit, which starts anew with every sign of life (`beat`, 256
+// iterations or the end of any run), and ends at once when some other wait has given up.
 struct Spin {
-    uint32_t limit, polls = 0;
-    bool ok = true;
-    __device__ __forceinline__ explicit Spin(uint32_t l) : limit(l) {}
-    __device__ __forceinline__ void begin() { polls = 0; }
-    __device__ __forceinline__ bool again() {
+    uint32_t limit, polls = 0, seen = 0;
+    bool ok = true, queued = false;
+    __device__ __forceinline__ void begin(uint32_t l, bool q) {
+        limit = l;
+        polls = 0;
+        queued = q;
+    }
+    __device__ __forceinline__ bool again(const uint32_t *beat, const int *err) {
+        if (queued && (polls & 1023u) == 1023u) {
+            const uint32_t now = ld_relaxed(beat);
+            if (now != seen) polls = 0;
+            seen = now;
+            if (ld_relaxed(reinterpret_cast<const uint32_t *>(err))) ok = false;
+        }
         if (++polls >= limit) ok = false;
         if (polls > 4096u) __nanosleep(64);
         return ok;
@@ -384,10 +403,13 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
         contrib[B.n_star * kPatchSlots] = T(0);   // the lists' padding
     }
     __syncthreads();
-    Spin spin(A.spin_limit);
+    Spin spin;
     for (int it = 0;; ++it) {
         const uint32_t tag = A.tag0 + (uint32_t)it;
-        spin.begin();   // (an iteration's words are waited for together)
+        // (an iteration's words are waited for together)
+        const bool queued = it == 0 && A.beat;
+        spin.begin(queued ? kGridSpinLimit : A.spin_limit, queued);
+        if (A.beat && (it & 255) == 255 && bid == 0 && tid == 0) atomicAdd(A.beat, 1u);
         // ---- update
         const T al = s_alpha, be = s_beta;
 #pragma unroll 1
@@ -499,7 +521,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                     if (all) {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) w += Tagged<T>::of(f + k * kW);
-                    } else if (spin.again()) {
+                    } else if (spin.again(A.beat, A.err)) {
                         k0 -= 8;
                     }
                 }
@@ -514,7 +536,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                 if (b < G) {
                     const uint4 *w = mine + q * G + b;
                     uint4 x = ld_pair(w);
-                    while ((x.y != tag || x.w != tag) && spin.again()) x = ld_pair(w);
+                    while ((x.y != tag || x.w != tag) && spin.again(A.beat, A.err)) x = ld_pair(w);
                     v = Sh::from(x.x, x.z);
                 }
                 __syncwarp();
@@ -605,13 +627,14 @@ __global__ void __launch_bounds__(512, 1) k_solo_batch(const SoloJob *jobs, cons
         if (!s_run) continue;
         const int end = J.dim == 3 ? solo_run_block<3, float>(J.A, me.y, J.G)
                                    : solo_run_block<2, float>(J.A, me.y, J.G);
-        if (end == kSoloRuns) return;       // a wait gave up: the others' will
+        if (end == kSoloRuns) return;       // a wait gave up: the others' will, those for this thread block too
         if (me.y == 0 && threadIdx.x == 0) {
             BState *st = J.bst;
             const long long iters = st->in.iters;   // (this thread wrote it)
             st->iters_total += iters;
             st->phase = kPhResid;
             *J.tag = J.A.tag0 + (uint32_t)iters + 1u;
+            atomicAdd(J.A.beat, 1u);
         }
     }
 }
@@ -903,10 +926,10 @@ int solo_plan_build(BatchPlan &plan, cudaStream_t s) {
         ptr.push_back((int)list.size());
         plan.launches.push_back(w);
     }
-    // jobs, block lists, then what starts at zero: tags and words
+    // jobs, block lists, then what starts at zero: tags, the beat and words
     auto pad = [](size_t b) { return (b + 255) / 256 * 256; };
     const size_t at_list = pad(jobs.size() * sizeof(SoloJob)), at_ptr = at_list + pad(list.size() * sizeof(int2)),
-                 at_tag = at_ptr + pad(ptr.size() * 4), at_words = at_tag + pad(jobs.size() * 4);
+                 at_tag = at_ptr + pad(ptr.size() * 4), at_words = at_tag + pad((jobs.size() + 1) * 4);
     int rc = plan_buf(plan.ctx, plan.buf_solo, at_words + words);
     if (rc != PS_OK) return rc;
     char *base = (char *)plan.buf_solo.p, *next = base + at_words;
@@ -919,6 +942,7 @@ int solo_plan_build(BatchPlan &plan, cudaStream_t s) {
         next += solo_part_bytes<float>(S) + solo_exch_bytes(S);
         J.A.drop = 0;      // (the batch's correction follows a breakdown too)
         J.A.spin_limit = plan.spin_limit;
+        J.A.beat = (uint32_t *)(base + at_tag) + jobs.size();
         J.bst = plan.d_st + order[j];
         J.A.st = &J.bst->in;
         J.tag = (uint32_t *)(base + at_tag) + j;

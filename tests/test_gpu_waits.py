@@ -50,3 +50,23 @@ def test_limit_bounds_one_wait_not_a_run(env):
         assert oracle.PressureMatrix.from_case(c).residual(c.b, x.cpu().numpy()) <= 1.05e-10
     finally:
         P.ps_mesh_free(m)
+
+
+def test_blocks_may_wait_for_busy_ones(env):
+    """More meshes than the SMs hold at once, some slow: a mesh's blocks start
+    when the thread blocks they are placed on are free, and the time until then
+    is no wait between running blocks."""
+    P, torch, ctx = env
+    cases = [_stretched(130 + 4 * (k % 6), 1e3 if k % 3 == 0 else 1.0) for k in range(48)]
+    ms = [_upload(P, ctx, c) for c in cases]
+    try:
+        bs = [torch.as_tensor(c.b, device="cuda") for c in cases]
+        xs = [torch.zeros_like(b) for b in bs]
+        st, infos = P.ps_batch_solve(ms, bs, xs, P.make_opts(grid_spin_limit=150))
+        assert st == P.PS_OK
+        for k in (0, 1, 20, 47):
+            A = oracle.PressureMatrix.from_case(cases[k])
+            assert A.residual(cases[k].b, xs[k].cpu().numpy()) <= 1.05e-10
+    finally:
+        for m in ms:
+            P.ps_mesh_free(m)
