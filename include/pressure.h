@@ -131,11 +131,12 @@ typedef struct {
                              /* persistent engine on a batch of one, which gives    */
                              /* bitwise the result the mesh gets in any batch       */
     int32_t grid_spin_limit; /* diagnostic: polls of a wait between the running     */
-                             /* blocks of a batch's kernels before it gives up and  */
-                             /* the call returns PS_ETIMEOUT (batched, persistent   */
-                             /* and served solves; 0 = 2^26 polls).  Blocks that    */
-                             /* wait for others to finish an earlier mesh have the  */
-                             /* default limit and count from the last sign of life  */
+                             /* blocks of a kernel before it gives up and the call  */
+                             /* returns PS_ETIMEOUT (solves on chip, batched,       */
+                             /* persistent and served ones; 0 = 2^26 polls).  In a  */
+                             /* batch, blocks that wait for others to finish an     */
+                             /* earlier mesh have the default limit and count from  */
+                             /* the last sign of life                               */
     int32_t batch_threads;   /* batched / persistent / served solves, meshes too    */
                              /* large for the on-chip kernel: threads per block of  */
                              /* the persistent kernel (0 = 256, 128, 256)           */

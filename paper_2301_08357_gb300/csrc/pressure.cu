@@ -1138,6 +1138,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
     m->dev.dinv32 = dinv32;
     m->dev.dinv64 = dinv64;
     const int gi = o.graph_iters == 0 ? 32 : o.graph_iters;
+    const uint32_t spin = o.grid_spin_limit > 0 ? (uint32_t)o.grid_spin_limit : kGridSpinLimit;
     int rc = PS_OK;
     if (o.mode == PS_MODE_FP64) {
         const int max_restarts = o.max_outer > 0 ? o.max_outer : 40;
@@ -1149,7 +1150,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
             if (rr <= stop_abs2) { status = PS_OK; break; }
             if (used >= max_it || outer > max_restarts) { status = PS_ENOTCONV; break; }
             if (solo) {
-                if ((rc = solo_run<double>(m, 1.0, stop_abs2, max_it - used, true, s)) != PS_OK) break;
+                if ((rc = solo_run<double>(m, 1.0, stop_abs2, max_it - used, true, spin, s)) != PS_OK) break;
             } else {
                 Cg2Args<double> a = cg2_args<double>(m);
                 k_cg2_start<double><<<m->g3c, kBlock, 0, s>>>(m->dev, a, nullptr, 1.0, nullptr, stop_abs2, 0,
@@ -1185,7 +1186,7 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
             // needs (with a factor 10 of margin) when that is less
             const double it_k = inner_reduction(itol, tol, bb, rr);
             if (solo) {
-                rc = solo_run<float>(m, scale, it_k * it_k, max_it - used, m->dev.n_nodes > kFusedMaxNodes, s);
+                rc = solo_run<float>(m, scale, it_k * it_k, max_it - used, m->dev.n_nodes > kFusedMaxNodes, spin, s);
                 if (rc != PS_OK) break;
             } else if (fused) {
                 const CG1Vec v = cg1_vec(m);

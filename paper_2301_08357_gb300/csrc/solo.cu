@@ -805,7 +805,6 @@ static SoloArgs<T> solo_args(const ps_mesh *m, const Solo &S, void *part, uint4 
     A.x64 = m->ws.x64;
     A.relative = F32 ? 1 : 0;
     A.drop = F32 ? 1 : 0;
-    A.spin_limit = kGridSpinLimit;
     A.exch = exch;
     A.st = m->ws.st;
     A.err = m->ctx->d_err;
@@ -814,7 +813,8 @@ static SoloArgs<T> solo_args(const ps_mesh *m, const Solo &S, void *part, uint4 
 }
 
 template <typename T>
-int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, cudaStream_t s) {
+int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, uint32_t spin_limit,
+             cudaStream_t s) {
     constexpr bool F32 = sizeof(T) == 4;
     Solo &S = *m->solo;
     // tags of a run: tag + 1 .. tag + its iterations + 1 (never reused before
@@ -829,6 +829,7 @@ int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool na
     A.inv_scale = 1.0 / scale;
     A.tol2 = tol2;
     A.nan_breaks = nan_breaks ? 1 : 0;
+    A.spin_limit = spin_limit;
     A.max_iters = std::min(max_iters, (long long)0x20000000);
     A.tag0 = S.tag + 1;
     cudaLaunchConfig_t cfg;
@@ -847,8 +848,8 @@ int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool na
     m->launches += 1;
     return solo_rc(cudaLaunchKernelExC(&cfg, k, args));
 }
-template int solo_run<float>(ps_mesh *, double, double, long long, bool, cudaStream_t);
-template int solo_run<double>(ps_mesh *, double, double, long long, bool, cudaStream_t);
+template int solo_run<float>(ps_mesh *, double, double, long long, bool, uint32_t, cudaStream_t);
+template int solo_run<double>(ps_mesh *, double, double, long long, bool, uint32_t, cudaStream_t);
 
 // ---------------------------------------------------------------- batches
 int solo_batch_layout(ps_mesh *m, std::vector<DevAlloc> &owner, Solo **out) {

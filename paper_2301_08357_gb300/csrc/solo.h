@@ -62,9 +62,10 @@ int solo_plan_clear(BatchPlan &plan, cudaStream_t s);
 // One inner run from the residual r64 (times scale) in the mesh's workspace:
 // x64 += the correction found / scale; the CG state receives the iteration
 // count and status.  T = float: relative reduction tol2 of r.r; double: stop
-// at r.r <= tol2.
+// at r.r <= tol2.  spin_limit: polls of a wait (ps_solve_opts.grid_spin_limit).
 template <typename T>
-int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, cudaStream_t s);
+int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, uint32_t spin_limit,
+             cudaStream_t s);
 // After the run's state is on the host: iters of it (done) or no end (a wait
 // gave up).
 inline void solo_end(Solo &S, bool done, long long iters) { S.tag = done ? S.tag + (uint32_t)iters + 2u : 0u; }

@@ -70,3 +70,29 @@ def test_blocks_may_wait_for_busy_ones(env):
     finally:
         for m in ms:
             P.ps_mesh_free(m)
+
+
+@pytest.mark.parametrize("mode", [1, 0], ids=["mixed", "fp64"])
+@pytest.mark.parametrize("make", [lambda: S.make_c1(48), lambda: S.make_c2(12)], ids=["square", "cube"])
+def test_single_solve_reports_and_recovers(env, make, mode):
+    P, torch, ctx = env
+    c = make()
+    A = oracle.PressureMatrix.from_case(c)
+    m = _upload(P, ctx, c)
+    try:
+        b = torch.as_tensor(c.b, device="cuda")
+        x = torch.zeros_like(b)
+        P.ps_pressure_solve(m, b, x, P.make_opts(mode=mode))     # (words with tags of an earlier run)
+        with pytest.raises(P.PressureError) as e:
+            x.zero_()
+            P.ps_pressure_solve(m, b, x, P.make_opts(mode=mode, grid_spin_limit=1))
+        assert e.value.status == P.PS_ETIMEOUT
+        out = []
+        for _ in range(2):
+            x = torch.zeros_like(b)
+            st, info = P.ps_pressure_solve(m, b, x, P.make_opts(mode=mode))
+            assert st == P.PS_OK and A.residual(c.b, x.cpu().numpy()) <= 1.05e-10
+            out.append(x)
+        assert torch.equal(*out)
+    finally:
+        P.ps_mesh_free(m)
