@@ -1150,7 +1150,14 @@ int solve_internal(ps_mesh *m, const ps_solve_opts &o, ps_solve_info *info, cuda
             if (rr <= stop_abs2) { status = PS_OK; break; }
             if (used >= max_it || outer > max_restarts) { status = PS_ENOTCONV; break; }
             if (solo) {
-                if ((rc = solo_run<double>(m, 1.0, stop_abs2, max_it - used, true, spin, s)) != PS_OK) break;
+                // r scaled by a power of two to a norm near 1 (every number of the
+                // run is the same but for its exponent): the quotients are formed
+                // from products of two dot products, which would leave the range of
+                // a double for right-hand sides of 1e80 or 1e-80
+                int e = 0;
+                if (std::isfinite(rr)) std::frexp(std::sqrt(rr), &e);
+                rc = solo_run<double>(m, std::ldexp(1.0, -e), std::ldexp(stop_abs2, -2 * e), max_it - used, true, spin, s);
+                if (rc != PS_OK) break;
             } else {
                 Cg2Args<double> a = cg2_args<double>(m);
                 k_cg2_start<double><<<m->g3c, kBlock, 0, s>>>(m->dev, a, nullptr, 1.0, nullptr, stop_abs2, 0,
