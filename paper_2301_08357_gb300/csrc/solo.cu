@@ -122,30 +122,36 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t *p) {
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// A wait's budget: false once it has given up.  begin() before every wait (a
-// budget spent over a whole run ended healthy long runs, and after its first
-// 4,096 polls every later one slept).
-// queued: the first wait of a run in a batch, which lasts until thread blocks that
-// still run earlier meshes come to this one.  That may be many runs, so the wait
-// has the default limit, which starts anew with every sign of life (`beat`, 256
-// iterations or the end of any run), and ends at once when some other wait has given up.
-struct Spin {
-    uint32_t limit, polls = 0, seen = 0;
-    bool ok = true, queued = false;
-    __device__ __forceinline__ void begin(uint32_t l, bool q) {
-        limit = l;
-        polls = 0;
-        queued = q;
+// The first wait of a run in a batch lasts until thread blocks that still run
+// earlier meshes come to this one, which may be many runs: past the first polls
+// it is waited for here.  The polls are counted from the last sign of life of any
+// run (the beat), and the wait ends at once when some other wait has given up.
+__device__ __noinline__ bool solo_queue_wait(const uint2 *word, uint32_t tag, const uint32_t *beat, const int *err) {
+    uint32_t seen = ld_relaxed(beat);
+    for (uint32_t polls = 0; polls < kGridSpinLimit; ++polls) {
+        if (ld_tagged(word).y == tag) return true;
+        if (ld_relaxed(reinterpret_cast<const uint32_t *>(err))) return false;
+        const uint32_t now = ld_relaxed(beat);
+        if (now != seen) polls = 0;
+        seen = now;
+        __nanosleep(64);
     }
-    __device__ __forceinline__ bool again(const uint32_t *beat, const int *err) {
-        if (queued && (polls & 1023u) == 1023u) {
-            const uint32_t now = ld_relaxed(beat);
-            if (now != seen) polls = 0;
-            seen = now;
-            if (ld_relaxed(reinterpret_cast<const uint32_t *>(err))) ok = false;
-        }
+    return false;
+}
+// A wait's budget: false once it has given up.  The polls are set to 0 before
+// every wait (a budget spent over a whole run ended healthy long runs, and after
+// its first 4,096 polls every later one slept).
+struct Spin {
+    uint32_t polls = 0;
+    bool ok = true;
+    __device__ __forceinline__ bool again(uint32_t limit) {
         if (++polls >= limit) ok = false;
         if (polls > 4096u) __nanosleep(64);
+        return ok;
+    }
+    // in the first wait of a run in a batch
+    __device__ __forceinline__ bool again_queued(const uint2 *word, uint32_t tag, const uint32_t *beat, const int *err) {
+        if (++polls >= 1024u) ok = solo_queue_wait(word, tag, beat, err);
         return ok;
     }
 };
@@ -333,9 +339,9 @@ __device__ __forceinline__ typename Share<T>::type sum16(const typename Share<T>
 // (dependent FP64 operations), 3.5k the update, stars and node sums; 64^3: 4.5k
 // of 21k the stars (half their records stream from L2), 4.5k the node sums;
 // FP64 40^3: 14.6k the stars, at the FP64 pipe's rate.
-// bid, G: this block's number among the mesh's G blocks.  The run's end, or
-// kSoloRuns after a wait's limit.
-template <int D, typename T>
+// bid, G: this block's number among the mesh's G blocks.  BATCH: other runs share
+// the SMs.  The run's end, or kSoloRuns after a wait's limit.
+template <int D, typename T, bool BATCH>
 __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bid, const int G) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr bool F32 = sizeof(T) == 4;
@@ -406,10 +412,8 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
     Spin spin;
     for (int it = 0;; ++it) {
         const uint32_t tag = A.tag0 + (uint32_t)it;
-        // (an iteration's words are waited for together)
-        const bool queued = it == 0 && A.beat;
-        spin.begin(queued ? kGridSpinLimit : A.spin_limit, queued);
-        if (A.beat && (it & 255) == 255 && bid == 0 && tid == 0) atomicAdd(A.beat, 1u);
+        spin.polls = 0;   // (an iteration's words are waited for together)
+        if (BATCH && (it & 255) == 255 && bid == 0 && tid == 0) atomicAdd(A.beat, 1u);
         // ---- update
         const T al = s_alpha, be = s_beta;
 #pragma unroll 1
@@ -521,7 +525,13 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                     if (all) {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) w += Tagged<T>::of(f + k * kW);
-                    } else if (spin.again(A.beat, A.err)) {
+                    } else if (BATCH && it == 0) {
+                        int k = 0;   // the first that is not there
+#pragma unroll
+                        for (int j = 8 * kW - 1; j >= 0; --j)
+                            if (f[j].y != tag) k = j;
+                        if (spin.again_queued(part + k % kW * A.n_slots + k0 + k / kW, tag, A.beat, A.err)) k0 -= 8;
+                    } else if (spin.again(A.spin_limit)) {
                         k0 -= 8;
                     }
                 }
@@ -536,7 +546,11 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                 if (b < G) {
                     const uint4 *w = mine + q * G + b;
                     uint4 x = ld_pair(w);
-                    while ((x.y != tag || x.w != tag) && spin.again(A.beat, A.err)) x = ld_pair(w);
+                    while ((x.y != tag || x.w != tag) &&
+                           (BATCH && it == 0 ? spin.again_queued(reinterpret_cast<const uint2 *>(w) + (x.y == tag), tag,
+                                                                 A.beat, A.err)
+                                             : spin.again(A.spin_limit)))
+                        x = ld_pair(w);
                     v = Sh::from(x.x, x.z);
                 }
                 __syncwarp();
@@ -581,7 +595,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
 
 template <int D, typename T>
 __global__ void __launch_bounds__(512, 1) k_solo_cg(const __grid_constant__ SoloArgs<T> A) {
-    solo_run_block<D, T>(A, blockIdx.x, gridDim.x);
+    solo_run_block<D, T, false>(A, blockIdx.x, gridDim.x);
 }
 
 // The same for the meshes of a batch that are in their inner solve.  A thread
@@ -625,8 +639,8 @@ __global__ void __launch_bounds__(512, 1) k_solo_batch(const SoloJob *jobs, cons
         }
         __syncthreads();
         if (!s_run) continue;
-        const int end = J.dim == 3 ? solo_run_block<3, float>(J.A, me.y, J.G)
-                                   : solo_run_block<2, float>(J.A, me.y, J.G);
+        const int end = J.dim == 3 ? solo_run_block<3, float, true>(J.A, me.y, J.G)
+                                   : solo_run_block<2, float, true>(J.A, me.y, J.G);
         if (end == kSoloRuns) return;       // a wait gave up: the others' will, those for this thread block too
         if (me.y == 0 && threadIdx.x == 0) {
             BState *st = J.bst;
