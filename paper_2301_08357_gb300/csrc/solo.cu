@@ -287,12 +287,14 @@ struct SoloScalars {
         } else {
             iters += 1;
             const bool pos = __shfl_sync(0xffffffffu, positive(den) ? 1 : 0, 0) && positive(ra);
-            if (!Sh::finite(t[0]) || !Sh::finite(t[1]) || !Sh::finite(t[2]) || !pos) {
-                done = 1;
-                status = kCgBreakdown;
-            } else if (rho <= stop_rr) {
+            const bool fin = Sh::finite(t[0]) && Sh::finite(t[1]) && Sh::finite(t[2]);
+            // (before the quotient is looked at: a residual of 0 makes it 0 / 0)
+            if (fin && rho <= stop_rr) {
                 done = 1;
                 status = kCgConverged;
+            } else if (!fin || !pos) {
+                done = 1;
+                status = kCgBreakdown;
             } else if (iters >= A.max_iters) {
                 done = 1;
                 status = kCgMaxIter;

@@ -41,3 +41,22 @@ def test_size_of_the_right_hand_side(env, make, precond):
             assert it == out[0][1] and np.array_equal(x, out[0][0]), k
     finally:
         P.ps_mesh_free(m)
+
+
+def test_residual_that_reaches_zero(env):
+    """One free vertex, every number of the run exact: the residual is 0 after
+    one iteration, which is convergence (the next quotient would be 0 / 0)."""
+    P, torch, ctx = env
+    X = np.array([[0.0, 0.0], [1.0, 0.0], [0.0, 1.0]])
+    m = P.ps_mesh_upload(ctx, 2, X, np.array([[0, 1, 2]], np.int32), np.array([0, 1, 1], np.uint8))
+    try:
+        P.ps_coeff_set(m, np.full(3, 6.0), np.array([3.0]), 1.0)
+        P.ps_mesh_set_mass(m, P.PS_MASS_LUMPED)        # A = 6 / 6 + 3 = 4
+        b = torch.tensor([1.0, 0.0, 0.0], dtype=torch.float64, device="cuda")
+        for mode in (P.PS_MODE_FP64, P.PS_MODE_MIXED):
+            x = torch.zeros_like(b)
+            st, info = P.ps_pressure_solve(m, b, x, P.make_opts(mode=mode))
+            assert st == P.PS_OK, info.as_dict()
+            assert x.cpu().numpy().tolist() == [0.25, 0.0, 0.0] and info.iters_inner == 1
+    finally:
+        P.ps_mesh_free(m)
