@@ -631,6 +631,15 @@ int batch_plan_build(ps_ctx *ctx, ps_mesh *const *meshes, int n, int epoch_iters
     if (e != cudaSuccess) return cuda_rc(e);
     std::memset(plan.h_st, 0, (size_t)n * sizeof(BState));
     rc = solo_plan_build(plan, s);
+    if (rc == PS_ENOMEM) {
+        // no room for the words that blocks exchange (some 100 bytes per pair of a
+        // mesh's blocks): the meshes run chunk by chunk, which needs none
+        cudaGetLastError();
+        plan.launches.clear();
+        for (BMesh &B : plan.h_meshes) B.solo = nullptr;
+        plan.chunked = true;
+        rc = PS_OK;
+    }
     if (rc != PS_OK) return rc;
     plan.L32 = max_layout(plan.meshes, false);
     plan.L64 = max_layout(plan.meshes, true);
@@ -673,6 +682,9 @@ int batch_upload_states(BatchPlan &plan, cudaStream_t s) {
     // meshes carried over mid inner solve are counted as active
     int act = 0;
     for (int i = 0; i < n; ++i) act += plan.h_st[i].phase == kPhInner && !plan.h_st[i].in.done;
+    // (also when an earlier plan had no room to run the mesh on chip)
+    for (int i = 0; i < n; ++i)
+        plan.chunked = plan.chunked || (plan.h_st[i].phase >= kPhInnerInit && plan.h_st[i].phase <= kPhCorrect);
     plan.h_active = act;
     int *active = (int *)(plan_bar(plan) + 128);
     cudaError_t e = cudaMemcpyAsync(plan.d_meshes, plan.h_meshes.data(), n * sizeof(BMesh), cudaMemcpyHostToDevice, s);
