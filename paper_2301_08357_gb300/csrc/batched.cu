@@ -468,13 +468,18 @@ static int ensure_batch_ws(ps_mesh *m) {
     return PS_OK;
 }
 
-int64_t batch_ws_bytes(const ps_mesh *m) {
+int64_t solve_ws_bytes(const ps_mesh *m) {
     // vectors of ps_mesh::ws and BatchMeshWs (an estimate for admission):
     // FP64 x b r p q, FP32 x r p q (two buffers each), s (two), D^-1 copies
     // of the unpreconditioned mode, partial sums, per-chunk dots
     const int64_t np = m->dev.n_pad, sh = m->prep.sh_total;
-    // and the on-chip layout: ids, lists and exchanged words
-    return np * (5 * 8 + 12 * 4) + sh * 16 + (int64_t)m->dev.n_chunks * 48 + m->prep.patch_total * 64;
+    return np * (5 * 8 + 12 * 4) + sh * 16 + (int64_t)m->dev.n_chunks * 48;
+}
+
+int64_t batch_ws_bytes(const ps_mesh *m) {
+    // and, for a mesh of a size that gets a layout of its own in batches, that
+    // layout: ids, lists and exchanged words
+    return solve_ws_bytes(m) + (solo_batch_size(m) ? m->prep.patch_total * 64 : 0);
 }
 
 void batched_release_mesh(ps_mesh *m) {

@@ -328,8 +328,8 @@ extern "C" int ps_server_add_case(ps_server *s, ps_mesh *mesh, const double *x0,
     if (!mesh->coeff_ok) return PS_ESTATE;
     Case c;
     c.mesh = mesh;
-    c.ws_bytes = batch_ws_bytes(mesh);
     c.single = s->opts.single_nodes > 0 && mesh->prep.n_nodes >= (int64_t)s->opts.single_nodes;
+    c.ws_bytes = c.single ? solve_ws_bytes(mesh) : batch_ws_bytes(mesh);
     const size_t bytes = (size_t)mesh->prep.n_nodes * 8;
     {
         std::lock_guard<std::mutex> ctx_lk(s->ctx->mu);

@@ -868,11 +868,14 @@ template int solo_run<float>(ps_mesh *, double, double, long long, bool, uint32_
 template int solo_run<double>(ps_mesh *, double, double, long long, bool, uint32_t, cudaStream_t);
 
 // ---------------------------------------------------------------- batches
+bool solo_batch_size(const ps_mesh *m) {
+    return !solo_too_large(m) && m->prep.n_patches <= (int64_t)std::min(m->ctx->sms, kSoloMaxBlocks) * kSoloBatchStars;
+}
+
 int solo_batch_layout(ps_mesh *m, std::vector<DevAlloc> &owner, Solo **out) {
     *out = nullptr;
     if (solo_too_large(m)) return PS_OK;
-    const int64_t cap = std::min(m->ctx->sms, kSoloMaxBlocks);
-    if (m->prep.n_patches > cap * kSoloBatchStars) {
+    if (!solo_batch_size(m)) {
         // every SM either way: the layout of the mesh alone
         if (m->solo && m->solo->fp32 &&
             solo_resident(k_solo_batch, m->solo->threads, m->solo->sm32.total, m->ctx->sms) >= m->solo->n_blocks)

@@ -47,6 +47,8 @@ bool solo_ready(ps_mesh *m);
 // when that has the same blocks), or null: the mesh does not fit, the batch
 // runs it chunk by chunk.
 int solo_batch_layout(ps_mesh *m, std::vector<DevAlloc> &owner, Solo **out);
+// The mesh's size is one of those that get a layout of their own there.
+bool solo_batch_size(const ps_mesh *m);
 // One cooperative launch: its thread blocks run the meshes' blocks that are
 // theirs in the plan's list, one after another.
 struct SoloLaunch {
