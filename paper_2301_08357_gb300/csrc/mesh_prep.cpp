@@ -81,6 +81,10 @@ struct PatchRec {
     int elem[kPatchMax];   // chunk-local element index
 };
 
+// Vertices by rank in build_patches (2D); kept from chunk to chunk for its memory.
+constexpr int kRankCount = 16, kRankTouch = 32;
+using RankBuckets = std::array<std::vector<int>, kRankCount * kRankTouch>;
+
 // Group the elements of one chunk into star patches.  lc: [n][4] local vertex
 // ids; lx: [local node][dim] coordinates (3D only, may be null).  Pivots are
 // edges (3D) or vertices (2D); pivots are taken greedily by the number of
@@ -93,25 +97,34 @@ struct PatchRec {
 // share its main diagonal, the longest edge of the cell, so every cell
 // becomes one closed star of six.
 void build_patches(int dim, int n, const std::vector<std::array<int, 4>> &lc, std::vector<PatchRec> &out,
-                   const double *lx) {
+                   const double *lx, RankBuckets &bucket) {
     const int nv = dim + 1;
     out.clear();
     std::vector<char> used(n, 0);
     std::vector<std::pair<uint64_t, int>> inc;   // (pivot key, element)
-    inc.reserve((size_t)n * (dim == 3 ? 6 : 3));
-    for (int e = 0; e < n; ++e) {
-        if (dim == 3) {
+    int nloc = 0;
+    if (dim == 3) {
+        inc.reserve((size_t)n * 6);
+        for (int e = 0; e < n; ++e)
             for (int i = 0; i < 4; ++i)
                 for (int j = i + 1; j < 4; ++j) {
                     uint64_t u = (uint64_t)std::min(lc[e][i], lc[e][j]);
                     uint64_t v = (uint64_t)std::max(lc[e][i], lc[e][j]);
                     inc.push_back({(u << 20) | v, e});
                 }
-        } else {
-            for (int i = 0; i < 3; ++i) inc.push_back({(uint64_t)lc[e][i], e});
-        }
+        std::sort(inc.begin(), inc.end());
+    } else {
+        // (the keys are local vertices: sorted by counting)
+        for (int e = 0; e < n; ++e)
+            for (int i = 0; i < 3; ++i) nloc = std::max(nloc, lc[e][i] + 1);
+        std::vector<int> at(nloc + 1, 0);
+        for (int e = 0; e < n; ++e)
+            for (int i = 0; i < 3; ++i) at[lc[e][i] + 1]++;
+        for (int v = 0; v < nloc; ++v) at[v + 1] += at[v];
+        inc.resize((size_t)n * 3);
+        for (int e = 0; e < n; ++e)
+            for (int i = 0; i < 3; ++i) inc[at[lc[e][i]]++] = {(uint64_t)lc[e][i], e};
     }
-    std::sort(inc.begin(), inc.end());
     std::vector<size_t> gstart;
     for (size_t k = 0; k < inc.size(); ++k)
         if (k == 0 || inc[k].first != inc[k - 1].first) gstart.push_back(k);
@@ -139,6 +152,7 @@ void build_patches(int dim, int n, const std::vector<std::array<int, 4>> &lc, st
     }
     std::vector<int> cand;
     std::vector<std::array<int, 2>> rp;   // ring pair of each candidate
+    std::vector<char> taken;
     // the stars of pivot g if at least c elements around it are unassigned
     auto take = [&](size_t g, int c) {
         cand.clear();
@@ -164,7 +178,7 @@ void build_patches(int dim, int n, const std::vector<std::array<int, 4>> &lc, st
             }
             rp.push_back(r);
         }
-        std::vector<char> taken(cand.size(), 0);
+        taken.assign(cand.size(), 0);
         size_t left = cand.size();
         while (left > 0) {
             // start from a ring vertex of degree 1 among the remaining, if any
@@ -212,17 +226,16 @@ void build_patches(int dim, int n, const std::vector<std::array<int, 4>> &lc, st
         // of earlier stars first: the stars grow as a compact tiling and
         // leave few gaps (by key alone, every second vertex of every second row
         // is taken, and 301 x 301 squares have 2.7 triangles per star
-        // instead of 4.8, 5.4 with chunks of 1,536; preparation time is the
-        // same).  FP64 CG on 64 x 64 squares 1.29 -> 1.23 ms.
+        // instead of 4.8, 5.4 with chunks of 1,536).  FP64 CG on 64 x 64
+        // squares 1.29 -> 1.23 ms.  Preparing 301 x 301 squares: 69 ms by key
+        // alone, 88 ranked, 45 with the counting sort above and buckets that
+        // keep their memory.
         // Buckets by (unassigned elements, touched ring vertices, counted once
         // per element); a vertex is entered again whenever its bucket changes.
-        constexpr int kC = 16, kT = 32;
-        int nloc = 0;
-        for (int e = 0; e < n; ++e)
-            for (int i = 0; i < 3; ++i) nloc = std::max(nloc, lc[e][i] + 1);
+        constexpr int kC = kRankCount, kT = kRankTouch;
         std::vector<int> group(nloc, -1), count(nloc, 0), touch(nloc, 0);
         std::vector<char> touched(nloc, 0);
-        std::vector<std::vector<int>> bucket(kC * kT);
+        for (auto &b : bucket) b.clear();
         auto slot = [&](int v) { return std::min(count[v], kC - 1) * kT + std::min(touch[v], kT - 1); };
         for (size_t g = ng; g-- > 0;) {
             const int v = (int)inc[gstart[g]].first;
@@ -536,6 +549,7 @@ std::string prepare_mesh(int dim, int64_t n_nodes, const double *coords, int64_t
     std::vector<int32_t> shr_cnt(m.n_shared + 1, 0);
     std::vector<std::array<int, 4>> lc;
     std::vector<PatchRec> patches;
+    RankBuckets ranks;
     std::vector<double> lxyz;                        // the chunk's local node coordinates (3D)
     for (int c = 0; c < nc; ++c) {
         ChunkDesc &cd = m.chunks[c];
@@ -583,7 +597,7 @@ std::string prepare_mesh(int dim, int64_t n_nodes, const double *coords, int64_t
                 for (int k = 0; k < 3; ++k) lxyz[(size_t)l * 3 + k] = coords[(int64_t)vtx * 3 + k];
             }
         }
-        build_patches(dim, n_el, lc, patches, dim == 3 ? lxyz.data() : nullptr);
+        build_patches(dim, n_el, lc, patches, dim == 3 ? lxyz.data() : nullptr, ranks);
         balance_patches(patches);
         const int np = (int)patches.size();
         if (np > kMaxChunkPatches) return "internal: too many patches in a chunk";
