@@ -85,6 +85,7 @@ struct SoloArgs {
     int relative, nan_breaks;
     int drop;                   // 1: a breakdown leaves x64 alone, 0: it keeps the last iterate
     uint32_t spin_limit;        // polls of a wait before it gives up
+    uint32_t nap;               // ns before an iteration's first poll (solo_nap)
     uint32_t *beat;             // in a batch: counts its runs' iterations by 256 and their ends (null: a run alone)
     long long max_iters;
     uint4 *exch;                // [2 buffers][reader][3 products][writer], two tagged words each
@@ -176,11 +177,20 @@ template <> struct Tagged<double> {
 };
 
 // A dot product's share: a float pair (unevaluated sum) for FP32 vectors, a
-// double for FP64 ones; two words either way.  FP64 additions cost an SM 16
-// cycles per warp, so pairs stay in FP32 until the totals.
+// double for FP64 ones; two words either way.  Inside a warp pairs are added as
+// pairs; above it, where the rounding of a single addition still shows in the
+// total, as three floats (Wide), which lose nothing that a double would keep.
+// FP64 additions there were slower (a warp's takes its SM sub-partition 64
+// cycles: 301 x 301 squares 10% per solve).  Relative error of a total against
+// exact sums, rms over random vectors of 4,225 to 274,625 nodes: pairs
+// throughout 1.6e-15 to 2.4e-15, the fused pass of cg1.cuh 5.1e-16 to 8.0e-16,
+// this 3.2e-16 to 4.3e-16.
 template <typename T> struct Share;
 template <> struct Share<float> {
     using type = float2;
+    struct Wide {
+        float hi, lo, t;
+    };
     static __device__ __forceinline__ float2 zero() { return make_float2(0.f, 0.f); }
     static __device__ __forceinline__ float2 add(float2 a, float2 b) {
         DotF t;
@@ -193,34 +203,55 @@ template <> struct Share<float> {
     static __device__ __forceinline__ float2 shfl(float2 a, int o) {
         return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
     }
-    static __device__ __forceinline__ float2 bcast(float2 a, int l) {
-        return make_float2(__shfl_sync(0xffffffffu, a.x, l), __shfl_sync(0xffffffffu, a.y, l));
-    }
-    static __device__ __forceinline__ uint2 bits(float2 a) { return make_uint2(__float_as_uint(a.x), __float_as_uint(a.y)); }
     static __device__ __forceinline__ float2 from(uint32_t x, uint32_t y) {
         return make_float2(__uint_as_float(x), __uint_as_float(y));
     }
-    static __device__ __forceinline__ double total(float2 a) { return (double)a.x + (double)a.y; }
-    static __device__ __forceinline__ bool finite(float2 a) { return isfinite(a.x) && isfinite(a.y); }
+    static __device__ __forceinline__ Wide wide(float2 a) { return {a.x, a.y, 0.f}; }
+    // s + e = a + b exactly (Knuth's TwoSum)
+    static __device__ __forceinline__ float two_sum(float a, float b, float &e) {
+        const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+        e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+        return s;
+    }
+    static __device__ __forceinline__ Wide add(Wide a, Wide b) {
+        float e, f, g;
+        Wide o;
+        o.hi = two_sum(a.hi, b.hi, e);
+        const float u = two_sum(a.lo, b.lo, f);
+        o.lo = two_sum(u, e, g);
+        o.t = __fadd_rn(__fadd_rn(a.t, b.t), __fadd_rn(f, g));
+        return o;
+    }
+    static __device__ __forceinline__ Wide shfl(Wide a, int o) {
+        return {__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o),
+                __shfl_xor_sync(0xffffffffu, a.t, o)};
+    }
+    static __device__ __forceinline__ uint2 bits(Wide a) {
+        // hi + lo renormalised (|lo| is far below |hi|), then t into the rest
+        const float s = __fadd_rn(a.hi, a.lo), r = __fsub_rn(a.lo, __fsub_rn(s, a.hi));
+        return make_uint2(__float_as_uint(s), __float_as_uint(__fadd_rn(r, a.t)));
+    }
+    static __device__ __forceinline__ double total(Wide a) { return (double)a.hi + ((double)a.lo + (double)a.t); }
 };
 template <> struct Share<double> {
     using type = double;
+    using Wide = double;
     static __device__ __forceinline__ double zero() { return 0.0; }
     static __device__ __forceinline__ double add(double a, double b) { return a + b; }
     static __device__ __forceinline__ double of(const DotD &a) { return a.v; }
     static __device__ __forceinline__ double shfl(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-    static __device__ __forceinline__ double bcast(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+    static __device__ __forceinline__ double wide(double a) { return a; }
     static __device__ __forceinline__ uint2 bits(double a) {
         return make_uint2((uint32_t)__double2loint(a), (uint32_t)__double2hiint(a));
     }
     static __device__ __forceinline__ double from(uint32_t x, uint32_t y) { return __hiloint2double((int)y, (int)x); }
     static __device__ __forceinline__ double total(double a) { return a; }
-    static __device__ __forceinline__ bool finite(double a) { return isfinite(a); }
 };
-template <typename T>
-__device__ __forceinline__ typename Share<T>::type warp_share(typename Share<T>::type v) {
+// Sum of each group of N lanes, in all of them.
+template <typename T, int N>
+__device__ __forceinline__ typename Share<T>::Wide sum_lanes(typename Share<T>::Wide v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = Share<T>::add(v, Share<T>::shfl(v, o));
+    for (int o = N / 2; o > 0; o >>= 1) v = Share<T>::add(v, Share<T>::shfl(v, o));
     return v;
 }
 // Three warp sums at once: after two exchanges each lane carries one product
@@ -240,6 +271,7 @@ __device__ __forceinline__ typename Share<T>::type warp_share3(typename Share<T>
     for (int o = 4; o > 0; o >>= 1) v = Sh::add(v, Sh::shfl(v, o));
     return v;
 }
+__device__ __forceinline__ bool finite(double v) { return (__double2hiint(v) & 0x7fffffff) < 0x7ff00000; }
 // Positive (not 0, not NaN), from the sign and exponent word.
 __device__ __forceinline__ bool positive(double v) {
     const int h = __double2hiint(v);
@@ -257,15 +289,13 @@ __device__ __forceinline__ double fma_rn(double a, double b, double c) { return 
 // block from the same totals.
 template <typename T>
 struct SoloScalars {
-    using Sh = Share<T>;
     double rz = 0.0, ra = 0.0, rr0 = 0.0, stop_rr = 0.0;   // gamma; gamma * alpha
     long long iters = 0;
     int status = kCgRunning;
-    // t: gamma, delta, rho of iteration `it` in every lane.  quot: alpha in
+    // g, d, rho: gamma, delta, rho of iteration `it` in every lane.  quot: alpha in
     // lane 0, beta in lane 1.  Returns 1 if the run ends.
-    __device__ __forceinline__ int advance(const SoloArgs<T> &A, int bid, int it, const typename Sh::type (&t)[3],
-                                           int lane, double &quot) {
-        const double g = Sh::total(t[0]), d = Sh::total(t[1]), rho = Sh::total(t[2]);
+    __device__ __forceinline__ int advance(const SoloArgs<T> &A, int bid, int it, double g, double d, double rho, int lane,
+                                           double &quot) {
         int done = 0;
         // alpha' = g / (d - beta g / alpha) = g (rz alpha) / (d (rz alpha) - g g), beta = g / rz
         const double num = it == 0 || lane == 1 ? g : g * ra;
@@ -274,20 +304,20 @@ struct SoloScalars {
         if (it == 0) {
             rr0 = rho;
             stop_rr = A.relative ? A.tol2 * rho : A.tol2;
-            if (A.nan_breaks && !Sh::finite(t[2])) {
+            if (A.nan_breaks && !finite(rho)) {
                 done = 1;
                 status = kCgBreakdown;
             } else if (!(rho > 0.0) || (!A.relative && rho <= stop_rr)) {
                 done = 1;
                 status = kCgConverged;
-            } else if (!positive(d) || !Sh::finite(t[0]) || !Sh::finite(t[1])) {
+            } else if (!positive(d) || !finite(g) || !finite(d)) {
                 done = 1;
                 status = kCgBreakdown;
             }
         } else {
             iters += 1;
             const bool pos = __shfl_sync(0xffffffffu, positive(den) ? 1 : 0, 0) && positive(ra);
-            const bool fin = Sh::finite(t[0]) && Sh::finite(t[1]) && Sh::finite(t[2]);
+            const bool fin = finite(g) && finite(d) && finite(rho);
             // (before the quotient is looked at: a residual of 0 makes it 0 / 0)
             if (fin && rho <= stop_rr) {
                 done = 1;
@@ -309,38 +339,38 @@ struct SoloScalars {
         }
         return done;
     }
-    __device__ __forceinline__ void next(const typename Sh::type (&t)[3], double quot) {
-        rz = Sh::total(t[0]);
+    __device__ __forceinline__ void next(double g, double quot) {
+        rz = g;
         ra = rz * __shfl_sync(0xffffffffu, quot, 0);
     }
 };
 // What a finished run tells the blocks.
 enum SoloEnd : int { kSoloRuns = 0, kSoloKeep = 1, kSoloDrop = 2 };
 
-// Sum of a block's (up to) 16 warp sums in a fixed order.
+// The block's three sums from its (up to) 16 warp sums, by one warp: product q
+// in lanes 8 q .. 8 q + 7 (0 in the last eight).
 template <typename T>
-__device__ __forceinline__ typename Share<T>::type sum16(const typename Share<T>::type *v) {
+__device__ __forceinline__ typename Share<T>::Wide block_shares(const typename Share<T>::type (*red)[16], int nw,
+                                                                int lane) {
     using Sh = Share<T>;
-    typename Sh::type a[4] = {v[0], v[1], v[2], v[3]};
-#pragma unroll 1
-    for (int w = 4; w < 16; w += 4)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) a[k] = Sh::add(a[k], v[w + k]);
-    return Sh::add(Sh::add(a[0], a[1]), Sh::add(a[2], a[3]));
+    const int q = lane >> 3, k = lane & 7;
+    typename Sh::Wide v = Sh::wide(q < 3 ? red[q][k] : Sh::zero());
+    if (nw > 8) v = Sh::add(v, Sh::wide(q < 3 ? red[q][k + 8] : Sh::zero()));
+    return sum_lanes<T, 8>(v);
 }
 
 // The loop of the kernel below is kept small on purpose (no unrolling, one copy
 // of the star arithmetic): each of its phases runs once per iteration, and
 // with 40 KB of loop the instruction fetches took longer than the phases
 // (301 x 301 squares: 15k cycles per iteration).
-// Measured per iteration, with the kernels it replaces: 301 x 301 squares 5.8 us
-// (fused pass 16), 64^3 Kuhn 10.2 (operator, update and halo kernels 28), FP64
-// 64 x 64 squares 9.8 (25), FP64 40^3 24 (68).  Bound, 301 x 301 squares: 5.4k of
-// 11.9k cycles are the exchange (a word from one SM's store to another's poll
-// takes 1.7 us on this part, the rest overlaps or adds sums), 3.1k the scalars
-// (dependent FP64 operations), 3.5k the update, stars and node sums; 64^3: 4.5k
-// of 21k the stars (half their records stream from L2), 4.5k the node sums;
-// FP64 40^3: 14.6k the stars, at the FP64 pipe's rate.
+// Measured per iteration, with the kernels it replaces: 301 x 301 squares 4.3 us
+// (fused pass 16), 64^3 Kuhn 9.8 (operator, update and halo kernels 25), FP64
+// 64 x 64 squares 7.7 (25), FP64 40^3 17 (68).  Bound (cycles of an iteration's
+// phases): 301 x 301 squares 3.7k the update, stars and node sums, 2 to 3k the
+// scalars (dependent FP64 operations), the rest the exchange (a word from one
+// SM's store to another's poll takes 1.7 us on this part); 64^3: 4.6k the stars
+// (half their records stream from L2), 4.5k the node sums, 6k the exchange; FP64
+// 40^3: 15k of 37k the stars, at the FP64 pipe's rate.
 // bid, G: this block's number among the mesh's G blocks.  BATCH: other runs share
 // the SMs.  The run's end, or kSoloRuns after a wait's limit.
 template <int D, typename T, bool BATCH>
@@ -361,11 +391,12 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
     using Sh = Share<T>;
     using ST = typename Sh::type;
     __shared__ ST s_red[3][16];   // warps' sums; entries past the last warp stay 0
-    __shared__ ST s_seg[3][kSoloMaxBlocks / 32];
+    __shared__ typename Sh::Wide s_sum[3][BATCH ? kSoloMaxBlocks / 32 : 1];   // parts of the products' sums
     __shared__ T s_alpha, s_beta;
     __shared__ int s_end;
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = NT >> 5;
     const int n_seg = (G + 31) / 32;
+    const int ns = F32 ? nw : 4;   // warps that send the block's shares
     const SoloBlock B = A.blocks[bid];
     const int n_sh = B.n_loc - B.n_int;
     // ---- the block's part of the mesh and of the residual
@@ -493,16 +524,23 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
             if ((lane & 7) == 0 && lane < 24) s_red[lane >> 3][wid] = v;
         }
         __syncthreads();
-        if (G > 1) {
+        if (wid < ns) {
             // every block's share to every block: a reader's words lie
-            // together and have no other reader
-            uint4 *exch = A.exch + (size_t)(it & 1) * 3 * G * G;
+            // together and have no other reader (each warp forms the sums)
+            const typename Sh::Wide t = block_shares<T>(s_red, nw, lane);
+            const int q = lane >> 3, k = lane & 7;
+            if (G == 1) {
+                if (tid < 24 && k == 0) s_sum[q][0] = t;
+            } else if (q < 3) {
+                uint4 *exch = A.exch + (size_t)(it & 1) * 3 * G * G + q * G + bid;
+                const uint2 b = Sh::bits(t);
 #pragma unroll 1
-            for (int t = tid; t < 3 * G; t += NT) {
-                const int dst = t / 3, q = t - 3 * dst;
-                const uint2 b = Sh::bits(sum16<T>(s_red[q]));
-                st_pair(exch + (size_t)(3 * dst + q) * G + bid, b.x, b.y, tag);
+                for (int dst = wid * 8 + k; dst < G; dst += 8 * ns) st_pair(exch + (size_t)3 * dst * G, b.x, b.y, tag);
             }
+            __syncwarp();
+        }
+        if (G > 1) {
+            if (F32 && !BATCH && it > 0) __nanosleep(A.nap);
             // the shared unknowns' partials, which travel beside the shares
 #pragma unroll 1
             for (int j = tid; j < n_sh; j += NT) {
@@ -540,44 +578,80 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                 const T mr = sm[l];
                 sw[l] = is_dirichlet(mr) ? T(0) : fma_rn(mr, val[l], w);
             }
-            const uint4 *mine = exch + (size_t)3 * bid * G;
+            if constexpr (BATCH) {
+                // the blocks' shares, 32 of a product to a warp at a time (one
+                // warp per product, as below, took the batch 3% longer)
+                const uint4 *mine = A.exch + ((size_t)(it & 1) * 3 * G + 3 * bid) * G;
 #pragma unroll 1
-            for (int sg = wid; sg < 3 * n_seg; sg += nw) {
-                const int q = sg / n_seg, b = (sg - q * n_seg) * 32 + lane;
-                ST v = Sh::zero();
-                if (b < G) {
-                    const uint4 *w = mine + q * G + b;
-                    uint4 x = ld_pair(w);
-                    while ((x.y != tag || x.w != tag) &&
-                           (BATCH && it == 0 ? spin.again_queued(reinterpret_cast<const uint2 *>(w) + (x.y == tag), tag,
-                                                                 A.beat, A.err)
-                                             : spin.again(A.spin_limit)))
-                        x = ld_pair(w);
-                    v = Sh::from(x.x, x.z);
+                for (int sg = wid; sg < 3 * n_seg; sg += nw) {
+                    const int q = sg / n_seg, b = (sg - q * n_seg) * 32 + lane;
+                    ST v = Sh::zero();
+                    if (b < G) {
+                        const uint4 *w = mine + q * G + b;
+                        uint4 x = ld_pair(w);
+                        while ((x.y != tag || x.w != tag) &&
+                               (it == 0 ? spin.again_queued(reinterpret_cast<const uint2 *>(w) + (x.y == tag), tag, A.beat,
+                                                            A.err)
+                                        : spin.again(A.spin_limit)))
+                            x = ld_pair(w);
+                        v = Sh::from(x.x, x.z);
+                    }
+                    __syncwarp();
+                    v = Sh::add(v, Sh::shfl(v, 16));
+                    v = Sh::add(v, Sh::shfl(v, 8));
+                    const typename Sh::Wide t = sum_lanes<T, 8>(Sh::wide(v));
+                    if (lane == 0) s_sum[q][sg - q * n_seg] = t;
+                }
+            } else if (wid < 3) {
+                // the blocks' shares, one warp per product: a lane has up to five of
+                // them in flight, re-reads those not there yet and adds them in order
+                constexpr int kSeg = kSoloMaxBlocks / 32;
+                const uint4 *mine = A.exch + ((size_t)(it & 1) * 3 * G + 3 * bid + wid) * G + lane;
+                uint4 x[kSeg];
+#pragma unroll
+                for (int k = 0; k < kSeg; ++k) x[k].y = x[k].w = 32 * k + lane < G ? ~tag : tag, x[k].x = x[k].z = 0u;
+                for (;;) {
+                    bool all = true;
+#pragma unroll
+                    for (int k = 0; k < kSeg; ++k)
+                        if (x[k].y != tag || x[k].w != tag) x[k] = ld_pair(mine + 32 * k);
+#pragma unroll
+                    for (int k = 0; k < kSeg; ++k)
+                        all = all && x[k].y == tag && x[k].w == tag;
+                    if (all || !spin.again(A.spin_limit)) break;
                 }
                 __syncwarp();
-                v = warp_share<T>(v);
-                if (lane == 0) s_seg[q][sg - q * n_seg] = v;
+                static_assert(kSeg == 5, "the sum below");
+                ST v = Sh::add(Sh::add(Sh::from(x[0].x, x[0].z), Sh::from(x[1].x, x[1].z)),
+                               Sh::add(Sh::from(x[2].x, x[2].z), Sh::from(x[3].x, x[3].z)));
+                v = Sh::add(v, Sh::from(x[4].x, x[4].z));
+                v = Sh::add(v, Sh::shfl(v, 16));
+                const typename Sh::Wide t = sum_lanes<T, 16>(Sh::wide(v));
+                if (lane == 0) s_sum[wid][0] = t;
             }
-        } else if (tid < 3) {
-            s_seg[tid][0] = sum16<T>(s_red[tid]);
         }
         __syncthreads();
         if (wid == 0) {
-            // lane 8 q + k: segment k of product q
-            const int q = lane >> 3, k = lane & 7;
-            ST v = q < 3 && k < n_seg ? s_seg[q][k] : Sh::zero();
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) v = Sh::add(v, Sh::shfl(v, o));
-            const ST t[3] = {Sh::bcast(v, 0), Sh::bcast(v, 8), Sh::bcast(v, 16)};
+            // lane 8 q + k: part k of product q
+            typename Sh::Wide w = Sh::wide(Sh::zero());
+            if constexpr (BATCH) {   // lane 8 q + k: part k of product q
+                const int q = lane >> 3, k = lane & 7;
+                if (q < 3 && k < n_seg) w = s_sum[q][k];
+                w = sum_lanes<T, 8>(w);
+            } else {
+                w = s_sum[min(lane >> 3, 2)][0];
+            }
+            const double v = Sh::total(w);
+            const double g = __shfl_sync(0xffffffffu, v, 0), d = __shfl_sync(0xffffffffu, v, 8),
+                         rho = __shfl_sync(0xffffffffu, v, 16);
             double quot;
-            const int done = sc.advance(A, bid, it, t, lane, quot);
+            const int done = sc.advance(A, bid, it, g, d, rho, lane, quot);
             if (lane == 0) {
                 s_alpha = (T)quot;
                 s_end = !done ? kSoloRuns : sc.status == kCgBreakdown && A.drop ? kSoloDrop : kSoloKeep;
             }
             if (lane == 1 && it > 0) s_beta = (T)quot;
-            sc.next(t, quot);
+            sc.next(g, quot);
         }
         const bool ok = __syncthreads_and(spin.ok) != 0;
         if (!ok) {
@@ -707,6 +781,7 @@ static Solo *solo_sizes(const ps_mesh *m, int stars, SoloPrep &sp) {
     Solo *S = new Solo();
     S->n_blocks = (int)sp.blocks.size();
     S->n_slots = sp.n_slots;
+    S->max_star = sp.max_star;
     S->sm32 = solo_smem(sp, 4);
     S->sm64 = solo_smem(sp, 8);
     S->threads = sp.max_star <= 128 ? 128 : sp.max_star <= 256 ? 256 : 512;
@@ -828,6 +903,19 @@ static SoloArgs<T> solo_args(const ps_mesh *m, const Solo &S, void *part, uint4 
     return A;
 }
 
+// Time between a block's stores and its first poll, in FP32 runs alone on the
+// GPU.  A word that is polled before it has arrived comes about 2 us later than
+// one that is not (its line is then held where the poll went), so the first poll
+// waits as long as the words of this size of mesh take.  Iterations in us
+// without / with this wait, and of the code before it: 20^3 Kuhn 5.5 / 4.1, 5.1;
+// 28^3 5.9 / 5.3, 5.5; 181 x 181 squares 5.9 / 4.1, 5.1; 301 x 301 5.2 (550 ns:
+// 5.7) / 4.4, 5.4; 48 x 48 5.1 (550 ns: 4.7) / 3.8, 3.5.  FP64 runs, whose
+// blocks reach the poll later, are up to 3% slower with any.
+static uint32_t solo_nap(const Solo &S, int dim) {
+    if (S.n_blocks <= 24) return 400;
+    return S.max_star > (dim == 2 ? 128 : 640) ? 250 : 550;
+}
+
 template <typename T>
 int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool nan_breaks, uint32_t spin_limit,
              cudaStream_t s) {
@@ -846,6 +934,7 @@ int solo_run(ps_mesh *m, double scale, double tol2, long long max_iters, bool na
     A.tol2 = tol2;
     A.nan_breaks = nan_breaks ? 1 : 0;
     A.spin_limit = spin_limit;
+    A.nap = solo_nap(S, m->dev.dim);
     A.max_iters = std::min(max_iters, (long long)0x20000000);
     A.tag0 = S.tag + 1;
     cudaLaunchConfig_t cfg;
