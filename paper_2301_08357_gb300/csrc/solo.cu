@@ -781,7 +781,7 @@ static Solo *solo_sizes(const ps_mesh *m, int stars, SoloPrep &sp) {
     Solo *S = new Solo();
     S->n_blocks = (int)sp.blocks.size();
     S->n_slots = sp.n_slots;
-    S->max_star = sp.max_star;
+    S->mean_star = (int)(m->prep.n_patches / std::max(1, S->n_blocks));
     S->sm32 = solo_smem(sp, 4);
     S->sm64 = solo_smem(sp, 8);
     S->threads = sp.max_star <= 128 ? 128 : sp.max_star <= 256 ? 256 : 512;
@@ -904,16 +904,16 @@ static SoloArgs<T> solo_args(const ps_mesh *m, const Solo &S, void *part, uint4 
 }
 
 // Time between a block's stores and its first poll, in FP32 runs alone on the
-// GPU.  A word that is polled before it has arrived comes about 2 us later than
-// one that is not (its line is then held where the poll went), so the first poll
-// waits as long as the words of this size of mesh take.  Iterations in us
-// without / with this wait, and of the code before it: 20^3 Kuhn 5.5 / 4.1, 5.1;
-// 28^3 5.9 / 5.3, 5.5; 181 x 181 squares 5.9 / 4.1, 5.1; 301 x 301 5.2 (550 ns:
-// 5.7) / 4.4, 5.4; 48 x 48 5.1 (550 ns: 4.7) / 3.8, 3.5.  FP64 runs, whose
-// blocks reach the poll later, are up to 3% slower with any.
+// GPU.  A word that is polled before it has arrived was seen about 2 us later than
+// one that is not, so the first poll waits as long as the words of this size of
+// mesh take.  Iterations in us without / with this wait, and of the code before
+// it: 20^3 Kuhn 5.5 / 4.1, 5.1; 28^3 5.9 / 5.3, 5.5; 181 x 181 squares 5.9 / 4.1,
+// 5.1; 301 x 301 5.2 (550 ns: 5.7) / 4.3, 5.4; 50^3 6.9 (550 ns: 7.1) / 6.7, 7.0;
+// 48 x 48 5.1 (550 ns: 4.7) / 3.5, 3.5.  FP64 runs, whose blocks reach the poll
+// later, are up to 3% slower with any.
 static uint32_t solo_nap(const Solo &S, int dim) {
     if (S.n_blocks <= 24) return 400;
-    return S.max_star > (dim == 2 ? 128 : 640) ? 250 : 550;
+    return S.mean_star > (dim == 2 ? 150 : 640) ? 250 : 550;
 }
 
 template <typename T>

@@ -19,7 +19,7 @@ struct SoloSmem {
 
 // Device copy, owned by the mesh (null: the mesh does not fit).
 struct Solo {
-    int n_blocks = 0, n_slots = 0, max_star = 0;
+    int n_blocks = 0, n_slots = 0, mean_star = 0;
     int threads = 0;               // FP32 kernels (the FP64 one: at most 256)
     SoloBlock *blocks = nullptr;
     uint4 *ids4 = nullptr;
