@@ -233,7 +233,7 @@ int launch_pass(ps_mesh *m, const VecArgs<T> &a, cudaStream_t s) {
         k_chunks<3, T, MODE><<<m->dev.n_chunks, kBlock, L.total, s>>>(m->dev, a);
     CK(cudaGetLastError());
     // Kernel 2's launch overlaps kernel 1 (apply 45^3 FP32: 12.3 -> 10.3 us per
-    // call of a loop, 8.6 -> 7.9 in a graph; general-EOS step 181^2 2.37 -> 2.24 ms).
+    // call of a loop, 8.6 -> 7.9 in a graph).
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(m->grid2);
@@ -886,9 +886,8 @@ static cudaError_t reset_shares(ps_mesh *m, cudaStream_t s) {
     return cudaMemsetAsync(m->ws.pqu, 0xff, ((size_t)m->dev.n_chunks + 8) * sizeof(float2), s);
 }
 
-// FP32 operator kernel of the two-kernel iteration.  (Measured on 64^3..160^3:
-// 512-thread blocks, with or without a register cap for 3 blocks per SM, are
-// 15-55% slower than 256-thread blocks capped at 64 registers.)
+// FP32 operator kernel of the two-kernel iteration (block sizes: see
+// kStarThreads).
 static void launch_k1_f32(ps_mesh *m, const Cg2Args<float> &a, cudaStream_t s) {
     const MeshDev &d = m->dev;
     if (m->use_halo) {
@@ -1074,6 +1073,12 @@ static int check_dev_err(ps_ctx *c) {
     return PS_OK;
 }
 
+// PS_ENGINE_AUTO where a mixed solve cannot run on chip (regular meshes of this
+// size only when the context has no room for its workspace): the fused pass up
+// to here, the two-kernel iteration above.  Per iteration, fused / two-kernel, in
+// us: 2D 4,225 nodes 11.8 / 16.3, 91,204 15.7 / 17.2, 251,001 17.0 / 18.4,
+// 491,401 26.8 / 26.1; 3D 35,937 20.6 / 18.4, 97,336 16.5 / 18.0, 148,877 24.4 /
+// 20.6, 274,625 33.9 / 25.4.
 static constexpr int64_t kFusedMaxNodes = 200000;
 
 }  // namespace ps
