@@ -51,7 +51,10 @@ UNIT = "DOF-iter/s"
 # stands, keyed by (kernel, workload), with the capture it came from.  An
 # entry is removed whenever the kernel changes; missing means not captured
 # (the line then reports null).
-TRAFFIC = {}
+TRAFFIC = {
+    ("k_cg2_stars<384,3>", "c3_3d_kuhn_160^3_stiff_warm_tets24576000_nodes4173281"): {
+        "bytes": 586_630_000, "source": "profiles/launches_c3_kuhn160.md"},
+}
 
 
 def parse():
@@ -70,7 +73,7 @@ def parse():
                     help="c1/c2/c3: warm-up and timed solves alone (no e2e pass, no kernel timing, no CPU "
                          "baseline), for a profiler's launch list; the line then has no roofline or e2e")
     ap.add_argument("--chunk", type=int, default=0, help="elements per chunk (0 = library default)")
-    ap.add_argument("--pipeline", type=int, default=0, help="persistent double-buffered operator kernel")
+    ap.add_argument("--pipeline", type=int, default=0, help="no effect (accepted for old command lines)")
     ap.add_argument("--operator-kernel", type=int, default=0,
                     help="FP32 CG operator kernel of 3D meshes: 0 auto, 1 gathered shared nodes, 2 staged records with a halo")
     ap.add_argument("--operator-threads", type=int, default=0, help="threads per block of operator kernel 2")
@@ -288,13 +291,25 @@ def run_reference(args):
 
 # FP64 peak of the part: 152 SMs x 2 DFMA per clock x 2 flops x 2.07 GHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
+FP64_PEAK_TOPS = FP64_PEAK_TFLOPS / 2      # instructions: additions take the pipe as long as FMAs
+
+
+def fp64_star_ops(stats, cg):
+    """FP64 instructions of one operator pass over star patches, counted for
+    stars of six elements (a mesh's stars hold six at most, and fewer elements
+    per star need more): per edge one difference and two FMAs (3D: 19 edges for
+    six tetrahedra, 2D: 12 for six triangles), per star one addition for each of
+    its nodes (8; 7), per node 3 (row-sum term, residual, its dot) or 4 (CG
+    direction and p.Ap)."""
+    per_star = 3 * 19 + 8 if stats.dim == 3 else 3 * 12 + 7
+    return per_star * stats.n_elems / 6 + (4 if cg else 3) * stats.n_nodes
 
 
 def fp64_flops(stats, lumped, cg):
-    """Algorithmic FP64 flops of one FP64 operator pass element by element, with
-    precomputed element geometry (the passes over star patches do about a
-    quarter of them, so a fraction of the FP64 peak above 1 is possible; an FMA
-    counts 2): per element the stiffness differences
+    """FP64 flops of one operator pass done element by element with precomputed
+    element geometry, for an effective rate (the passes over star patches do
+    about a quarter of them; an FMA counts 2): per element the stiffness
+    differences
     (3D 24, 2D 13) and the mass term (consistent 3D 47 / 2D 35, lumped 4(d+1)+1),
     3 accumulations; per node the incidence sums E(d+1)/N plus 3 (residual and
     its dot) or 4 (CG direction and p.Ap)."""
@@ -306,13 +321,62 @@ def fp64_flops(stats, lumped, cg):
     return per_elem * E + per_node * N
 
 
-def kernel_roofline(P, m, stats, mode, fused, stream, workload, lumped=False):
-    """Roofline entry of the solve's dominant kernel: algorithmic bytes per
-    launch over its CUDA-event time (ps_profile_kernel, back-to-back launches
-    on `stream`), against the measured HBM copy bandwidth.  The FP64 passes
-    are bound by the FP64 pipe instead: FP64 mode reports its operator kernel
-    as "alu" (algorithmic FP64 flops against FP64_PEAK_TFLOPS, HBM fraction
-    beside it), and every line carries the FP64 residual pass the same way."""
+def on_chip_roofline(P, m, stats, mode, stream, alg_bytes):
+    """The on-chip kernel's time per iteration, from two solves that differ only
+    in their iteration count; None if this mesh's solves do not run on chip (a
+    run is one kernel there, every other engine launches at least one per
+    iteration: there the launches grow with the iterations).  Its vectors and most records stay on the SMs, so its bound is
+    the exchange between them; alg_bytes (what an iteration of separate kernels
+    moves) gives an effective rate only."""
+    import torch
+    n = stats.n_nodes
+    g = torch.Generator(device="cuda").manual_seed(5)
+    b = torch.randn(n, generator=g, device="cuda", dtype=torch.float64)
+    x = torch.zeros_like(b)
+    fp64 = mode == P.PS_MODE_FP64
+
+    def solve_ms(its):
+        o = P.make_opts(mode=mode, tol=1e-30, inner_tol=1e-30, max_iters=its, max_outer=1)
+        best = launches = None
+        for _ in range(8):
+            x.zero_()
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            e0.record(stream)
+            _, info = P.ps_pressure_solve(m, b, x, o, stream)
+            e1.record(stream)
+            torch.cuda.synchronize()
+            t = e0.elapsed_time(e1)
+            if info.iters_inner == its:
+                best, launches = t if best is None else min(best, t), info.kernel_launches
+        return best, launches
+
+    # (well-conditioned systems reach a residual of 0 before the longer pair)
+    for short, long in ((16, 56), (8, 24)):
+        (t0, l0), (t1, l1) = solve_ms(short), solve_ms(long)
+        if t0 is not None and t1 is not None:
+            break
+    else:
+        return None
+    if l0 != l1:
+        return None
+    it_ms = (t1 - t0) / (long - short)
+    return {"kernel": "k_solo_cg<%d,%s>" % (stats.dim, "double" if fp64 else "float"), "bound": "latency",
+            "iteration_us": 1e3 * it_ms, "effective_gbs": alg_bytes / (it_ms / 1e3) / 1e9,
+            "note": "vectors stay in shared memory; one exchange between the SMs per iteration; effective_gbs is "
+                    "over the bytes that separate kernels would move, no fraction of a peak"}
+
+
+def kernel_roofline(P, m, stats, mode, fused, stream, workload, lumped=False, auto=True):
+    """Roofline entry of the operator kernel of the solve's engine: algorithmic
+    bytes per launch over its CUDA-event time (ps_profile_kernel, back-to-back
+    launches on `stream`), against the measured HBM copy bandwidth.  The FP64
+    passes are bound by the FP64 pipe instead: FP64 mode reports its operator
+    kernel as "alu" (instructions of the star pass against FP64_PEAK_TOPS, HBM
+    fraction beside it), and every line carries the FP64 residual pass the same
+    way.  `auto`: the solves chose their engine; where that is the on-chip
+    kernel the entry is that kernel's, with the one of the separate kernels
+    that it replaces in "separate_kernels"."""
     if fused:
         which, kname = P.PS_KERNEL_CG1_F32, "k_cg1_chunks<%d>" % stats.dim
     elif mode == P.PS_MODE_MIXED and stats.operator_kernel == 2:
@@ -340,22 +404,27 @@ def kernel_roofline(P, m, stats, mode, fused, stream, workload, lumped=False):
     peak, peak_kind = peaks()
     achieved = alg_bytes / (kern_ms / 1e3) / 1e9
     res_ms = kern_other["resid_f64"]
-    res_flops = fp64_flops(stats, lumped, cg=False)
+    res_ops = fp64_star_ops(stats, cg=False)
     res_bytes = (4 * (d + 1) + 8) * E + (8 * (d + 1) + 3 * 8) * N
-    fp64_resid = {"kernel": "k_chunks<%d,double,kResid>" % d, "bound": "alu", "unit": "TFLOP/s",
-                  "achieved": res_flops / (res_ms / 1e3) / 1e12, "peak": FP64_PEAK_TFLOPS,
-                  "frac": res_flops / (res_ms / 1e3) / 1e12 / FP64_PEAK_TFLOPS,
-                  "hbm_frac": res_bytes / (res_ms / 1e3) / 1e9 / peak, "flops_per_launch": res_flops,
+    fp64_resid = {"kernel": "k_chunks<%d,double,kResid>" % d, "bound": "alu", "unit": "T FP64 op/s",
+                  "achieved": res_ops / (res_ms / 1e3) / 1e12, "peak": FP64_PEAK_TOPS,
+                  "frac": res_ops / (res_ms / 1e3) / 1e12 / FP64_PEAK_TOPS,
+                  "hbm_frac": res_bytes / (res_ms / 1e3) / 1e9 / peak, "ops_per_launch": res_ops,
+                  "effective_tflops": fp64_flops(stats, lumped, cg=False) / (res_ms / 1e3) / 1e12,
                   "kernel_ms": res_ms}
+    on_chip = on_chip_roofline(P, m, stats, mode, stream, alg_bytes) if auto else None
     if mode == P.PS_MODE_FP64:
-        flops = fp64_flops(stats, lumped, cg=True)
-        tf = flops / (kern_ms / 1e3) / 1e12
+        ops = fp64_star_ops(stats, cg=True)
+        top = ops / (kern_ms / 1e3) / 1e12
         tr = TRAFFIC.get((kname, workload))
-        return {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": tf / FP64_PEAK_TFLOPS, "traffic": tr["bytes"] if tr else None, "kernel": kname,
-                "kernel_ms": kern_ms, "flops_per_launch": flops, "hbm_frac": achieved / peak,
-                "alg_bytes_per_launch": alg_bytes, "peak_kind": "nominal FP64 (2 DFMA/clk/SM x 152 SMs x 2.07 GHz)",
+        out = {"bound": "alu", "achieved": top, "peak": FP64_PEAK_TOPS, "unit": "T FP64 op/s",
+                "frac": top / FP64_PEAK_TOPS, "traffic": tr["bytes"] if tr else None, "kernel": kname,
+                "kernel_ms": kern_ms, "ops_per_launch": ops, "hbm_frac": achieved / peak,
+                "effective_tflops": fp64_flops(stats, lumped, cg=True) / (kern_ms / 1e3) / 1e12,
+                "alg_bytes_per_launch": alg_bytes,
+                "peak_kind": "nominal FP64 (2 instructions/clk/SM x 152 SMs x 2.07 GHz)",
                 "other_kernels_ms": kern_other, "fp64_resid": fp64_resid, "chunks": stats.n_chunks}
+        return dict(on_chip, separate_kernels=out) if on_chip else out
     tr = TRAFFIC.get((kname, workload))
     upd_ms = kern_other["update_f32"]
     upd_bytes = 28 * N   # x, r, p, q, D^-1 read and x, r written, FP32
@@ -365,7 +434,7 @@ def kernel_roofline(P, m, stats, mode, fused, stream, workload, lumped=False):
     if stats.operator_kernel == 2:
         update["note"] = ("blocks store their rz, rr shares only; the halo gather (halo_f32) sums them in its "
                           "first block and ends the iteration")
-    return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+    out = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": tr["bytes"] if tr else None,
             "traffic_source": tr["source"] if tr else "not captured for the kernel as it stands",
             "kernel": kname, "update": update,
@@ -374,6 +443,7 @@ def kernel_roofline(P, m, stats, mode, fused, stream, workload, lumped=False):
             "shared_node_frac": stats.n_shared / stats.n_nodes,
             "note": "working set ~%.0f MB/launch: %s" % (
                 alg_bytes / 1e6, "L2-resident between iterations" if alg_bytes < 100e6 else "exceeds L2 (129 MB)")}
+    return dict(on_chip, separate_kernels=out) if on_chip else out
 
 
 def run_ours(args):
@@ -479,7 +549,7 @@ def run_ours(args):
 
     # ---- roofline of the dominant kernel
     fused = mode == P.PS_MODE_MIXED and (args.engine == "fused" or (args.engine == "auto" and case.n_nodes <= 200000))
-    roof = kernel_roofline(P, m, stats, mode, fused, stream, workload_name(args.n))
+    roof = kernel_roofline(P, m, stats, mode, fused, stream, workload_name(args.n), auto=args.engine == "auto")
 
     cpu = None
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
@@ -581,7 +651,7 @@ def run_single(args, which):
         P.ps_ctx_destroy(ctx)
         return
     stats = P.ps_mesh_get_stats(m)
-    roof = kernel_roofline(P, m, stats, mode, False, stream, case.name)
+    roof = kernel_roofline(P, m, stats, mode, False, stream, case.name, auto=args.engine == "auto")
     err = None
     if which == "c3":
         xs_h = case.extra["xstar"]
@@ -668,12 +738,11 @@ def bench_batch(args, P, S, autotune, torch):
                          for c, inf in zip(cases, infos))
     clk = clocks.stop() if not args.no_clocks else None
     tot = float(np.sum(times))
-    peak, peak_kind = peaks()
-    ach = alg_bytes / (tot / 1e3) / 1e9
-    roof = {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-            "peak_kind": peak_kind, "alg_bytes_per_batch": alg_bytes / args.steps,
-            "basis": "whole batch solve time (every kernel of the solve, FP64 passes and launch gaps "
-                     "included): a lower bound on the persistent inner kernel's own fraction"}
+    roof = {"bound": "latency", "effective_gbs": alg_bytes / (tot / 1e3) / 1e9,
+            "alg_bytes_per_batch": alg_bytes / args.steps,
+            "basis": "what the inner iterations would move as separate passes, over the whole batch solve time "
+                     "(FP64 passes and launch gaps included); meshes solved on chip keep their vectors there, so "
+                     "this is no fraction of a peak"}
     # the oracle's residual of every 32nd mesh's solution (assembled on the host)
     check = None
     if not args.no_cpu_baseline:
@@ -1159,12 +1228,13 @@ def run_headline(args):
     e2e_val = case.n_free * e2e_it / (np.sum(e2e_ms) / 1e3)
 
     # ---- roofline of the dominant kernels
-    roof = kernel_roofline(P, m, stats, P.PS_MODE_MIXED, False, stream, c3_name(case))
+    roof = kernel_roofline(P, m, stats, P.PS_MODE_MIXED, False, stream, c3_name(case), auto=args.engine == "auto")
     ipi = (last.iters_inner + last.iters_outer)
+    kernels = roof.get("separate_kernels", roof)
     roof["in_solve_check"] = {
         "solve_ms_per_iteration": total_ms / args.steps / max(ipi, 1),
-        "isolated_iteration_kernels_ms": roof["kernel_ms"] + roof["update"]["kernel_ms"] +
-                                          (roof["other_kernels_ms"]["halo_f32"] if stats.operator_kernel == 2 else 0.0),
+        "isolated_iteration_kernels_ms": kernels["kernel_ms"] + kernels["update"]["kernel_ms"] +
+                                          (kernels["other_kernels_ms"]["halo_f32"] if stats.operator_kernel == 2 else 0.0),
         "note": "kernel_ms is the mean of back-to-back launches of the kernel alone; the solve's time per "
                 "iteration also holds the outer FP64 passes and graph launch gaps"}
     P.ps_mesh_free(m)
