@@ -102,29 +102,28 @@ void build_patches(int dim, int n, const std::vector<std::array<int, 4>> &lc, st
     out.clear();
     std::vector<char> used(n, 0);
     std::vector<std::pair<uint64_t, int>> inc;   // (pivot key, element)
+    // sorted by counting on the pivot's (smaller) vertex, in 3D then by key
+    // within each
     int nloc = 0;
-    if (dim == 3) {
-        inc.reserve((size_t)n * 6);
+    for (int e = 0; e < n; ++e)
+        for (int i = 0; i < nv; ++i) nloc = std::max(nloc, lc[e][i] + 1);
+    auto each_pivot = [&](auto &&fn) {   // element, vertex, key
         for (int e = 0; e < n; ++e)
-            for (int i = 0; i < 4; ++i)
-                for (int j = i + 1; j < 4; ++j) {
-                    uint64_t u = (uint64_t)std::min(lc[e][i], lc[e][j]);
-                    uint64_t v = (uint64_t)std::max(lc[e][i], lc[e][j]);
-                    inc.push_back({(u << 20) | v, e});
+            for (int i = 0; i < nv; ++i) {
+                if (dim == 2) fn(e, lc[e][i], (uint64_t)lc[e][i]);
+                for (int j = i + 1; dim == 3 && j < nv; ++j) {
+                    const int u = std::min(lc[e][i], lc[e][j]), v = std::max(lc[e][i], lc[e][j]);
+                    fn(e, u, ((uint64_t)u << 20) | (uint64_t)v);
                 }
-        std::sort(inc.begin(), inc.end());
-    } else {
-        // (the keys are local vertices: sorted by counting)
-        for (int e = 0; e < n; ++e)
-            for (int i = 0; i < 3; ++i) nloc = std::max(nloc, lc[e][i] + 1);
-        std::vector<int> at(nloc + 1, 0);
-        for (int e = 0; e < n; ++e)
-            for (int i = 0; i < 3; ++i) at[lc[e][i] + 1]++;
-        for (int v = 0; v < nloc; ++v) at[v + 1] += at[v];
-        inc.resize((size_t)n * 3);
-        for (int e = 0; e < n; ++e)
-            for (int i = 0; i < 3; ++i) inc[at[lc[e][i]]++] = {(uint64_t)lc[e][i], e};
-    }
+            }
+    };
+    std::vector<int> at(nloc + 1, 0);
+    each_pivot([&](int, int u, uint64_t) { at[u + 1]++; });
+    for (int v = 0; v < nloc; ++v) at[v + 1] += at[v];
+    inc.resize(at[nloc]);
+    each_pivot([&](int e, int u, uint64_t key) { inc[at[u]++] = {key, e}; });
+    if (dim == 3)
+        for (int v = 0; v < nloc; ++v) std::sort(inc.begin() + (v ? at[v - 1] : 0), inc.begin() + at[v]);
     std::vector<size_t> gstart;
     for (size_t k = 0; k < inc.size(); ++k)
         if (k == 0 || inc[k].first != inc[k - 1].first) gstart.push_back(k);
