@@ -356,7 +356,9 @@ __device__ __forceinline__ typename Share<T>::Wide block_shares(const typename S
     const int q = lane >> 3, k = lane & 7;
     typename Sh::Wide v = Sh::wide(q < 3 ? red[q][k] : Sh::zero());
     if (nw > 8) v = Sh::add(v, Sh::wide(q < 3 ? red[q][k + 8] : Sh::zero()));
-    return sum_lanes<T, 8>(v);
+    v = Sh::add(v, Sh::shfl(v, 4));
+    v = Sh::add(v, Sh::shfl(v, 1));
+    return Sh::add(v, Sh::shfl(v, 2));
 }
 
 // The loop of the kernel below is kept small on purpose (no unrolling, one copy
@@ -365,7 +367,7 @@ __device__ __forceinline__ typename Share<T>::Wide block_shares(const typename S
 // (301 x 301 squares: 15k cycles per iteration).
 // Measured per iteration, with the kernels it replaces: 301 x 301 squares 4.3 us
 // (fused pass 16), 64^3 Kuhn 9.8 (operator, update and halo kernels 25), FP64
-// 64 x 64 squares 7.7 (25), FP64 40^3 17 (68).  Bound (cycles of an iteration's
+// 64 x 64 squares 8.3 (25), FP64 40^3 18 (68).  Bound (cycles of an iteration's
 // phases): 301 x 301 squares 3.7k the update, stars and node sums, 2 to 3k the
 // scalars (dependent FP64 operations), the rest the exchange (a word from one
 // SM's store to another's poll takes 1.7 us on this part); 64^3: 4.6k the stars
@@ -379,6 +381,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
     constexpr bool F32 = sizeof(T) == 4;
     constexpr int RES = F32 ? kSoloResident : 1;
     constexpr int kW = Tagged<T>::kWords;
+    constexpr bool kLanes = F32 && !BATCH;   // one warp reads a product's shares, else 32 at a time
     // (done: set when the run ends, by this thread, and not after a wait's limit)
     if (bid == 0 && threadIdx.x == 0) A.st->done = 0;
     T *val = reinterpret_cast<T *>(smem + A.L.val), *sr = reinterpret_cast<T *>(smem + A.L.r),
@@ -391,7 +394,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
     using Sh = Share<T>;
     using ST = typename Sh::type;
     __shared__ ST s_red[3][16];   // warps' sums; entries past the last warp stay 0
-    __shared__ typename Sh::Wide s_sum[3][BATCH ? kSoloMaxBlocks / 32 : 1];   // parts of the products' sums
+    __shared__ typename Sh::Wide s_sum[3][kLanes ? 1 : kSoloMaxBlocks / 32];   // parts of the products' sums
     __shared__ T s_alpha, s_beta;
     __shared__ int s_end;
     const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = NT >> 5;
@@ -540,7 +543,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
             __syncwarp();
         }
         if (G > 1) {
-            if (F32 && !BATCH && it > 0) __nanosleep(A.nap);
+            if (kLanes && it > 0) __nanosleep(A.nap);
             // the shared unknowns' partials, which travel beside the shares
 #pragma unroll 1
             for (int j = tid; j < n_sh; j += NT) {
@@ -578,9 +581,10 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                 const T mr = sm[l];
                 sw[l] = is_dirichlet(mr) ? T(0) : fma_rn(mr, val[l], w);
             }
-            if constexpr (BATCH) {
+            if constexpr (!kLanes) {
                 // the blocks' shares, 32 of a product to a warp at a time (one
-                // warp per product, as below, took the batch 3% longer)
+                // warp per product, as below, took the batch 3% longer; FP64 runs
+                // 8% shorter on 64 x 64 squares, but with other roundings)
                 const uint4 *mine = A.exch + ((size_t)(it & 1) * 3 * G + 3 * bid) * G;
 #pragma unroll 1
                 for (int sg = wid; sg < 3 * n_seg; sg += nw) {
@@ -590,9 +594,9 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
                         const uint4 *w = mine + q * G + b;
                         uint4 x = ld_pair(w);
                         while ((x.y != tag || x.w != tag) &&
-                               (it == 0 ? spin.again_queued(reinterpret_cast<const uint2 *>(w) + (x.y == tag), tag, A.beat,
-                                                            A.err)
-                                        : spin.again(A.spin_limit)))
+                               (BATCH && it == 0 ? spin.again_queued(reinterpret_cast<const uint2 *>(w) + (x.y == tag),
+                                                                     tag, A.beat, A.err)
+                                                 : spin.again(A.spin_limit)))
                             x = ld_pair(w);
                         v = Sh::from(x.x, x.z);
                     }
@@ -634,7 +638,7 @@ __device__ __forceinline__ int solo_run_block(const SoloArgs<T> &A, const int bi
         if (wid == 0) {
             // lane 8 q + k: part k of product q
             typename Sh::Wide w = Sh::wide(Sh::zero());
-            if constexpr (BATCH) {   // lane 8 q + k: part k of product q
+            if constexpr (!kLanes) {   // lane 8 q + k: part k of product q
                 const int q = lane >> 3, k = lane & 7;
                 if (q < 3 && k < n_seg) w = s_sum[q][k];
                 w = sum_lanes<T, 8>(w);
