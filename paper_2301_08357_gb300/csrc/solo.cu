@@ -12,7 +12,7 @@
 // through L2.  The recurrences are the one-reduction form of cg1.cuh
 // (Chronopoulos and Gear), so there is one exchange per iteration: a block
 // stores its shares into every block's own list, each block waits for its
-// list, sums it in block order and advances the scalars (the same words in
+// list, sums it in a fixed order and advances the scalars (the same words in
 // the same order, so all take the same decision); the others' partial sums
 // travel, and are read, at the same time.  Every word exchanged carries the iteration's tag
 // beside 32 bits of its value, so a reader knows a word by itself: no fence,
